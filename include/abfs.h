@@ -72,7 +72,15 @@ typedef enum {
 #define ABFS_MODE_PLAIN 1u      /* comparator: masked SpMSpV, multiply every entry, mask after */
 
 /* Tunable launch parameters.  abfs_default_params() fills sound values;
- * abfs_tune() measures and picks them for a graph. */
+ * abfs_tune() measures and picks them for a graph.
+ *
+ * Two engines run single searches, with the same results.  With the default
+ * values of the scheduling knobs (tile, unit_entries, narrow_*, ctas_per_sm,
+ * claim_scan, cluster_*), submatrix searches without a physical shrink run on
+ * the level-synchronous engine, which takes one search at a time and none of
+ * those knobs.  A search that sets any of them, the comparator, shrinks,
+ * abfs_run_static and serving run on the unit scheduler, whose knobs they
+ * are. */
 typedef struct {
     uint32_t mode;            /* ABFS_MODE_SUBMATRIX or ABFS_MODE_PLAIN */
     uint32_t tile;            /* frontier vertices staged per step, 32..1024, multiple of 32 */
@@ -285,8 +293,9 @@ int abfs_run_host_many(abfs_graph_t g, const uint32_t* sources, uint32_t count,
  *   7 frontier bitmap of a bottom-up level, 8 bottom-up level,
  *   0xFE start, 0xFF end), [3] 0 if the phase was published to the whole
  *   grid, 1 if it ran on one CTA (or started a cluster run), 2 if it is a
- *   further level of a resident narrow run, 3 if it is a further level of a
- *   cluster run ([4] then holds the run's CTAs), [4] units or touched rows of
+ *   further level of a resident narrow run, 4 if it is a thin level of the
+ *   level-synchronous engine ([5] then counts list items), 3 if it is a further
+ *   level of a cluster run ([4] then holds the run's CTAs), [4] units or touched rows of
  *   the phase, [5] frontier
  *   vertices, [6] entry slots of that frontier (column entries plus up to 6
  *   per vertex, low 32 bits), [7] 0.  For a level, [4] is its number of work

@@ -192,16 +192,36 @@ EngineParams engine_params(const abfs_params& p) {
     return e;
 }
 
+// Whether a workspace for these parameters is laid out for the level-synchronous
+// engine too (a property that same_layout keeps).
+bool sync_layout(const abfs_params& p) {
+    return p.mode == ABFS_MODE_SUBMATRIX && !shrink_enabled(p) &&
+           p.unit_entries == default_params().unit_entries;
+}
+
 bool same_layout(const abfs_params& a, const abfs_params& b) {
     return a.mode == b.mode && a.unit_entries == b.unit_entries && shrink_enabled(a) == shrink_enabled(b) &&
            (!shrink_enabled(a) || std::min(a.shrink_max, 2u) == std::min(b.shrink_max, 2u));
+}
+
+// The knobs of the unit scheduler (units, narrow and cluster runs, the grid and
+// the reduction threshold) mean nothing to the level-synchronous engine: a
+// search that sets any of them asks for the scheduler.
+bool sync_applies(uint32_t n, uint64_t nnz, const abfs_params& p) {
+    const abfs_params d = default_params();
+    return p.mode == ABFS_MODE_SUBMATRIX && !shrink_enabled(p) && p.tile == d.tile &&
+           p.unit_entries == d.unit_entries && p.narrow_max == d.narrow_max &&
+           p.narrow_edges == d.narrow_edges && p.ctas_per_sm == d.ctas_per_sm &&
+           p.narrow_resident == d.narrow_resident && p.claim_scan == d.claim_scan &&
+           p.cluster_ctas == d.cluster_ctas && p.cluster_min == d.cluster_min &&
+           p.cluster_max == d.cluster_max && p.cluster_edges == d.cluster_edges;
 }
 
 // ---------------------------------------------------------------------------
 // per-search workspace layout
 // ---------------------------------------------------------------------------
 
-Layout layout_for(uint32_t n, uint64_t nnz, const abfs_params& p, uint32_t ms, bool relabel) {
+Layout layout_for(uint32_t n, uint64_t nnz, const abfs_params& p, uint32_t ms, bool relabel, bool sync) {
     Layout L;
     std::memset(&L, 0, sizeof(L));
     const size_t A = 256;
@@ -226,6 +246,21 @@ Layout layout_for(uint32_t n, uint64_t nnz, const abfs_params& p, uint32_t ms, b
         L.flen[i] = take((size_t)n * 4);
         L.blk[i] = take((size_t)L.bcap * sizeof(Block));
         L.ustart[i] = take((size_t)L.ucap * sizeof(uint2));
+    }
+    if (sync) {
+        // a list holds each vertex's column once, in ceil((h + len) / kSyncSeg)
+        // items, h <= kChunk - 1
+        L.icap = (uint32_t)(n + (nnz + (uint64_t)kChunk * n) / kSyncSeg + 64);
+        size_t x = L.fq[0];
+        auto over = [&](size_t bytes) {
+            size_t at = x;
+            x = align_up(x + bytes, A);
+            return at;
+        };
+        L.skey = over((size_t)n * 8);
+        for (int i = 0; i < 2; ++i)
+            for (int c = 0; c < 3; ++c) L.slist[i][c] = over((size_t)L.icap * 4);
+        o = std::max(o, x);
     }
     if (p.mode == ABFS_MODE_SUBMATRIX)
         for (int i = 0; i < 2; ++i) L.bm[i] = take((size_t)L.nwords * 4);
@@ -331,10 +366,11 @@ struct Workspace {
     bool relabel = false;     // laid out for searches on the relabelled copy too
     Inst* d_inst = nullptr;   // device descriptor (instance 0)
     Inst* d_inst_r = nullptr; // the same on the relabelled copy
-    uint32_t* d_done = nullptr;
+    uint32_t* d_done = nullptr;  // and, from byte kBarAt on, the SyncBar
     unsigned long long* d_beat = nullptr;
     InstCtl* h_ctl = nullptr; // pinned copy for stats
 };
+constexpr size_t kBarAt = 256;
 
 struct abfs_graph_s {
     uint32_t* d_colptr = nullptr;
@@ -428,10 +464,10 @@ int ensure_workspace(abfs_graph_s* g, const abfs_params& p) {
         if (g->used) CK(cudaEventSynchronize(g->last_use));
         free_workspace(w);
     }
-    Layout L = layout_for(g->n, g->nnz, p, 0, g->relabeled);
+    Layout L = layout_for(g->n, g->nnz, p, 0, g->relabeled, sync_layout(p));
     int rc = dev_alloc((void**)&w.base, L.total);
     if (rc) return rc;
-    rc = dev_alloc((void**)&w.d_done, 64);
+    rc = dev_alloc((void**)&w.d_done, kBarAt + sizeof(SyncBar));
     if (!rc) rc = dev_alloc((void**)&w.d_beat, 64);
     if (rc) {
         free_workspace(w);
@@ -460,6 +496,8 @@ int ensure_workspace(abfs_graph_s* g, const abfs_params& p) {
     // the initialisation kernel of single searches counts its blocks in the
     // control block, which must start at zero
     if (e == cudaSuccess) e = cudaMemset(w.base + L.ctl, 0, sizeof(InstCtl));
+    // so must the barrier words of the level-synchronous engine
+    if (e == cudaSuccess) e = cudaMemset(reinterpret_cast<char*>(w.d_done) + kBarAt, 0, sizeof(SyncBar));
     if (e != cudaSuccess) {
         free_workspace(w);
         return cuda_fail(e);
@@ -491,6 +529,58 @@ const abfs_params& pick_params(const abfs_graph_s* g, const abfs_params* params,
     return tmp;
 }
 
+// The search as the level-synchronous engine takes it: the workspace's buffers
+// and the input CSC, or with `rel` the relabelled copy.
+SyncSearch make_sync(const abfs_graph_s* g, const Workspace& w, uint32_t source, bool rel,
+                     const abfs_params& p) {
+    SyncSearch S;
+    std::memset(&S, 0, sizeof(S));
+    const Layout& L = w.L;
+    S.colptr = rel ? g->r_colptr : g->d_colptr;
+    S.rowidx = rel ? g->r_rowidx : g->d_rowidx;
+    S.nnz = g->nnz;
+    S.n = g->n;
+    S.nwords = L.nwords;
+    S.src = rel ? g->h_pos[source] : source;
+    S.src_label = source;
+    S.inb = rel ? g->r_inb : g->d_inb;
+    if (rel) {
+        S.lab = g->d_lab;
+        S.pos = g->d_pos;
+        S.n_keep = g->r_keep;
+    }
+    S.icap = L.icap;
+    S.key = reinterpret_cast<unsigned long long*>(w.base + L.skey);
+    S.bm = reinterpret_cast<uint32_t*>(w.base + L.bm[0]);
+    for (int i = 0; i < 2; ++i) {
+        S.fbm[i] = reinterpret_cast<uint32_t*>(w.base + L.fbm[i]);
+        S.lj[i] = reinterpret_cast<uint32_t*>(w.base + L.slist[i][0]);
+        S.lb[i] = reinterpret_cast<uint32_t*>(w.base + L.slist[i][1]);
+        S.ll[i] = reinterpret_cast<uint32_t*>(w.base + L.slist[i][2]);
+    }
+    S.ctl = reinterpret_cast<InstCtl*>(w.base + L.ctl);
+    S.bar = reinterpret_cast<SyncBar*>(reinterpret_cast<char*>(w.d_done) + kBarAt);
+    // A wide level costs a bitmap (8 bytes per vertex), an extraction and a
+    // barrier more than a thin one and saves a returned 64-bit atomic per entry.
+    // Those atomics queue where many columns share hub rows, which a frontier
+    // of columns well above the mean is a sign of (undirected graphs): R-MAT of scale 16, 1.2 M
+    // entries, 150 us with its hub levels thin, 75 us wide.  Without hubs thin
+    // levels stay ahead longer: ER of 2^18 vertices of degree 8, 85 us thin, 100 us
+    // with the lower line.
+    S.wide_min = (3ull << 19) + g->n;
+    S.wide_hub = (1ull << 18) + g->n / 4;
+    S.hub_avg = (uint32_t)std::max<uint64_t>(8, 3 * g->nnz / (2ull * g->n));
+    S.timeout_ns = (unsigned long long)p.timeout_ms * 1000000ull;
+    S.hold_units = test_hold_units();
+    return S;
+}
+
+// CTAs of a search's team: enough that each has a few thousand entries.
+int sync_ctas(const abfs_graph_s* g, int most) {
+    const uint64_t want = g->nnz <= 16384 ? 1 : (g->nnz + 4095) / 4096;
+    return (int)std::min<uint64_t>((uint64_t)most, std::max<uint64_t>(want, 1));
+}
+
 // Enqueues one search into g's workspace; caller holds g->mu.
 int enqueue_single(abfs_graph_s* g, uint32_t source, int32_t* level, int32_t* parent,
                    cudaStream_t s, const abfs_params& p, uint4* trace = nullptr,
@@ -506,6 +596,21 @@ int enqueue_single(abfs_graph_s* g, uint32_t source, int32_t* level, int32_t* pa
     const bool bu_wanted = p.bottom_up_alpha && !g->directed && g->sorted;
     const bool rel = w.relabel && p.mode == ABFS_MODE_SUBMATRIX && !sigma && !bu_wanted;
     const uint32_t bu_ok = (!rel && !g->directed && g->sorted && !sigma) ? 1u : 0u;
+    const int most = sync_applies(g->n, g->nnz, p) ? sync_max_ctas(g->device, g->sms) : 0;
+    if (most > 0) {
+        SyncSearch S = make_sync(g, w, source, rel, p);
+        S.sigma = reinterpret_cast<unsigned long long*>(sigma);
+        S.level = level;
+        S.parent = reinterpret_cast<uint32_t*>(parent);
+        S.trace = trace;
+        S.trace_cap = trace_cap;
+        S.bu_alpha = bu_ok ? p.bottom_up_alpha : 0u;
+        S.bu_beta = p.bottom_up_beta;
+        CK(launch_sync(S, sync_ctas(g, most), s));
+        CK(cudaEventRecord(g->last_use, s));
+        g->used = true;
+        return ABFS_OK;
+    }
     EngineArgs a;
     a.insts = rel ? w.d_inst_r : w.d_inst;
     a.ninst = 1;
@@ -806,7 +911,7 @@ extern "C" int abfs_graph_footprint(abfs_graph_t g, const abfs_params* params, s
     const abfs_params& p = pick_params(g, params, tmp);
     int rc = check_params(p);
     if (rc) return rc;
-    *bytes = layout_for(g->n, g->nnz, p, 0, g->relabeled).total;
+    *bytes = layout_for(g->n, g->nnz, p, 0, g->relabeled, sync_layout(p)).total;
     return ABFS_OK;
 }
 
@@ -1363,8 +1468,14 @@ extern "C" int abfs_tune(abfs_graph_t g, const uint32_t* sources, uint32_t count
             }
         }
     }
-    // candidate sets
+    // candidate sets: the defaults (level-synchronous engine in submatrix mode)
+    // and the unit scheduler's
     std::vector<abfs_params> cands;
+    {
+        abfs_params p = default_params();
+        p.mode = mode;
+        cands.push_back(p);
+    }
     const uint32_t units[] = {512, 1024, 4096};
     const uint32_t narrow_e[] = {0, 16384, 65536};
     const uint32_t ctas[] = {1, 2};

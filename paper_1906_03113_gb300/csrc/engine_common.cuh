@@ -274,7 +274,6 @@ __device__ __forceinline__ void prof_add(Smem& sm, int slot, long long t0) {
     if (sm.prof_on && threadIdx.x == 0) sm.prof[slot] += (unsigned long long)(clock64() - t0);
 }
 
-size_t engine_smem_bytes() { return sizeof(Smem); }
 
 // ---------------------------------------------------------------------------
 // block-level building blocks

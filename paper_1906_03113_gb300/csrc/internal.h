@@ -57,6 +57,8 @@ static_assert((kUnitMax & (kUnitMax - 1)) == 0 && kUnitMax >= 1024, "unit size")
 // lane): slots come in chunks of four, and the start bitmap has a bit per chunk.
 constexpr uint32_t kChunk = 4;
 constexpr int kStartWords = kUnitMax / kChunk / 32 + 2;
+// Column entries per item of the level-synchronous engine's lists.
+constexpr uint32_t kSyncSeg = 256;
 // Marker of an unset parent / unclaimed vertex (reads as -1 through int32).
 constexpr uint32_t kUnset = 0xFFFFFFFFu;
 // Weight of a frontier vertex in its level's work space: the chunks that hold
@@ -235,6 +237,47 @@ struct EngineArgs {
     uint32_t hold_units = 0;
 };
 
+// Level-synchronous engine (sync_engine.cu): the words its barriers and lists
+// count in.  Zero between searches (the last CTA of a search clears them).
+struct SyncBar {
+    unsigned long long word[2];  // arrivals and totals, by barrier number modulo 2
+    unsigned long long aux[2];   // vertices and entries beside them
+    uint32_t lcnt[2];            // items appended to the global list, by level parity
+    uint32_t exited;             // CTAs that have left (wraps to 0)
+};
+
+// One search of the level-synchronous engine (a kernel argument).
+struct SyncSearch {
+    const uint32_t* colptr;
+    const uint32_t* rowidx;      // 16-byte aligned
+    unsigned long long nnz;
+    uint32_t n, nwords;
+    uint32_t src, src_label;     // the source and the label its products carry
+    const uint32_t* inb;         // rows that occur in some column (nullptr: not known)
+    const uint32_t* lab;         // relabelled graph: internal -> input label (nullptr: none)
+    const uint32_t* pos;         // relabelled graph: input -> internal label
+    uint32_t n_keep;             // relabelled graph: vertices from n_keep on are unreachable
+    uint32_t icap;               // items each global list holds
+    unsigned long long* key;     // level << 32 | parent per vertex (16-byte aligned)
+    uint32_t* bm;                // visited bitmap of wide and bottom-up levels
+    uint32_t* fbm[2];            // hybrid: frontier bitmaps, by level parity
+    uint32_t *lj[2], *lb[2], *ll[2];  // frontier lists: column label, first row index, entries
+    unsigned long long* sigma;   // shortest-path counts (nullptr: off)
+    int32_t* level;              // outputs
+    uint32_t* parent;
+    InstCtl* ctl;
+    SyncBar* bar;
+    uint4* trace;
+    uint32_t trace_cap;
+    uint32_t bu_alpha, bu_beta;  // hybrid thresholds (0: off or not allowed)
+    uint32_t hold_units;         // test control: arrivals that never come
+    // a level of this many entries is wide; the same for frontiers whose items
+    // average hub_avg entries or more
+    unsigned long long wide_min, wide_hub;
+    uint32_t hub_avg;
+    unsigned long long timeout_ns;
+};
+
 // Cycle accounting of the engine's CTAs (profiling runs only).
 enum ProfSlot : int {
     kProfIdle = 0,     // no unit available
@@ -268,6 +311,10 @@ struct Layout {
         srows[2], ctl, inst, inst_r;
     size_t ms_vis, ms_fr[2], ms_nx, ms_src, ms_lev, ms_par;  // multi-source searches only
     size_t lev_i, par_i;  // searches on a relabelled graph: internal outputs
+    // level-synchronous engine: key words and lists, laid over the buffers from
+    // fq[0] on (a search uses one engine or the other); 0 when not laid out
+    size_t skey, slist[2][3], sbar;
+    uint32_t icap;
     size_t total;
     uint32_t nwords, bcap, ncopies;
     unsigned long long ucap, scap;
@@ -279,7 +326,10 @@ bool shrink_enabled(const abfs_params& p);
 int check_params(const abfs_params& p);
 EngineParams engine_params(const abfs_params& p);
 Layout layout_for(uint32_t n, uint64_t nnz, const abfs_params& p, uint32_t ms = 0,
-                  bool relabel = false);
+                  bool relabel = false, bool sync = false);
+// Whether a search of this size with these parameters runs on the
+// level-synchronous engine.
+bool sync_applies(uint32_t n, uint64_t nnz, const abfs_params& p);
 Inst make_inst_raw(const uint32_t* colptr, const uint32_t* rowidx, uint32_t n, char* base,
                    const Layout& L, uint32_t src, int32_t* level, int32_t* parent);
 int grid_for(int sms, const abfs_params& p);
@@ -314,6 +364,8 @@ cudaError_t launch_engine(const EngineArgs& a, int grid, cudaStream_t s);
 cudaError_t engine_occupancy(uint32_t mode, int* blocks_per_sm);
 // Clusters of `cluster` CTAs of the engine that can be resident at once.
 cudaError_t engine_max_clusters(uint32_t mode, uint32_t cluster, int* clusters);
-size_t engine_smem_bytes();
+// Level-synchronous engine (sync_engine.cu).
+int sync_max_ctas(int device, int sms);
+cudaError_t launch_sync(const SyncSearch& S, int ctas, cudaStream_t s);
 
 }  // namespace abfs

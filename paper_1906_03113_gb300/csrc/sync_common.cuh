@@ -1,0 +1,233 @@
+// Level-synchronous engine: shared state, the team barrier and the frontier
+// lists.  Part of sync_engine.cu, split by topic; included in order.
+//
+// One search runs on a team of P CTAs that are resident together (a
+// cooperative launch).  Every vertex has one 64-bit word
+//     key[v] = level << 32 | parent   (all ones: not reached)
+// and a level is a bulk-synchronous step between two team barriers.  Because
+// the level is the high half, one atomicMin on the word masks and claims at
+// once: a row reached earlier has a smaller level and keeps its word, a row of
+// the next level keeps the least column index, and the returned value tells
+// whether the row was new (Theorem 1's product in the (min, index) semiring
+// with the mask V_{k+1} folded into the order of the keys).
+#pragma once
+
+#include "engine_common.cuh"
+
+namespace abfs {
+
+constexpr int kSyncThreads = 1024;
+constexpr int kSyncWarps = kSyncThreads / 32;
+// Columns are listed in items of at most kSeg entries (split where the row
+// index is a multiple of kChunk), so that any number of warps can share a hub.
+constexpr uint32_t kSeg = kSyncSeg;
+// Items a CTA keeps of a thin level's frontier.  Two lists of 12-byte items
+// stay under the 32 KB shared-memory split, which leaves 224 KB of L1 for the
+// bitmap words of wide levels.
+constexpr uint32_t kThinCap = 1024;
+constexpr unsigned long long kKeyUnset = ~0ull;
+// A barrier word holds the arrivals and the totals of the next level; it only
+// ever grows, and what a barrier added is its difference to the barrier two
+// steps back (barriers alternate between two words, so nobody can add to a
+// word that a slower CTA still waits on, and no word is cleared in flight).
+//   thin level:  [arrived : 8][full lists : 8][heavy lists : 8][items : 21][entries / 64 : 19]
+//   otherwise:   [arrived : 8][items : 56]
+// (a CTA's share of a thin word is clamped so that 240 of them fit their field;
+// exact totals follow with the next barrier where they matter).  Beside it,
+// for the hybrid and traces: [vertices : 31][column entries : 33].
+constexpr uint32_t kArriveShift = 56, kFullShift = 48, kHeavyShift = 40, kItemShift = 19;
+constexpr uint32_t kEntUnit = 64, kEntClamp = 2184, kItemClamp = 8191;
+constexpr uint32_t kAuxShift = 33;
+
+// What a level is followed by; the team's CTAs agree on it because they decide
+// from the same totals.
+enum SyncAct : uint32_t {
+    kActThin = 0,    // the next level is thin, the lists stay where they are
+    kActEven = 1,    // thin, after the lists were evened out through the global list
+    kActWide = 2,    // the next level is wide
+    kActSlice = 3,   // thin, from the global list a wide level left
+    kActBottomUp = 4,
+    kActDone = 5,
+    kActFailed = 6,  // the bounded wait ran out, or an append failed
+};
+
+struct SyncSmem {
+    // items of the current and the next thin level: column label, first row
+    // index, entries
+    uint32_t ij[2][kThinCap], ib[2][kThinCap], il[2][kThinCap];
+    // [0] items appended to each list (may exceed kThinCap: the rest is
+    // spilled), [1] column entries of their vertices
+    uint32_t app[2][2];
+    uint32_t verts, ent;              // wide levels: vertices this CTA reached, their entries
+    uint32_t tick;                    // wide levels: runs this CTA's warps have taken
+    uint32_t base;
+    uint32_t wsum[kSyncWarps], wpre[kSyncWarps];
+    uint32_t act;                     // SyncAct after the last barrier
+    unsigned long long items;         // the next level's items
+    // thread 0's state of the search
+    uint32_t lim_items, lim_ent;      // a list above either is heavy
+    uint32_t bu;
+    unsigned long long nf, entries, seen;
+    unsigned long long st_read, st_unmasked, st_verts, st_ent;
+    uint32_t levels;
+    uint32_t step;                            // barriers passed
+    unsigned long long word[2], aux[2];       // the barrier words as last seen
+};
+
+// A CTA's place in its team.
+struct Team {
+    uint32_t rank, size;
+    uint32_t expect;  // arrivals a barrier waits for (more than size only in the held test)
+};
+
+// Counters of a thread over a whole search.
+struct SyncTally {
+    uint32_t read = 0, unmasked = 0, verts = 0, levels = 0;
+};
+
+// Adds a warp's counters to the CTA's.  Whole warp.
+__device__ __forceinline__ void tally_add(SyncSmem& sm, uint32_t read, uint32_t unmasked) {
+    read = __reduce_add_sync(0xFFFFFFFFu, read);
+    unmasked = __reduce_add_sync(0xFFFFFFFFu, unmasked);
+    if ((threadIdx.x & 31) == 0) {
+        if (read) atomicAdd(&sm.st_read, (unsigned long long)read);
+        if (unmasked) atomicAdd(&sm.st_unmasked, (unsigned long long)unmasked);
+    }
+}
+
+__device__ __forceinline__ void red_add64(unsigned long long* p, unsigned long long v) {
+    asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+// The least value wins; nothing comes back.  (atomicMin with its result unused
+// is compiled to an atomic that returns.)
+__device__ __forceinline__ void red_min32(uint32_t* p, uint32_t v) {
+    asm volatile("red.relaxed.gpu.global.min.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ void red_add_release64(unsigned long long* p, unsigned long long v) {
+    asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+// Thread 0 of each CTA: adds `add` and the arrival to the barrier's word, waits
+// until the team has arrived and returns the totals, or ~0 when the bounded
+// wait ran out.  The wait itself delivers the totals: no further read follows
+// unless `aux` is wanted.
+//
+// FULL: what the CTAs wrote before the barrier can be read after it.  Without
+// it the barrier orders only the claims of a thin level: each was an atomic on
+// a key word whose returned value its CTA has used before it arrived, so it
+// has been performed at the L2, and everything the next level does with a key
+// word is another atomic or a strong load there.  The release and the acquire
+// cost 1.1 + 0.8 thousand cycles of a thin level's 8.4.
+template <bool FULL>
+__device__ __forceinline__ unsigned long long bar_wait(SyncSmem& sm, const SyncSearch& S, const Team& T,
+                                                       unsigned long long add, unsigned long long& aux) {
+    if (T.expect == 1) return add;
+    const uint32_t b = sm.step & 1u;
+    ++sm.step;
+    unsigned long long* w = &S.bar->word[b];
+    const unsigned long long before = sm.word[b];
+    if (FULL) {
+        if (aux) red_add64(&S.bar->aux[b], aux);
+        red_add_release64(w, add + (1ull << kArriveShift));
+    } else {
+        red_add64(w, add + (1ull << kArriveShift));
+    }
+    unsigned long long v;
+    uint64_t t0 = 0;
+    for (uint32_t spin = 0;; ++spin) {
+        v = ld_relaxed64(w);
+        if ((uint32_t)((v - before) >> kArriveShift) == T.expect) break;
+        // reading %globaltimer is slow: the clock starts after 4096 polls
+        if ((spin & 4095u) == 4095u) {
+            const uint64_t now = globaltimer();
+            if (t0 == 0) {
+                t0 = now;
+            } else if (now - t0 > S.timeout_ns) {
+                fail(S.ctl, 5 /* ABFS_ERR_TIMEOUT */);
+                return ~0ull;
+            }
+        }
+    }
+    sm.word[b] = v;
+    if (FULL) {
+        __threadfence();  // acquire: what the others wrote before they arrived
+        const unsigned long long x = ld_relaxed64(&S.bar->aux[b]);
+        aux = x - sm.aux[b];
+        sm.aux[b] = x;
+    }
+    return (v - before) & ((1ull << kArriveShift) - 1);
+}
+
+// A plain full barrier; the sums of `add` and `ent` (thread 0's) reach sm.items
+// and sm.entries.
+// Returns false when the bounded wait ran out.  Whole CTA.
+__device__ __forceinline__ bool team_sync(SyncSmem& sm, const SyncSearch& S, const Team& T,
+                                          unsigned long long add = 0, unsigned long long ent = 0) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        sm.items = bar_wait<true>(sm, S, T, add, ent);
+        sm.entries = ent;
+    }
+    __syncthreads();
+    return sm.items != ~0ull;
+}
+
+// Items of the column [beg, beg + len).
+__device__ __forceinline__ uint32_t items_of(uint32_t beg, uint32_t len) {
+    return len ? ((beg & (kChunk - 1)) + len + kSeg - 1) / kSeg : 0u;
+}
+// Item i of that column: every item but the first starts on a chunk.
+__device__ __forceinline__ void item_at(uint32_t beg, uint32_t len, uint32_t i, uint32_t& b, uint32_t& l) {
+    const uint32_t h = beg & (kChunk - 1);
+    const uint32_t lo = i ? i * kSeg - h : 0u;
+    b = beg + lo;
+    l = min(len, (i + 1) * kSeg - h) - lo;
+}
+
+// Writes item (j, b, l) at position `at` of the global list of parity p.
+__device__ __forceinline__ void list_put(const SyncSearch& S, uint32_t p, unsigned long long at,
+                                         uint32_t j, uint32_t b, uint32_t l) {
+    if (at < S.icap) {
+        S.lj[p][at] = j;
+        S.lb[p][at] = b;
+        S.ll[p][at] = l;
+    } else {
+        fail(S.ctl, 7 /* ABFS_ERR_DEVICE */);
+    }
+}
+
+// Moves this CTA's list `q` to the global list of parity p (the spilled part
+// is there already).  A team barrier follows.  Whole CTA.
+__device__ __noinline__ void list_dump(SyncSmem& sm, const SyncSearch& S, uint32_t q, uint32_t p) {
+    const uint32_t c = min(sm.app[q][0], kThinCap);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        sm.base = c ? atomicAdd(&S.bar->lcnt[p], c) : 0u;
+        sm.app[q][0] = sm.app[q][1] = 0;
+    }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < c; i += kSyncThreads)
+        list_put(S, p, (unsigned long long)sm.base + i, sm.ij[q][i], sm.ib[q][i], sm.il[q][i]);
+}
+
+// Takes this CTA's even share of the global list of parity p (`items` items,
+// at most kThinCap per CTA) into its list `q`.  Whole CTA.
+__device__ __noinline__ void list_slice(SyncSmem& sm, const SyncSearch& S, const Team& T, uint32_t q,
+                                        uint32_t p, unsigned long long items) {
+    const unsigned long long lo = items * T.rank / T.size, hi = items * (T.rank + 1) / T.size;
+    const uint32_t c = (uint32_t)(hi - lo);
+    for (uint32_t i = threadIdx.x; i < c && lo + i < S.icap; i += kSyncThreads) {
+        sm.ij[q][i] = ld_l2(S.lj[p] + lo + i);
+        sm.ib[q][i] = ld_l2(S.lb[p] + lo + i);
+        sm.il[q][i] = ld_l2(S.ll[p] + lo + i);
+    }
+    if (threadIdx.x == 0) {
+        sm.app[q][0] = c;
+        sm.app[q][1] = ~0u;  // entries: not known
+        // every reservation in this list was made before the last barrier
+        if (T.rank == 0) st_relaxed(&S.bar->lcnt[p], 0u);
+    }
+    __syncthreads();
+}
+
+}  // namespace abfs

@@ -1,0 +1,552 @@
+// Level-synchronous engine: the levels of a search.
+// Part of sync_engine.cu, split by topic; included in order.
+#pragma once
+
+#include "sync_common.cuh"
+
+namespace abfs {
+
+// ---------------------------------------------------------------------------
+// thin levels
+// ---------------------------------------------------------------------------
+// The frontier is spread over the CTAs' private lists: a CTA expands the
+// columns it listed and lists the rows it wins, so a level needs no shared
+// queue, no reservation in global memory and no reload -- its dependent chain
+// is row index, atomicMin, barrier.  The lists are evened out only when a few
+// CTAs hold much more than their share (see sync_search).
+
+// Appends the rows won by this warp's lanes (row r, column [cb, ce)) to the
+// CTA's list `q` (level k + 1); what does not fit goes to the global list.
+// Whole warp.
+__device__ __forceinline__ void thin_append(SyncSmem& sm, const SyncSearch& S, uint32_t k, uint32_t q,
+                                            bool win, uint32_t r, uint32_t cb, uint32_t ce) {
+    if (!__any_sync(0xFFFFFFFFu, win)) return;
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t len = win ? ce - cb : 0u;
+    const uint32_t ns = items_of(cb, len);
+    const uint32_t ent = __reduce_add_sync(0xFFFFFFFFu, len);
+    const uint32_t j = ns && S.lab ? ld_ro(S.lab + r) : r;
+    // the next level starts with these row indices
+    if (ns) asm volatile("prefetch.global.L2 [%0];" ::"l"(S.rowidx + cb));
+    const bool longs = __any_sync(0xFFFFFFFFu, ns > 1);
+    uint32_t incl = 0, pre = 0, tot;
+    if (longs) {
+        incl = warp_incl_scan(ns);
+        tot = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    } else {
+        const uint32_t m = __ballot_sync(0xFFFFFFFFu, ns != 0);
+        tot = __popc(m);
+        pre = __popc(m & lanemask_lt());
+    }
+    // lane 0 reserves the items, lane 1 counts the entries
+    uint32_t at = 0;
+    if (lane < 2) at = atomicAdd(&sm.app[q][lane], lane ? ent : tot);
+    at = __shfl_sync(0xFFFFFFFFu, at, 0);
+    if (!longs && at + tot <= kThinCap) {
+        if (ns) {
+            sm.ij[q][at + pre] = j;
+            sm.ib[q][at + pre] = cb;
+            sm.il[q][at + pre] = len;
+        }
+        return;
+    }
+    // long columns or a full list: the warp writes the items together, those
+    // from position `room` on to the global list
+    if (!longs) incl = pre + (ns != 0);
+    const uint32_t p = (k + 1) & 1;
+    const uint32_t room = at < kThinCap ? min(kThinCap - at, tot) : 0u;
+    uint32_t spill = 0;
+    if (room < tot) {
+        if (lane == 0) spill = atomicAdd(&S.bar->lcnt[p], tot - room);
+        spill = __shfl_sync(0xFFFFFFFFu, spill, 0);
+    }
+    for (uint32_t x0 = 0; x0 < tot; x0 += 32) {
+        const uint32_t x = x0 + lane;
+        uint32_t own = 0;  // the first lane whose inclusive count exceeds x
+#pragma unroll
+        for (uint32_t d = 16; d > 0; d >>= 1)
+            if (x >= __shfl_sync(0xFFFFFFFFu, incl, own + d - 1)) own += d;
+        const uint32_t oj = __shfl_sync(0xFFFFFFFFu, j, own), ob = __shfl_sync(0xFFFFFFFFu, cb, own);
+        const uint32_t ol = __shfl_sync(0xFFFFFFFFu, len, own);
+        const uint32_t of = __shfl_sync(0xFFFFFFFFu, incl - ns, own);
+        if (x < tot) {
+            uint32_t b, l;
+            item_at(ob, ol, x - of, b, l);
+            if (x < room) {
+                sm.ij[q][at + x] = oj;
+                sm.ib[q][at + x] = b;
+                sm.il[q][at + x] = l;
+            } else {
+                list_put(S, p, (unsigned long long)spill + (x - room), oj, b, l);
+            }
+        }
+    }
+}
+
+// Expands the columns of this CTA's list of level k (list k & 1) into its list
+// of level k + 1.  The warps share the list's batches of 32 items evenly; the
+// warps of a batch take its groups of 32 entries in turn, one entry per lane
+// and kThinIlp groups in flight, so that one hub or a handful of columns keeps
+// all of them busy.  Whole CTA.
+constexpr int kThinIlp = 2;
+
+template <bool SIG>
+__device__ __forceinline__ void thin_level(SyncSmem& sm, const SyncSearch& S, uint32_t k, SyncTally& t) {
+    const uint32_t cur = k & 1;
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t cnt = min(sm.app[cur][0], kThinCap);
+    // batches of 32 items, rounded up to a power of two (at most one per warp)
+    const uint32_t lb = cnt > 32 ? 32 - __clz((cnt - 1) / 32) : 0;
+    const uint32_t batch = warp & ((1u << lb) - 1u), nth = warp >> lb;
+    const uint32_t i0 = 32 * batch;
+    if (i0 >= cnt || (lb == 0 && 32 * nth >= sm.app[cur][1])) return;
+    const uint32_t step = (32 * kSyncWarps) >> lb;  // entries between a warp's groups
+    const uint32_t le_mask = (2u << lane) - 1u;
+    const unsigned long long hi = (unsigned long long)(k + 1) << 32;
+    const uint32_t m = min(32u, cnt - i0);
+    uint32_t j = 0, beg = 0, len = 0;
+    if (lane < m) {
+        j = sm.ij[cur][i0 + lane];
+        beg = sm.ib[cur][i0 + lane];
+        len = sm.il[cur][i0 + lane];
+    }
+    if (nth == 0) t.read += len;
+    const uint32_t incl = warp_incl_scan(len);
+    const uint32_t total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    const uint32_t first = incl - len;  // this item's first entry
+    const uint32_t shift = beg - first;
+    // a warp with a group or two is bound by latency: the columns of all rows
+    // are looked up beside the claims instead of after them
+    const bool early = total <= kThinIlp * step;
+    for (uint32_t e0 = 32 * nth; e0 < total; e0 += kThinIlp * step) {
+        uint32_t r[kThinIlp], jj[kThinIlp];
+#pragma unroll
+        for (int u = 0; u < kThinIlp; ++u) {
+            const uint32_t g = e0 + u * step;
+            r[u] = kUnset;
+            jj[u] = 0;
+            if (g < total) {
+                const uint32_t rel = first - g;
+                const uint32_t before = __popc(__ballot_sync(0xFFFFFFFFu, lane < m && first < g));
+                const uint32_t w =
+                    __reduce_or_sync(0xFFFFFFFFu, (lane < m && rel < 32u) ? 1u << rel : 0u);
+                // the item of entry g + lane
+                const uint32_t own = (before + __popc(w & le_mask) - 1u) & 31u;
+                const uint32_t pos = __shfl_sync(0xFFFFFFFFu, shift, own) + g + lane;
+                jj[u] = __shfl_sync(0xFFFFFFFFu, j, own);
+                if (g + lane < total) r[u] = ld_ro(S.rowidx + pos);
+            }
+        }
+        unsigned long long old[kThinIlp];
+        uint32_t cb[kThinIlp], ce[kThinIlp];
+#pragma unroll
+        for (int u = 0; u < kThinIlp; ++u) {
+            old[u] = 0;
+            cb[u] = ce[u] = 0;
+            if (r[u] != kUnset) {
+                old[u] = atomicMin(S.key + r[u], hi | jj[u]);
+                if (early) {
+                    cb[u] = ld_ro(S.colptr + r[u]);
+                    ce[u] = ld_ro(S.colptr + r[u] + 1);
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kThinIlp; ++u) {
+            if (e0 + u * step >= total) break;
+            const bool pass = r[u] != kUnset && (uint32_t)(old[u] >> 32) > k;
+            const bool win = pass && old[u] == kKeyUnset;
+            t.unmasked += pass;
+            if (win) {
+                ++t.verts;
+                t.levels = k + 2;
+            }
+            if (SIG && pass) red_add64(S.sigma + r[u], ld_l2(S.sigma + jj[u]));
+            if (win && !early) {
+                cb[u] = ld_ro(S.colptr + r[u]);
+                ce[u] = ld_ro(S.colptr + r[u] + 1);
+            }
+            thin_append(sm, S, k, cur ^ 1, win, r[u], cb[u], ce[u]);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// wide levels
+// ---------------------------------------------------------------------------
+// The frontier is a list in global memory.  A row is tested against the
+// visited bitmap (frozen during the level) and claimed by a 32-bit reduction
+// on the low half of its key word, whose all-ones high half still says
+// "unset"; after a barrier, sync_extract reads the new rows off the bitmap and
+// the keys.  (The bitmap in shared memory, whole or in part, costs the L1 that
+// the misses of the other loads wait in: an R-MAT of scale 20 the same, of
+// scale 22 758 -> 877 us.)
+
+// Bits of word w that stand for vertices.
+__device__ __forceinline__ uint32_t word_mask(const SyncSearch& S, uint32_t w) {
+    return w == S.nwords - 1 && (S.n & 31) ? (1u << (S.n & 31)) - 1u : 0xFFFFFFFFu;
+}
+
+// Expands the `items` items of the global list of level k.  A warp takes up to
+// 32 items at a time and walks their chunks of four row indices, one 16-byte
+// load per lane and step, the next step's loads issued before this step's
+// tests; there is no barrier inside.  Whole CTA.
+template <bool SIG>
+__device__ __noinline__ void wide_expand(SyncSmem& sm, const SyncSearch& S, const Team& T, uint32_t k,
+                                         unsigned long long items) {
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t le_mask = (2u << lane) - 1u;
+    const uint32_t p = k & 1;
+    // The list is dealt out to the CTAs in runs of items, round robin, and a CTA's
+    // runs to its warps as they become free, by a counter in shared memory (one
+    // counter for the whole team, taken at about 2 ns a time, set the pace of a
+    // level of 25 000 runs).  A run is about four steps of 32 chunks, so that one
+    // full of hub items does not outlast the level, and short enough for four
+    // per warp.
+    const uint32_t W = T.size * kSyncWarps;
+    const unsigned long long four = 4ull * 32 * kChunk * items / (sm.entries + kChunk * items);
+    const uint32_t run = (uint32_t)max(1ull, min(min(32ull, four), items / (4ull * W)));
+    const unsigned long long runs = (items + run - 1) / run;
+    const uint64_t pol = evict_first_policy();
+    const uint32_t* const bm = S.bm;
+    uint32_t* const klo = reinterpret_cast<uint32_t*>(S.key);
+    SyncTally t;
+    // the items of the run after this one
+    uint32_t nj = 0, nbeg = 0, nlen = 0;
+    auto fetch = [&]() {
+        uint32_t x = 0;
+        if (lane == 0) x = atomicAdd(&sm.tick, 1u);
+        const unsigned long long c = (unsigned long long)__shfl_sync(0xFFFFFFFFu, x, 0) * T.size + T.rank;
+        const unsigned long long at = c * run + lane;
+        nj = nbeg = nlen = 0;
+        if (lane < run && at < items) {
+            nj = ld_l2(S.lj[p] + at);
+            nbeg = ld_l2(S.lb[p] + at);
+            nlen = ld_l2(S.ll[p] + at);
+        }
+        return c < runs;
+    };
+    bool more = fetch();
+    while (more) {
+        const uint32_t j = nj, beg = nbeg, len = nlen;
+        more = fetch();
+        t.read += len;
+        const uint32_t nch = len ? ((beg & (kChunk - 1)) + len + kChunk - 1) / kChunk : 0u;
+        const uint32_t incl = warp_incl_scan(nch);
+        const uint32_t total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+        const uint32_t first = incl - nch;
+        const uint32_t shift = beg / kChunk - first;  // chunk number minus position
+        const uint32_t end = beg + len;
+        uint32_t started = 0;
+        // row indices of a lane's chunk, which of them belong to its column (bits
+        // of ok) and the column's label.  The raw indices are kept as loaded:
+        // anything computed from them here would wait for the load.
+        auto load = [&](uint32_t g, uint4& r, uint32_t& ok, uint32_t& jj) {
+            const uint32_t rel = first - g;
+            const uint32_t w = __reduce_or_sync(0xFFFFFFFFu, (nch && rel < 32u) ? 1u << rel : 0u);
+            const uint32_t own = (started + __popc(w & le_mask) - 1u) & 31u;
+            started += __popc(w);
+            const uint32_t pos = (__shfl_sync(0xFFFFFFFFu, shift, own) + g + lane) * kChunk;
+            const uint32_t lo = __shfl_sync(0xFFFFFFFFu, beg, own);
+            const uint32_t up = __shfl_sync(0xFFFFFFFFu, end, own);
+            jj = __shfl_sync(0xFFFFFFFFu, j, own);
+            ok = 0;
+            if (g + lane < total) {
+                // entries [max(pos, lo), min(pos + 4, up)) of the chunk
+                const uint32_t skip = lo > pos ? lo - pos : 0u;
+                const uint32_t have = min(up - pos, kChunk);
+                ok = (1u << have) - (1u << skip);
+                if ((unsigned long long)pos + kChunk <= S.nnz) {
+                    r = ld_row4(S.rowidx + pos, 0, pol);
+                } else {
+                    // the last chunk of the row array
+                    const uint32_t* const x = S.rowidx + pos;
+                    r.x = (ok & 1u) ? ld_ro(x) : 0u;
+                    r.y = (ok & 2u) ? ld_ro(x + 1) : 0u;
+                    r.z = (ok & 4u) ? ld_ro(x + 2) : 0u;
+                    r.w = 0u;
+                }
+            }
+        };
+        uint4 rr = make_uint4(0, 0, 0, 0);
+        uint32_t ok = 0, jj = 0;
+        if (total) load(0, rr, ok, jj);
+        for (uint32_t g = 0; g < total; g += 32) {
+            uint4 rr2 = make_uint4(0, 0, 0, 0);
+            uint32_t ok2 = 0, jj2 = 0;
+            if (g + 32 < total) load(g + 32, rr2, ok2, jj2);
+            const uint32_t r[kChunk] = {rr.x, rr.y, rr.z, rr.w};
+            uint32_t w[kChunk];
+#pragma unroll
+            for (uint32_t q = 0; q < kChunk; ++q)
+                w[q] = (ok >> q) & 1u ? ld_frozen(bm + (r[q] >> 5)) : 0xFFFFFFFFu;
+#pragma unroll
+            for (uint32_t q = 0; q < kChunk; ++q) {
+                if (!((w[q] >> (r[q] & 31)) & 1u)) {
+                    ++t.unmasked;
+                    red_min32(klo + 2ull * r[q], jj);
+                    if (SIG) red_add64(S.sigma + r[q], ld_l2(S.sigma + jj));
+                }
+            }
+            rr = rr2;
+            ok = ok2;
+            jj = jj2;
+        }
+    }
+    tally_add(sm, t.read, t.unmasked);
+}
+
+// The visited bitmap (and, for the hybrid, the frontier bitmap of level k)
+// from the key words, after thin levels.  Rows that no column contains count
+// as visited.  A warp has the keys of kBitmapWords words in flight: with four,
+// 33 MB of keys took 25 us.  Whole CTA.
+constexpr int kBitmapWords = 8;
+
+__device__ __noinline__ void sync_bitmaps(const SyncSearch& S, const Team& T, uint32_t k) {
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t W = T.size * kSyncWarps;
+    constexpr int Q = kBitmapWords;
+    for (uint32_t w0 = (warp * T.size + T.rank) * Q; w0 < S.nwords; w0 += Q * W) {
+        uint32_t lv[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const unsigned long long v = ((unsigned long long)w0 + q) * 32 + lane;
+            lv[q] = v < S.n ? (uint32_t)(ld_relaxed64(S.key + v) >> 32) : kUnset;
+        }
+        uint32_t vis = 0, fr = 0;  // lane q: word w0 + q
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const uint32_t a = __ballot_sync(0xFFFFFFFFu, lv[q] != kUnset);
+            const uint32_t b = __ballot_sync(0xFFFFFFFFu, lv[q] == k);
+            if (lane == (uint32_t)q) {
+                vis = a;
+                fr = b;
+            }
+        }
+        const uint32_t w = w0 + lane;
+        if (lane < (uint32_t)Q && w < S.nwords) {
+            if (S.inb) vis |= ~ld_ro(S.inb + w) & word_mask(S, w);
+            S.bm[w] = vis;
+            if (S.bu_alpha) S.fbm[k & 1][w] = fr;
+        }
+    }
+}
+
+// The frontier list of level k + 1.  FROM_KEYS: after a wide level, its new
+// vertices are those outside the bitmap whose key has a parent; they get their
+// level, join the bitmap (each word has one writer) and make up the frontier
+// bitmap of level k + 1.  Otherwise that bitmap is there already (after a
+// bottom-up level, which counted its vertices).
+//
+// Two passes over a warp's words, so that the CTA meets once and reserves its
+// items with one atomic: the first finds the new vertices and counts their
+// items, kExtractWords words at a time in flight, the second reads the columns
+// again (from L2) and writes the items in order.  One pass with a meeting and a
+// reservation per 8192 vertices took 58 us for two million new vertices of
+// four million, most of it waiting.  Whole CTA.
+constexpr uint32_t kExtractWords = 8;
+
+template <bool FROM_KEYS>
+__device__ __noinline__ void sync_extract(SyncSmem& sm, const SyncSearch& S, const Team& T, uint32_t k) {
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr uint32_t Q = kExtractWords;
+    const uint32_t pn = (k + 1) & 1;
+    const uint32_t W = T.size * kSyncWarps;
+    const uint32_t g0 = (warp * T.size + T.rank) * Q;  // groups of Q words, round robin
+    uint32_t* const khi = reinterpret_cast<uint32_t*>(S.key) + 1;
+    uint32_t verts = 0, entries = 0, mine = 0;
+    for (uint32_t wb = g0; wb < S.nwords; wb += Q * W) {
+        const bool own = lane < Q && wb + lane < S.nwords;
+        uint32_t word = 0, seen = 0, add = 0;
+        if (own) {
+            if (FROM_KEYS) {
+                seen = ld_l2(S.bm + wb + lane);
+                word = ~seen & word_mask(S, wb + lane);
+            } else {
+                word = ld_l2(S.fbm[pn] + wb + lane);
+            }
+        }
+        const unsigned long long v0 = (unsigned long long)wb * 32 + lane;
+        bool fresh[Q];
+#pragma unroll
+        for (uint32_t q = 0; q < Q; ++q) {
+            const uint32_t c = __shfl_sync(0xFFFFFFFFu, word, q);
+            fresh[q] = (c >> lane) & 1u;
+            if (FROM_KEYS && fresh[q]) fresh[q] = (uint32_t)ld_l2(S.key + v0 + 32 * q) != kUnset;
+        }
+#pragma unroll
+        for (uint32_t q = 0; q < Q; ++q) {
+            if (FROM_KEYS) {
+                const uint32_t bits = __ballot_sync(0xFFFFFFFFu, fresh[q]);
+                if (lane == q) add = bits;
+            }
+            if (fresh[q]) {
+                const uint32_t cb = ld_ro(S.colptr + v0 + 32 * q);
+                const uint32_t len = ld_ro(S.colptr + v0 + 32 * q + 1) - cb;
+                if (FROM_KEYS) khi[2 * (v0 + 32 * q)] = k + 1;
+                ++verts;
+                entries += len;
+                mine += items_of(cb, len);
+            }
+        }
+        if (FROM_KEYS && own) {
+            if (add) S.bm[wb + lane] = seen | add;
+            S.fbm[pn][wb + lane] = add;
+        }
+    }
+    const uint32_t wt = __reduce_add_sync(0xFFFFFFFFu, mine);
+    if (lane == 0) sm.wsum[warp] = wt;
+    __syncthreads();
+    if (warp == 0) {
+        const uint32_t x = sm.wsum[lane];
+        const uint32_t incl = warp_incl_scan(x);
+        uint32_t base = 0;
+        if (lane == 31) {
+            if (incl) base = atomicAdd(&S.bar->lcnt[pn], incl);
+            sm.app[0][0] = incl;
+        }
+        base = __shfl_sync(0xFFFFFFFFu, base, 31);
+        sm.wpre[lane] = base + incl - x;
+    }
+    if (FROM_KEYS) {
+        verts = __reduce_add_sync(0xFFFFFFFFu, verts);
+        entries = __reduce_add_sync(0xFFFFFFFFu, entries);
+        if (lane == 0 && verts) {
+            atomicAdd(&sm.verts, verts);
+            atomicAdd(&sm.ent, entries);
+        }
+    }
+    __syncthreads();
+    if (!wt) return;
+    uint32_t at = sm.wpre[warp];
+    for (uint32_t wb = g0; wb < S.nwords; wb += Q * W) {
+        // (this lane's own words of the first pass)
+        const uint32_t word = lane < Q && wb + lane < S.nwords ? ld_l2(S.fbm[pn] + wb + lane) : 0u;
+        if (!__any_sync(0xFFFFFFFFu, word != 0)) continue;
+        const unsigned long long v0 = (unsigned long long)wb * 32 + lane;
+        uint32_t cb[Q], len[Q];
+#pragma unroll
+        for (uint32_t q = 0; q < Q; ++q) {
+            const uint32_t c = __shfl_sync(0xFFFFFFFFu, word, q);
+            cb[q] = len[q] = 0;
+            if ((c >> lane) & 1u) {
+                cb[q] = ld_ro(S.colptr + v0 + 32 * q);
+                len[q] = ld_ro(S.colptr + v0 + 32 * q + 1) - cb[q];
+            }
+        }
+#pragma unroll
+        for (uint32_t q = 0; q < Q; ++q) {
+            const uint32_t ns = items_of(cb[q], len[q]);
+            if (!__any_sync(0xFFFFFFFFu, ns != 0)) continue;
+            const uint32_t incl = warp_incl_scan(ns);
+            if (ns) {
+                const unsigned long long v = v0 + 32 * q;
+                const uint32_t j = S.lab ? ld_ro(S.lab + v) : (uint32_t)v;
+                for (uint32_t i = 0; i < ns; ++i) {
+                    uint32_t b, l;
+                    item_at(cb[q], len[q], i, b, l);
+                    list_put(S, pn, (unsigned long long)at + incl - ns + i, j, b, l);
+                }
+            }
+            at += __shfl_sync(0xFFFFFFFFu, incl, 31);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// hybrid: bottom-up levels (direction optimisation; not the paper's method)
+// ---------------------------------------------------------------------------
+// As in the unit scheduler (engine_phases.cuh): an unvisited vertex scans its
+// ascending column for the first vertex of the frontier bitmap, which is its
+// least-index parent.  The CTAs take groups of four words in turn, a CTA's
+// warps its groups as they become free.
+constexpr uint32_t kBuWords = 4;
+
+__device__ __noinline__ void sync_bottom_up(SyncSmem& sm, const SyncSearch& S, const Team& T, uint32_t k) {
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t p = k & 1, pn = p ^ 1;
+    const uint32_t* const fbm = S.fbm[p];
+    SyncTally t;
+    uint32_t verts = 0, entries = 0;
+    for (;;) {
+        uint32_t x = 0;
+        if (lane == 0) x = atomicAdd(&sm.tick, 1u);
+        x = __shfl_sync(0xFFFFFFFFu, x, 0);
+        const unsigned long long c = ((unsigned long long)x * T.size + T.rank) * kBuWords;
+        if (c >= S.nwords) break;
+        const uint32_t w0 = (uint32_t)c;
+        const bool own = lane < kBuWords && w0 + lane < S.nwords;
+        uint32_t seen = 0, cand = 0, add = 0;
+        if (own) {
+            seen = ld_l2(S.bm + w0 + lane);
+            cand = ~seen & word_mask(S, w0 + lane);
+        }
+        for (uint32_t q = 0; q < kBuWords; ++q) {
+            const uint32_t cw = __shfl_sync(0xFFFFFFFFu, cand, q);
+            if (!cw) continue;
+            const uint32_t v = (w0 + q) * 32 + lane;
+            uint32_t cb = 0, e = 0, end = 0, par = kUnset;
+            if ((cw >> lane) & 1u) {
+                cb = e = ld_ro(S.colptr + v);
+                end = ld_ro(S.colptr + v + 1);
+            }
+            for (uint32_t b = 0; b < 4 && e < end; ++b) {
+                uint32_t jj[4], fw[4];
+#pragma unroll
+                for (int x = 0; x < 4; ++x) jj[x] = e + x < end ? ld_ro(S.rowidx + e + x) : kUnset;
+#pragma unroll
+                for (int x = 0; x < 4; ++x) fw[x] = jj[x] != kUnset ? ld_frozen(fbm + (jj[x] >> 5)) : 0u;
+                t.read += min(4u, end - e);
+#pragma unroll
+                for (int x = 3; x >= 0; --x)
+                    if ((fw[x] >> (jj[x] & 31)) & 1u) par = jj[x];
+                e = par != kUnset ? end : e + 4;
+            }
+            uint32_t dm;
+            bool defer = par == kUnset && e < end;
+            while ((dm = __ballot_sync(0xFFFFFFFFu, defer)) != 0u) {
+                const uint32_t ldr = __ffs(dm) - 1;
+                const uint32_t le = __shfl_sync(0xFFFFFFFFu, e, ldr);
+                const uint32_t lend = __shfl_sync(0xFFFFFFFFu, end, ldr);
+                uint32_t found = kUnset;
+                for (uint32_t x = le; x < lend; x += 32) {
+                    const uint32_t idx = x + lane;
+                    const uint32_t j = idx < lend ? ld_ro(S.rowidx + idx) : kUnset;
+                    const bool hit = j != kUnset && ((ld_frozen(fbm + (j >> 5)) >> (j & 31)) & 1u);
+                    const uint32_t hb = __ballot_sync(0xFFFFFFFFu, hit);
+                    if (lane == 0) t.read += min(32u, lend - x);
+                    if (hb) {
+                        found = __shfl_sync(0xFFFFFFFFu, j, __ffs(hb) - 1);
+                        break;
+                    }
+                }
+                if (lane == ldr) {
+                    par = found;
+                    defer = false;
+                }
+            }
+            const bool got = par != kUnset;
+            if (got) {
+                S.key[v] = (unsigned long long)(k + 1) << 32 | par;
+                ++t.unmasked;
+                ++verts;
+                entries += end - cb;
+            }
+            const uint32_t bits = __ballot_sync(0xFFFFFFFFu, got);
+            if (lane == q) add = bits;
+        }
+        if (own) {
+            if (add) S.bm[w0 + lane] = seen | add;
+            S.fbm[pn][w0 + lane] = add;
+        }
+    }
+    tally_add(sm, t.read, t.unmasked);
+    verts = __reduce_add_sync(0xFFFFFFFFu, verts);
+    entries = __reduce_add_sync(0xFFFFFFFFu, entries);
+    if (lane == 0 && verts) {
+        atomicAdd(&sm.verts, verts);
+        atomicAdd(&sm.ent, entries);
+    }
+}
+
+}  // namespace abfs

@@ -1,0 +1,391 @@
+// Level-synchronous engine: a whole search.
+// Part of sync_engine.cu, split by topic; included in order.
+#pragma once
+
+#include "sync_levels.cuh"
+
+namespace abfs {
+
+// One trace entry (abfs_run_trace), written by the team's first thread.
+__device__ __forceinline__ void sync_trace(const SyncSearch& S, const Team& T, uint32_t kind, uint32_t k,
+                                           uint32_t alone, uint32_t items, uint32_t verts, uint32_t ent) {
+    if (!S.trace || T.rank != 0 || threadIdx.x != 0) return;
+    const uint32_t tn = ld_relaxed(&S.ctl->trace_n);
+    if (tn >= S.trace_cap) return;
+    const uint64_t now = globaltimer();
+    S.trace[2 * tn] = make_uint4((uint32_t)now, (uint32_t)(now >> 32), (kind << 24) | (k & 0xFFFFFFu), alone);
+    S.trace[2 * tn + 1] = make_uint4(items, verts, ent, 0u);
+    st_relaxed(&S.ctl->trace_n, tn + 1);
+}
+
+// Clears the search's words, control block and (path counts) sums, and gives
+// the source its key.  Whole team.
+__device__ __forceinline__ void sync_init(const SyncSearch& S, const Team& T) {
+    const uint32_t stride = T.size * kSyncThreads;
+    const uint32_t t0 = T.rank * kSyncThreads + threadIdx.x;
+    // two keys per 16-byte store
+    ulonglong2* const k2 = reinterpret_cast<ulonglong2*>(S.key);
+    for (uint32_t i = t0; i < S.n / 2; i += stride) {
+        ulonglong2 x = make_ulonglong2(kKeyUnset, kKeyUnset);
+        if (2 * i == S.src) x.x = S.src_label;
+        if (2 * i + 1 == S.src) x.y = S.src_label;
+        k2[i] = x;
+    }
+    if ((S.n & 1) && t0 == 0) S.key[S.n - 1] = S.n - 1 == S.src ? S.src_label : kKeyUnset;
+    if (S.sigma)
+        for (uint32_t v = t0; v < S.n; v += stride) S.sigma[v] = v == S.src ? 1ull : 0ull;
+    if (T.rank == 0) {
+        uint32_t* c = reinterpret_cast<uint32_t*>(S.ctl);
+        for (uint32_t w = threadIdx.x; w < sizeof(InstCtl) / 4; w += kSyncThreads) c[w] = 0u;
+    }
+}
+
+// The caller's level and parent of every vertex from the key words; on a
+// relabelled graph, gathered in input order (vertices without edges of an
+// undirected graph, from n_keep on, are known to be unreached).  Four vertices
+// per thread and step, two steps in flight.  Whole team.
+__device__ __noinline__ void sync_outputs(const SyncSearch& S, const Team& T) {
+    const uint32_t stride = T.size * kSyncThreads;
+    const uint32_t t0 = T.rank * kSyncThreads + threadIdx.x;
+    const uint32_t quads = S.n / 4;
+    const bool vec = ((reinterpret_cast<uintptr_t>(S.level) | reinterpret_cast<uintptr_t>(S.parent)) & 15u) == 0;
+    auto key_at = [&](uint32_t o) -> unsigned long long {
+        if (!S.pos) return ld_relaxed64(S.key + o);
+        const uint32_t i = ld_ro(S.pos + o);
+        return i < S.n_keep || i == S.src ? ld_relaxed64(S.key + i) : kKeyUnset;
+    };
+    auto put = [&](uint32_t q, const unsigned long long (&x)[4]) {
+        const int4 lv = make_int4((int)(x[0] >> 32), (int)(x[1] >> 32), (int)(x[2] >> 32), (int)(x[3] >> 32));
+        const uint4 pr = make_uint4((uint32_t)x[0], (uint32_t)x[1], (uint32_t)x[2], (uint32_t)x[3]);
+        if (vec) {
+            reinterpret_cast<int4*>(S.level)[q] = lv;
+            reinterpret_cast<uint4*>(S.parent)[q] = pr;
+        } else {
+            int32_t* const l = S.level + 4ull * q;
+            uint32_t* const p = S.parent + 4ull * q;
+            l[0] = lv.x, l[1] = lv.y, l[2] = lv.z, l[3] = lv.w;
+            p[0] = pr.x, p[1] = pr.y, p[2] = pr.z, p[3] = pr.w;
+        }
+    };
+    for (uint32_t q = t0; q < quads; q += 2 * stride) {
+        const bool two = q + stride < quads;
+        unsigned long long a[4], b[4];
+#pragma unroll
+        for (int x = 0; x < 4; ++x) a[x] = key_at(4 * q + x);
+        if (two) {
+#pragma unroll
+            for (int x = 0; x < 4; ++x) b[x] = key_at(4 * (q + stride) + x);
+        }
+        put(q, a);
+        if (two) put(q + stride, b);
+    }
+    for (uint32_t v = 4 * quads + t0; v < S.n; v += stride) {
+        const unsigned long long x = key_at(v);
+        S.level[v] = (int32_t)(x >> 32);
+        S.parent[v] = (uint32_t)x;
+    }
+}
+
+// The team's share of level 0's list: the items of the source's column.
+__device__ __forceinline__ void sync_source(SyncSmem& sm, const SyncSearch& S, const Team& T,
+                                            unsigned long long& items) {
+    const uint32_t cb = ld_ro(S.colptr + S.src);
+    const uint32_t len = ld_ro(S.colptr + S.src + 1) - cb;
+    items = items_of(cb, len);
+    const uint32_t lo = (uint32_t)(items * T.rank / T.size), hi = (uint32_t)(items * (T.rank + 1) / T.size);
+    // a column too long for the team's lists starts in the global list
+    const bool global = items > (unsigned long long)T.size * kThinCap;
+    for (uint32_t i = lo + threadIdx.x; i < hi; i += kSyncThreads) {
+        uint32_t b, l;
+        item_at(cb, len, i, b, l);
+        if (global) {
+            list_put(S, 0, i, S.src_label, b, l);
+        } else {
+            sm.ij[0][i - lo] = S.src_label;
+            sm.ib[0][i - lo] = b;
+            sm.il[0][i - lo] = l;
+        }
+    }
+    if (threadIdx.x == 0) {
+        sm.step = sm.tick = 0;
+        sm.word[0] = sm.word[1] = sm.aux[0] = sm.aux[1] = 0;
+        sm.app[0][0] = global ? 0u : hi - lo;
+        sm.app[0][1] = ~0u;  // entries: not known
+        sm.app[1][0] = sm.app[1][1] = 0;
+        sm.verts = sm.ent = 0;
+        sm.lim_items = 64;
+        sm.lim_ent = 2048;
+        sm.bu = 0;
+        sm.nf = 1;
+        sm.seen = sm.entries = len;
+        sm.st_read = sm.st_unmasked = 0;
+        sm.st_verts = T.rank == 0 ? 1 : 0;
+        sm.st_ent = T.rank == 0 ? len : 0;
+        sm.levels = 1;
+    }
+}
+
+// A list is heavy above twice an even share of the current level and what a
+// CTA expands without queueing (64 items: two per warp; 2048 entries: two
+// groups per warp).
+__device__ __forceinline__ void heavy_limits(SyncSmem& sm, const Team& T, float items, float ent) {
+    const float share = 2.f / (float)T.size;
+    sm.lim_items = 64u + (uint32_t)(items * share);
+    sm.lim_ent = 2048u + (uint32_t)(ent * share);
+}
+__device__ __forceinline__ uint32_t tot_items(unsigned long long tot) {
+    return (uint32_t)(tot >> kItemShift) & ((1u << (kHeavyShift - kItemShift)) - 1u);
+}
+__device__ __forceinline__ uint32_t tot_ent(unsigned long long tot) {
+    return ((uint32_t)tot & ((1u << kItemShift) - 1u)) * kEntUnit;
+}
+
+// Entries from which the level of a frontier of `items` items is wide.
+__device__ __forceinline__ unsigned long long wide_line(const SyncSearch& S, unsigned long long items,
+                                                        unsigned long long ent) {
+    return ent >= S.hub_avg * items ? S.wide_hub : S.wide_min;
+}
+
+// Thread 0 after the barrier that ended a thin level (tot: the barrier's
+// totals): the next level's kind.  The first tests are the usual case.
+__device__ __forceinline__ uint32_t thin_next(SyncSmem& sm, const SyncSearch& S, const Team& T,
+                                              unsigned long long tot, unsigned long long aux, bool want_aux) {
+    const uint32_t flags = (uint32_t)(tot >> kHeavyShift);
+    const uint32_t items = tot_items(tot), ent = tot_ent(tot);
+    sm.items = items;
+    if (items == 0) return kActDone;
+    if (flags == 0 && ent < S.wide_hub && !want_aux) return kActThin;
+    if (tot == ~0ull) return kActFailed;
+    if (want_aux) {
+        sm.nf = items;
+        sm.entries = aux;
+        sm.seen += aux;
+        if (S.bu_alpha) {
+            const unsigned long long mu = S.nnz > sm.seen ? S.nnz - sm.seen : 0ull;
+            sm.bu = aux * S.bu_alpha > mu;
+            if (sm.bu) return kActBottomUp;
+        }
+    }
+    if (ent >= wide_line(S, items, ent) || items > T.size * kThinCap) return kActWide;
+    // a list is full, or a few CTAs hold much more than the others (but when
+    // the frontier has outgrown the limits, lists above them say nothing)
+    const uint32_t heavy = flags & 0xFFu;
+    const float n2 = 2.f / (float)T.size;
+    const bool grown = (float)sm.lim_items < n2 * (float)items && (float)sm.lim_ent < n2 * (float)ent;
+    if ((flags >> 8) || (heavy && 2 * heavy <= T.size && !grown)) {
+        heavy_limits(sm, T, (float)items, (float)ent);
+        return kActEven;
+    }
+    return kActThin;
+}
+
+// Runs thin levels from level k on until another kind of level follows
+// (sm.act); returns that level's number.  A function of its own, so that the
+// loop that long searches spend their time in has its own registers.
+// Whole CTA.
+template <bool SIG>
+__device__ __noinline__ uint32_t thin_run(SyncSmem& sm, const SyncSearch& S, const Team& team, uint32_t k) {
+    const Team T = team;
+    const bool lead = threadIdx.x == 0;
+    const bool want_aux = S.bu_alpha != 0 || S.trace != nullptr;
+    SyncTally t;
+    uint32_t act;
+    do {
+        if (S.trace) sync_trace(S, T, kPhLevel, k, 4u, (uint32_t)sm.items, (uint32_t)sm.nf, (uint32_t)sm.entries);
+        thin_level<SIG>(sm, S, k, t);
+        __syncthreads();
+        unsigned long long tot = 0, aux = 0;
+        if (lead) {
+            const uint32_t cur = k & 1;
+            const uint32_t c = sm.app[cur ^ 1][0], e = sm.app[cur ^ 1][1];
+            unsigned long long add =
+                (unsigned long long)min(c, kItemClamp) << kItemShift | min(e / kEntUnit, kEntClamp);
+            if (c > sm.lim_items || e > sm.lim_ent) add += 1ull << kHeavyShift;
+            if (c > kThinCap) add += 1ull << kFullShift;
+            sm.app[cur][0] = sm.app[cur][1] = 0;
+            sm.st_ent += e;
+            aux = e;
+            tot = SIG || want_aux ? bar_wait<true>(sm, S, T, add, aux) : bar_wait<false>(sm, S, T, add, aux);
+            sm.act = thin_next(sm, S, T, tot, aux, want_aux);
+        }
+        __syncthreads();
+        ++k;
+        act = sm.act;
+        if (lead && act == kActThin) heavy_limits(sm, T, (float)tot_items(tot), (float)tot_ent(tot));
+    } while (act == kActThin);
+    tally_add(sm, t.read, t.unmasked);
+    t.verts = __reduce_add_sync(0xFFFFFFFFu, t.verts);
+    t.levels = __reduce_max_sync(0xFFFFFFFFu, t.levels);
+    if ((threadIdx.x & 31) == 0 && t.verts) {
+        atomicAdd(&sm.st_verts, (unsigned long long)t.verts);
+        atomicMax(&sm.levels, t.levels);
+    }
+    __syncthreads();
+    return k;
+}
+
+// Thread 0 after the barrier that ended a wide or a bottom-up level.
+__device__ __forceinline__ uint32_t wide_next(SyncSmem& sm, const SyncSearch& S, const Team& T, bool bottom_up,
+                                              unsigned long long tot, unsigned long long aux) {
+    if (tot == ~0ull) return kActFailed;
+    sm.items = tot;
+    sm.nf = aux >> kAuxShift;
+    sm.entries = aux & ((1ull << kAuxShift) - 1);
+    sm.seen += sm.entries;
+    if (bottom_up ? sm.nf == 0 : tot == 0) return kActDone;
+    if (S.bu_alpha) {
+        // the direction, as the unit scheduler chooses it (decide_next)
+        const unsigned long long mu = S.nnz > sm.seen ? S.nnz - sm.seen : 0ull;
+        sm.bu = sm.bu ? sm.nf * S.bu_beta >= S.n : sm.entries * S.bu_alpha > mu;
+        if (sm.bu) return kActBottomUp;
+    }
+    if (bottom_up || tot > (unsigned long long)T.size * kThinCap ||
+        sm.entries >= wide_line(S, tot, sm.entries) / 2)
+        return kActWide;
+    heavy_limits(sm, T, (float)tot, (float)sm.entries);
+    return kActSlice;
+}
+
+// Runs one search on this team.  The outputs and the control block are written
+// when it returns (to be read after the kernel).
+//
+// Thin levels hold while the frontier fits the CTAs' lists and its entries
+// stay below wide_line; wide levels until it fits again with less than half
+// of that (each thin -> wide switch rebuilds the bitmap, 8 bytes per vertex).
+// After a barrier thread 0 alone decides what follows: the same decision made
+// by every thread took 1.3 us a level on 32 warps.
+template <bool SIG>
+__device__ __forceinline__ void sync_search(SyncSmem& sm, const SyncSearch& S, const Team& T) {
+    const bool lead = threadIdx.x == 0;
+    unsigned long long items;
+    uint32_t k = 0, wide_levels = 0, act = kActThin;
+    sync_init(S, T);
+    sync_source(sm, S, T, items);
+    if (!team_sync(sm, S, T)) act = kActFailed;
+    else if (items == 0) act = kActDone;
+    else if (items > (unsigned long long)T.size * kThinCap) {
+        sync_bitmaps(S, T, 0);
+        act = team_sync(sm, S, T) ? kActWide : kActFailed;
+        if (lead) sm.items = items;
+        __syncthreads();
+    }
+    sync_trace(S, T, 0xFEu, 0, 0, 0, 1, 0);
+    while (act < kActDone) {
+        if (act == kActThin) {
+            k = thin_run<SIG>(sm, S, T, k);
+            act = sm.act;
+            const uint32_t p = k & 1;
+            if (act == kActEven || act == kActWide) {
+                const uint32_t mine = sm.app[p][0], ent = sm.app[p][1];
+                list_dump(sm, S, p, p);
+                if (act == kActWide) sync_bitmaps(S, T, k);
+                if (!team_sync(sm, S, T, mine, ent)) {
+                    act = kActFailed;
+                } else if (act == kActEven) {
+                    // exact totals now: the thin level's were clamped per CTA
+                    const unsigned long long all = sm.items, entries = sm.entries;
+                    if (all <= (unsigned long long)T.size * kThinCap && entries < wide_line(S, all, entries)) {
+                        list_slice(sm, S, T, p, p, all);
+                        // a failed append leaves the list incomplete
+                        if (lead) sm.act = ld_relaxed(&S.ctl->err) ? kActFailed : kActThin;
+                        __syncthreads();
+                        act = sm.act;
+                    } else {
+                        sync_bitmaps(S, T, k);
+                        act = team_sync(sm, S, T) ? kActWide : kActFailed;
+                        if (lead) {
+                            sm.items = all;
+                            sm.entries = entries;
+                        }
+                        __syncthreads();
+                    }
+                }
+            } else if (act == kActBottomUp) {
+                sync_trace(S, T, kPhBuPrep, k, 0u, 0u, 0u, 0u);
+                sync_bitmaps(S, T, k);
+                if (lead) {
+                    sm.app[p][0] = sm.app[p][1] = 0;
+                    if (T.rank == 0) st_relaxed(&S.bar->lcnt[p], 0u);
+                }
+                if (!team_sync(sm, S, T)) act = kActFailed;
+            }
+        } else if (act == kActSlice) {
+            list_slice(sm, S, T, k & 1, k & 1, sm.items);
+            act = kActThin;
+        } else {
+            const bool up = act == kActBottomUp;
+            // read by nobody any more, and used again at the next level
+            if (T.rank == 0 && lead) st_relaxed(&S.bar->lcnt[k & 1], 0u);
+            if (S.trace)
+                sync_trace(S, T, up ? kPhBottomUp : kPhLevelScan, k, 0u, (uint32_t)sm.items, (uint32_t)sm.nf,
+                           (uint32_t)sm.entries);
+            ++wide_levels;
+            if (up) {
+                sync_bottom_up(sm, S, T, k);
+            } else {
+                wide_expand<SIG>(sm, S, T, k, sm.items);
+                if (!team_sync(sm, S, T)) {
+                    act = kActFailed;
+                    break;
+                }
+                sync_trace(S, T, kPhExtract, k, 0u, 0u, 0u, 0u);
+                sync_extract<true>(sm, S, T, k);
+            }
+            __syncthreads();
+            if (lead) {
+                const uint32_t c = sm.app[0][0], v = sm.verts, e = sm.ent;
+                sm.app[0][0] = 0;
+                sm.verts = sm.ent = sm.tick = 0;
+                if (v) sm.levels = k + 2;
+                sm.st_verts += v;
+                sm.st_ent += e;
+                unsigned long long aux = (unsigned long long)v << kAuxShift | e;
+                const unsigned long long tot = bar_wait<true>(sm, S, T, c, aux);
+                sm.act = wide_next(sm, S, T, up, tot, aux);
+                // a failed append leaves a list incomplete: nothing reads it
+                if (sm.act < kActDone && ld_relaxed(&S.ctl->err)) sm.act = kActFailed;
+            }
+            __syncthreads();
+            ++k;
+            act = sm.act;
+            if (up && act == kActWide) {
+                // back to top-down levels: the list of the frontier bitmap
+                sync_extract<false>(sm, S, T, k - 1);
+                __syncthreads();
+                const uint32_t c = sm.app[0][0];
+                if (!team_sync(sm, S, T, c)) act = kActFailed;
+                else if (sm.items == 0) act = kActDone;
+                if (lead) sm.app[0][0] = 0;
+                __syncthreads();
+            }
+        }
+    }
+    sync_trace(S, T, 0xFFu, k, 0u, 0u, 0u, 0u);
+    if (act == kActDone) sync_outputs(S, T);
+    __syncthreads();
+    if (lead) {
+        InstCtl* c = S.ctl;
+        if (sm.st_read) atomicAdd(&c->entries_read, sm.st_read);
+        if (sm.st_unmasked) {
+            atomicAdd(&c->entries_unmasked, sm.st_unmasked);
+            atomicAdd(&c->claims, sm.st_unmasked);
+        }
+        if (sm.st_ent) atomicAdd(&c->nnz_reached, sm.st_ent);
+        if (sm.st_verts) atomicAdd(&c->reached, (uint32_t)sm.st_verts);
+        atomicMax(&c->levels, sm.levels);
+        if (T.rank == 0 && wide_levels) atomicAdd(&c->wide_levels, wide_levels);
+        // the last CTA to leave sets the status and clears the barrier's words
+        // for the next search
+        __threadfence();
+        if (atomicInc(&S.bar->exited, T.size - 1) == T.size - 1) {
+            __threadfence();
+            for (int b = 0; b < 2; ++b) {
+                S.bar->word[b] = S.bar->aux[b] = 0;
+                S.bar->lcnt[b] = 0;
+            }
+            c->status = ld_relaxed(&c->err) ? kFailed : kDone;
+        }
+    }
+}
+
+}  // namespace abfs

@@ -1,0 +1,78 @@
+"""The level-synchronous engine (default parameters) at the sizes where its
+lists, items, bitmaps and vector loads change shape, against the oracle."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import paper_1906_03113_gb300 as abfs  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    abfs.build()
+    abfs.load()
+    torch.cuda.set_device(0)
+
+
+def _hubs(lengths, seed):
+    """A directed two-level tree: vertex 0 reaches one hub per length, hub i
+    reaches that many leaves (shared among the hubs, so the least hub wins)."""
+    leaves = max(lengths)
+    first = 1 + len(lengths)
+    src, dst = [], []
+    rng = np.random.default_rng(seed)
+    for i, m in enumerate(lengths):
+        src.append(0)
+        dst.append(1 + i)
+        pick = rng.permutation(leaves)[:m] + first
+        src.extend([1 + i] * m)
+        dst.extend(pick.tolist())
+    return synth.from_arcs(first + leaves, src, dst, directed=True)
+
+
+GRAPHS = {
+    # column lengths around an item (256 entries less the head) and two, at
+    # every alignment of the column's start
+    "items": lambda: _hubs([1, 2, 3, 4, 5, 253, 254, 255, 256, 257, 258, 259, 509, 511, 512, 513, 1027], 1),
+    # one CTA's list overflows into the global list, then is evened out
+    "spill": lambda: _hubs([1500, 9000, 3000] + [2] * 3000, 2),
+    "star": lambda: synth.from_arcs(300001, [0] * 300000, list(range(1, 300001)), directed=False),
+    # dense enough for wide levels, from thin ones and back
+    "wide": lambda: synth.rmat(17, 16.0, seed=11),
+    "wide_er": lambda: synth.er(131071, 32.0, seed=12),
+    # vertex counts off every vector width
+    "odd": lambda: synth.rmat(13, 12.0, seed=13, n_keep=8190 - 27),
+}
+
+
+@pytest.mark.parametrize("name", list(GRAPHS))
+@pytest.mark.parametrize("shift", [0, 1])
+def test_default_engine_at_its_edges(name, shift):
+    g = GRAPHS[name]()
+    G = abfs.graph_create(g.colptr, g.rowidx, directed=g.directed)
+    deg = g.degrees()
+    for relabel in (False, True):
+        if relabel:
+            abfs.graph_relabel(G)
+        for s in sorted({0, int(np.argmax(deg)), g.n - 1}):
+            # outputs off 16-byte alignment when shift is 1
+            lev, par = (torch.full((g.n + 1,), 7, dtype=torch.int32, device="cuda")[shift:shift + g.n]
+                        for _ in range(2))
+            lo, po = oracle.bfs(g, s)
+            for kw in ({}, {"bottom_up_alpha": 4}):
+                _, _, st = abfs.run(G, s, lev, par, params=abfs.default_params(**kw), stats=True)
+                assert np.array_equal(lev.cpu().numpy(), lo), (name, s, kw)
+                assert np.array_equal(par.cpu().numpy(), po), (name, s, kw)
+                assert st["reached"] == int((lo >= 0).sum()) and st["levels"] == int(lo.max()) + 1
+                assert st["nnz_reached"] == int(deg[lo >= 0].sum())
+    lev, par, sig, st = abfs.run_counts(G, s, stats=True)
+    assert np.array_equal(sig.cpu().numpy().view(np.uint64), oracle.path_counts(g, s)), name
+    assert st["entries_read"] == st["nnz_reached"]
+    G.destroy()
