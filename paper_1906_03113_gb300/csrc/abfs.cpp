@@ -529,13 +529,12 @@ const abfs_params& pick_params(const abfs_graph_s* g, const abfs_params* params,
     return tmp;
 }
 
-// The search as the level-synchronous engine takes it: the workspace's buffers
+// The search as the level-synchronous engine takes it: a workspace's buffers
 // and the input CSC, or with `rel` the relabelled copy.
-SyncSearch make_sync(const abfs_graph_s* g, const Workspace& w, uint32_t source, bool rel,
-                     const abfs_params& p) {
+SyncSearch make_sync(const abfs_graph_s* g, char* base, const Layout& L, SyncBar* bar, uint32_t source,
+                     bool rel, const abfs_params& p) {
     SyncSearch S;
     std::memset(&S, 0, sizeof(S));
-    const Layout& L = w.L;
     S.colptr = rel ? g->r_colptr : g->d_colptr;
     S.rowidx = rel ? g->r_rowidx : g->d_rowidx;
     S.nnz = g->nnz;
@@ -550,16 +549,16 @@ SyncSearch make_sync(const abfs_graph_s* g, const Workspace& w, uint32_t source,
         S.n_keep = g->r_keep;
     }
     S.icap = L.icap;
-    S.key = reinterpret_cast<unsigned long long*>(w.base + L.skey);
-    S.bm = reinterpret_cast<uint32_t*>(w.base + L.bm[0]);
+    S.key = reinterpret_cast<unsigned long long*>(base + L.skey);
+    S.bm = reinterpret_cast<uint32_t*>(base + L.bm[0]);
     for (int i = 0; i < 2; ++i) {
-        S.fbm[i] = reinterpret_cast<uint32_t*>(w.base + L.fbm[i]);
-        S.lj[i] = reinterpret_cast<uint32_t*>(w.base + L.slist[i][0]);
-        S.lb[i] = reinterpret_cast<uint32_t*>(w.base + L.slist[i][1]);
-        S.ll[i] = reinterpret_cast<uint32_t*>(w.base + L.slist[i][2]);
+        S.fbm[i] = reinterpret_cast<uint32_t*>(base + L.fbm[i]);
+        S.lj[i] = reinterpret_cast<uint32_t*>(base + L.slist[i][0]);
+        S.lb[i] = reinterpret_cast<uint32_t*>(base + L.slist[i][1]);
+        S.ll[i] = reinterpret_cast<uint32_t*>(base + L.slist[i][2]);
     }
-    S.ctl = reinterpret_cast<InstCtl*>(w.base + L.ctl);
-    S.bar = reinterpret_cast<SyncBar*>(reinterpret_cast<char*>(w.d_done) + kBarAt);
+    S.ctl = reinterpret_cast<InstCtl*>(base + L.ctl);
+    S.bar = bar;
     // A wide level costs a bitmap (8 bytes per vertex), an extraction and a
     // barrier more than a thin one and saves a returned 64-bit atomic per entry.
     // Those atomics queue where many columns share hub rows, which a frontier
@@ -598,7 +597,8 @@ int enqueue_single(abfs_graph_s* g, uint32_t source, int32_t* level, int32_t* pa
     const uint32_t bu_ok = (!rel && !g->directed && g->sorted && !sigma) ? 1u : 0u;
     const int most = sync_applies(g->n, g->nnz, p) ? sync_max_ctas(g->device, g->sms) : 0;
     if (most > 0) {
-        SyncSearch S = make_sync(g, w, source, rel, p);
+        SyncBar* bar = reinterpret_cast<SyncBar*>(reinterpret_cast<char*>(w.d_done) + kBarAt);
+        SyncSearch S = make_sync(g, w.base, w.L, bar, source, rel, p);
         S.sigma = reinterpret_cast<unsigned long long*>(sigma);
         S.level = level;
         S.parent = reinterpret_cast<uint32_t*>(parent);
@@ -1113,6 +1113,7 @@ struct abfs_batch_s {
     Inst* d_insts = nullptr;
     uint32_t* d_done = nullptr;
     unsigned long long* d_beat = nullptr;
+    char* d_sync = nullptr;      // plans on the level-synchronous engine: descriptors, barriers, steps
     std::vector<size_t> ctl_off; // offset of each search instance's InstCtl in ws
     std::vector<uint32_t> qinst; // query -> the search instance that answers it
     uint32_t ninst = 0;          // search instances (a multi-source search answers several queries)
@@ -1129,12 +1130,77 @@ extern "C" int abfs_batch_destroy(abfs_batch_t b) {
     dev_free(b->d_insts);
     dev_free(b->d_done);
     dev_free(b->d_beat);
+    dev_free(b->d_sync);
     if (b->h_ctl) cudaFreeHost(b->h_ctl);
     delete b;
     return ABFS_OK;
 }
 
 namespace {
+
+// Which CTAs run which searches of a batch on the level-synchronous engine.
+struct TeamPlan {
+    std::vector<uint32_t> off;     // CTA c runs steps [off[c], off[c + 1]) ...
+    std::vector<SyncStep> steps;
+    std::vector<uint32_t> queue;   // ... and then searches of one CTA, largest first
+    int ctas = 0;
+};
+
+// Plans searches of the given sizes (`work`: microseconds on one CTA; `cap`:
+// largest useful team) onto at most `most` CTAs.  Every search gets CTAs in
+// proportion to its work, so that none outlasts the batch: the share per CTA is
+// searched for over a few values, each judged by the finish time of a greedy
+// schedule (largest first, onto the CTAs that are free first).
+TeamPlan plan_teams(const std::vector<double>& work, const std::vector<uint32_t>& cap, int most) {
+    constexpr double kFixed = 25.0;  // levels' barriers and chains, whatever the team
+    const size_t ns = work.size();
+    std::vector<uint32_t> order(ns);
+    for (size_t i = 0; i < ns; ++i) order[i] = (uint32_t)i;
+    std::stable_sort(order.begin(), order.end(), [&](uint32_t a, uint32_t b) { return work[a] > work[b]; });
+    double total = 0;
+    for (double w : work) total += w + kFixed;
+    TeamPlan best;
+    double best_end = INFINITY;
+    for (double f = 0.25; f < 4.0; f *= 1.25) {
+        const double share = total / most * f;
+        TeamPlan t;
+        std::vector<double> load((size_t)most, 0.0);
+        std::vector<std::vector<SyncStep>> steps((size_t)most);
+        std::vector<uint32_t> ctas((size_t)most);
+        double end = 0;
+        for (uint32_t q : order) {
+            const uint32_t size = (uint32_t)std::max(
+                1.0, std::min({std::ceil(work[q] / share), (double)cap[q], (double)most}));
+            if (size == 1) {
+                // from the queue, onto whichever CTA is free first
+                const auto it = std::min_element(load.begin(), load.end());
+                *it += work[q] + kFixed;
+                end = std::max(end, *it);
+                t.queue.push_back(q);
+                continue;
+            }
+            for (int c = 0; c < most; ++c) ctas[c] = (uint32_t)c;
+            std::stable_sort(ctas.begin(), ctas.end(), [&](uint32_t a, uint32_t b) { return load[a] < load[b]; });
+            const double done = load[ctas[size - 1]] + work[q] / size + kFixed;
+            for (uint32_t r = 0; r < size; ++r) {
+                load[ctas[r]] = done;
+                steps[ctas[r]].push_back(SyncStep{q, r, size});
+            }
+            end = std::max(end, done);
+        }
+        if (end >= best_end) continue;
+        best_end = end;
+        t.off.push_back(0);
+        for (int c = 0; c < most; ++c) {
+            t.steps.insert(t.steps.end(), steps[c].begin(), steps[c].end());
+            t.off.push_back((uint32_t)t.steps.size());
+            if (load[c] > 0) t.ctas = c + 1;
+        }
+        best = std::move(t);
+    }
+    return best;
+}
+
 // Shared by abfs_batch_create and abfs_batch_create_counts (sigma == NULL: no counts).
 int batch_create(const abfs_graph_t* g, const uint32_t* sources, uint32_t count,
                  int32_t* const* level, int32_t* const* parent, uint64_t* const* sigma,
@@ -1197,6 +1263,8 @@ int batch_create(const abfs_graph_t* g, const uint32_t* sources, uint32_t count,
     }
     const uint32_t ninst = (uint32_t)inst.size();
     b->ninst = ninst;
+    const int most = sync_applies(g[0]->n, g[0]->nnz, p) ? sync_max_ctas(g[0]->device, g[0]->sms) : 0;
+    const bool sync = most > 0;
     std::vector<Layout> L(ninst);
     std::vector<size_t> base(ninst);
     size_t total = 0;
@@ -1204,7 +1272,7 @@ int batch_create(const abfs_graph_t* g, const uint32_t* sources, uint32_t count,
     for (uint32_t t = 0; t < ninst; ++t) {
         const abfs_graph_s* gt = g[inst[t].gi];
         const uint32_t ms = inst[t].q.size() > 1 ? (uint32_t)inst[t].q.size() : 0u;
-        L[t] = layout_for(gt->n, gt->nnz, p, ms);
+        L[t] = layout_for(gt->n, gt->nnz, p, ms, false, sync);
         base[t] = total;
         total = align_up(total + L[t].total, 256);
         max_n = std::max(max_n, gt->n);
@@ -1275,6 +1343,75 @@ int batch_create(const abfs_graph_t* g, const uint32_t* sources, uint32_t count,
         abfs_batch_destroy(b);
         return cuda_fail(e);
     }
+    SyncBatch sb;
+    std::memset(&sb, 0, sizeof(sb));
+    int sync_grid = 0;
+    if (sync) {
+        // one CTA's time for a search: 0.9 ns an entry and 1.5 ns a vertex; a
+        // multi-source search 2 ns an entry and 0.06 ns more for each source
+        std::vector<double> work(ninst);
+        std::vector<uint32_t> cap(ninst);
+        for (uint32_t t = 0; t < ninst; ++t) {
+            const abfs_graph_s* gt = g[inst[t].gi];
+            const double per = hI[t].ms ? 2e-3 + 6e-5 * hI[t].ms : 0.9e-3;
+            work[t] = per * (double)gt->nnz + 1.5e-3 * gt->n * (hI[t].ms ? 1.0 + hI[t].ms / 8.0 : 1.0);
+            cap[t] = (uint32_t)sync_ctas(gt, most);
+        }
+        const TeamPlan plan = plan_teams(work, cap, most);
+        sync_grid = plan.ctas;
+        size_t o = 0;
+        auto part = [&](size_t bytes) {
+            const size_t at = o;
+            o = align_up(o + bytes, 256);
+            return at;
+        };
+        const size_t at_search = part(sizeof(SyncSearch) * ninst), at_bar = part(256 * (size_t)ninst);
+        const size_t at_off = part(4 * plan.off.size());
+        const size_t at_steps = part(sizeof(SyncStep) * std::max<size_t>(plan.steps.size(), 1));
+        const size_t at_queue = part(4 * std::max<size_t>(plan.queue.size(), 1)), at_next = part(8);
+        static_assert(sizeof(SyncBar) <= 256, "a barrier per 256 bytes");
+        rc = dev_alloc((void**)&b->d_sync, o);
+        if (rc) {
+            abfs_batch_destroy(b);
+            return rc;
+        }
+        // barriers and the queue's counters start at zero
+        std::vector<char> h(o, 0);
+        for (uint32_t t = 0; t < ninst; ++t) {
+            const abfs_graph_s* gt = g[inst[t].gi];
+            SyncBar* bar = reinterpret_cast<SyncBar*>(b->d_sync + at_bar + 256 * (size_t)t);
+            SyncSearch S = make_sync(gt, b->ws + base[t], L[t], bar, hI[t].src, false, p);
+            S.level = hI[t].level;
+            S.parent = hI[t].parent;
+            S.sigma = hI[t].sigma;
+            S.bu_alpha = hI[t].bu_ok ? p.bottom_up_alpha : 0u;
+            S.bu_beta = p.bottom_up_beta;
+            S.ms = hI[t].ms;
+            S.ms_vis = hI[t].ms_vis;
+            S.ms_fr[0] = hI[t].ms_fr[0];
+            S.ms_fr[1] = hI[t].ms_fr[1];
+            S.ms_nx = hI[t].ms_nx;
+            S.ms_src = hI[t].ms_src;
+            S.ms_level = hI[t].ms_level;
+            S.ms_parent = hI[t].ms_parent;
+            std::memcpy(h.data() + at_search + sizeof(SyncSearch) * t, &S, sizeof(S));
+        }
+        std::memcpy(h.data() + at_off, plan.off.data(), 4 * plan.off.size());
+        std::memcpy(h.data() + at_steps, plan.steps.data(), sizeof(SyncStep) * plan.steps.size());
+        std::memcpy(h.data() + at_queue, plan.queue.data(), 4 * plan.queue.size());
+        e = cudaMemcpy(b->d_sync, h.data(), o, cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) {
+            abfs_batch_destroy(b);
+            return cuda_fail(e);
+        }
+        sb.searches = reinterpret_cast<const SyncSearch*>(b->d_sync + at_search);
+        sb.off = reinterpret_cast<const uint32_t*>(b->d_sync + at_off);
+        sb.steps = reinterpret_cast<const SyncStep*>(b->d_sync + at_steps);
+        sb.queue = reinterpret_cast<const uint32_t*>(b->d_sync + at_queue);
+        sb.nqueue = (uint32_t)plan.queue.size();
+        sb.hold_units = test_hold_units();
+        sb.next = reinterpret_cast<uint32_t*>(b->d_sync + at_next);
+    }
     // capture initialisation + the persistent launch in a CUDA graph
     cudaStream_t cap;
     e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
@@ -1296,8 +1433,13 @@ int batch_create(const abfs_graph_t* g, const uint32_t* sources, uint32_t count,
     a.hold_units = test_hold_units();
     e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        cudaError_t e1 = launch_init(a, max_n, cap);
-        cudaError_t e2 = launch_engine(a, grid_size(g[0], p, 0), cap);
+        cudaError_t e1 = cudaSuccess, e2;
+        if (sync) {
+            e2 = launch_sync_batch(sb, sigma != nullptr, sync_grid, cap);
+        } else {
+            e1 = launch_init(a, max_n, cap);
+            e2 = launch_engine(a, grid_size(g[0], p, 0), cap);
+        }
         e = cudaStreamEndCapture(cap, &b->graph);
         if (e == cudaSuccess) e = (e1 != cudaSuccess) ? e1 : e2;
     }
@@ -1660,8 +1802,14 @@ extern "C" int abfs_batch_tune(const abfs_graph_t* g, const uint32_t* sources, u
             }
         }
     }
-    // candidates: granule x narrow bounds (x reduction claims), plus shrink thresholds
+    // candidates: the defaults (level-synchronous engine in submatrix mode), then
+    // granule x narrow bounds (x reduction claims), plus shrink thresholds
     std::vector<abfs_params> cands;
+    {
+        abfs_params p = default_params();
+        p.mode = mode;
+        cands.push_back(p);
+    }
     const uint32_t granules[] = {512, 1024, 4096};
     const uint32_t narrow_e[] = {16384, 65536};
     const uint32_t scans[] = {0, 1u << 22};

@@ -270,12 +270,39 @@ struct SyncSearch {
     uint4* trace;
     uint32_t trace_cap;
     uint32_t bu_alpha, bu_beta;  // hybrid thresholds (0: off or not allowed)
+    // multi-source search (ms > 0, one bit of a 64-bit mask per source; key, bm,
+    // src, level and parent above are unused)
+    uint32_t ms;
+    unsigned long long* ms_vis;       // sources that have reached each vertex
+    unsigned long long* ms_fr[2];     // frontier masks, by level parity
+    unsigned long long* ms_nx;        // sources that reach each vertex next (pushed levels)
+    const uint32_t* ms_src;
+    int32_t* const* ms_level;
+    int32_t* const* ms_parent;
     uint32_t hold_units;         // test control: arrivals that never come
     // a level of this many entries is wide; the same for frontiers whose items
     // average hub_avg entries or more
     unsigned long long wide_min, wide_hub;
     uint32_t hub_avg;
     unsigned long long timeout_ns;
+};
+
+// A batch on the level-synchronous engine.  The searches that get a team of
+// several CTAs are fixed when the plan is made: CTA c runs steps
+// [off[c], off[c + 1]) in order, and every CTA meets the searches in the same
+// order, so a team's barrier only waits for CTAs that are on their way to it.
+// The other searches run on one CTA each, taken from a queue, largest first.
+struct SyncStep {
+    uint32_t search, rank, size;
+};
+struct SyncBatch {
+    const SyncSearch* searches;
+    const uint32_t* off;
+    const SyncStep* steps;
+    const uint32_t* queue;    // searches that run on one CTA
+    uint32_t nqueue;
+    uint32_t hold_units;
+    uint32_t* next;           // [0] taken from the queue, [1] CTAs that have left
 };
 
 // Cycle accounting of the engine's CTAs (profiling runs only).
@@ -367,5 +394,6 @@ cudaError_t engine_max_clusters(uint32_t mode, uint32_t cluster, int* clusters);
 // Level-synchronous engine (sync_engine.cu).
 int sync_max_ctas(int device, int sms);
 cudaError_t launch_sync(const SyncSearch& S, int ctas, cudaStream_t s);
+cudaError_t launch_sync_batch(const SyncBatch& B, bool sigma, int ctas, cudaStream_t s);
 
 }  // namespace abfs

@@ -70,6 +70,11 @@ struct SyncSmem {
     unsigned long long nf, entries, seen;
     unsigned long long st_read, st_unmasked, st_verts, st_ent;
     uint32_t levels;
+    // multi-source searches: columns left to the whole CTA, and the masks its
+    // warps found in a round
+    uint32_t nlong;
+    unsigned long long open;                  // entries of vertices some source has not reached
+    unsigned long long wm[2][kSyncWarps];
     uint32_t step;                            // barriers passed
     unsigned long long word[2], aux[2];       // the barrier words as last seen
 };
@@ -102,6 +107,9 @@ __device__ __forceinline__ void red_add64(unsigned long long* p, unsigned long l
 // is compiled to an atomic that returns.)
 __device__ __forceinline__ void red_min32(uint32_t* p, uint32_t v) {
     asm volatile("red.relaxed.gpu.global.min.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ void red_or64(unsigned long long* p, unsigned long long v) {
+    asm volatile("red.relaxed.gpu.global.or.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 __device__ __forceinline__ void red_add_release64(unsigned long long* p, unsigned long long v) {
     asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");

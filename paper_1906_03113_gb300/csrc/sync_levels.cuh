@@ -191,7 +191,14 @@ __device__ __forceinline__ uint32_t word_mask(const SyncSearch& S, uint32_t w) {
 // 32 items at a time and walks their chunks of four row indices, one 16-byte
 // load per lane and step, the next step's loads issued before this step's
 // tests; there is no barrier inside.  Whole CTA.
-template <bool SIG>
+enum WideKind : int {
+    kWidePlain = 0,
+    kWideCounts = 1,  // and shortest-path counts
+    kWideMulti = 2,   // multi-source search: every row gets the frontier bits of the column
+                      // that it lacks, in the next-bit masks
+};
+
+template <int KIND>
 __device__ __noinline__ void wide_expand(SyncSmem& sm, const SyncSearch& S, const Team& T, uint32_t k,
                                          unsigned long long items) {
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -276,6 +283,20 @@ __device__ __noinline__ void wide_expand(SyncSmem& sm, const SyncSearch& S, cons
             uint32_t ok2 = 0, jj2 = 0;
             if (g + 32 < total) load(g + 32, rr2, ok2, jj2);
             const uint32_t r[kChunk] = {rr.x, rr.y, rr.z, rr.w};
+            if (KIND == kWideMulti) {
+                const unsigned long long f = ok ? ld_l2(S.ms_fr[p] + jj) : 0ull;
+                unsigned long long vis[kChunk];
+#pragma unroll
+                for (uint32_t q = 0; q < kChunk; ++q)
+                    vis[q] = (ok >> q) & 1u ? ld_l2(S.ms_vis + r[q]) : ~0ull;
+#pragma unroll
+                for (uint32_t q = 0; q < kChunk; ++q)
+                    if (f & ~vis[q]) red_or64(S.ms_nx + r[q], f & ~vis[q]);
+                rr = rr2;
+                ok = ok2;
+                jj = jj2;
+                continue;
+            }
             uint32_t w[kChunk];
 #pragma unroll
             for (uint32_t q = 0; q < kChunk; ++q)
@@ -285,7 +306,7 @@ __device__ __noinline__ void wide_expand(SyncSmem& sm, const SyncSearch& S, cons
                 if (!((w[q] >> (r[q] & 31)) & 1u)) {
                     ++t.unmasked;
                     red_min32(klo + 2ull * r[q], jj);
-                    if (SIG) red_add64(S.sigma + r[q], ld_l2(S.sigma + jj));
+                    if (KIND == kWideCounts) red_add64(S.sigma + r[q], ld_l2(S.sigma + jj));
                 }
             }
             rr = rr2;
@@ -332,11 +353,12 @@ __device__ __noinline__ void sync_bitmaps(const SyncSearch& S, const Team& T, ui
     }
 }
 
-// The frontier list of level k + 1.  FROM_KEYS: after a wide level, its new
+// The frontier list of level k + 1.  kFromKeys: after a wide level, its new
 // vertices are those outside the bitmap whose key has a parent; they get their
 // level, join the bitmap (each word has one writer) and make up the frontier
-// bitmap of level k + 1.  Otherwise that bitmap is there already (after a
-// bottom-up level, which counted its vertices).
+// bitmap of level k + 1.  kFromBits: that bitmap is there already (after a
+// bottom-up level, which counted its vertices).  kFromMasks: the vertices with
+// frontier bits of a multi-source search.
 //
 // Two passes over a warp's words, so that the CTA meets once and reserves its
 // items with one atomic: the first finds the new vertices and counts their
@@ -346,8 +368,11 @@ __device__ __noinline__ void sync_bitmaps(const SyncSearch& S, const Team& T, ui
 // four million, most of it waiting.  Whole CTA.
 constexpr uint32_t kExtractWords = 8;
 
-template <bool FROM_KEYS>
+enum ExtractKind : int { kFromKeys, kFromBits, kFromMasks };
+
+template <int KIND>
 __device__ __noinline__ void sync_extract(SyncSmem& sm, const SyncSearch& S, const Team& T, uint32_t k) {
+    constexpr bool FROM_KEYS = KIND == kFromKeys, MASKS = KIND == kFromMasks;
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr uint32_t Q = kExtractWords;
     const uint32_t pn = (k + 1) & 1;
@@ -362,6 +387,8 @@ __device__ __noinline__ void sync_extract(SyncSmem& sm, const SyncSearch& S, con
             if (FROM_KEYS) {
                 seen = ld_l2(S.bm + wb + lane);
                 word = ~seen & word_mask(S, wb + lane);
+            } else if (MASKS) {
+                word = word_mask(S, wb + lane);
             } else {
                 word = ld_l2(S.fbm[pn] + wb + lane);
             }
@@ -373,10 +400,11 @@ __device__ __noinline__ void sync_extract(SyncSmem& sm, const SyncSearch& S, con
             const uint32_t c = __shfl_sync(0xFFFFFFFFu, word, q);
             fresh[q] = (c >> lane) & 1u;
             if (FROM_KEYS && fresh[q]) fresh[q] = (uint32_t)ld_l2(S.key + v0 + 32 * q) != kUnset;
+            if (MASKS && fresh[q]) fresh[q] = ld_l2(S.ms_fr[pn] + v0 + 32 * q) != 0ull;
         }
 #pragma unroll
         for (uint32_t q = 0; q < Q; ++q) {
-            if (FROM_KEYS) {
+            if (FROM_KEYS || MASKS) {
                 const uint32_t bits = __ballot_sync(0xFFFFFFFFu, fresh[q]);
                 if (lane == q) add = bits;
             }
@@ -389,10 +417,8 @@ __device__ __noinline__ void sync_extract(SyncSmem& sm, const SyncSearch& S, con
                 mine += items_of(cb, len);
             }
         }
-        if (FROM_KEYS && own) {
-            if (add) S.bm[wb + lane] = seen | add;
-            S.fbm[pn][wb + lane] = add;
-        }
+        if (FROM_KEYS && own && add) S.bm[wb + lane] = seen | add;
+        if ((FROM_KEYS || MASKS) && own) S.fbm[pn][wb + lane] = add;
     }
     const uint32_t wt = __reduce_add_sync(0xFFFFFFFFu, mine);
     if (lane == 0) sm.wsum[warp] = wt;
@@ -408,7 +434,7 @@ __device__ __noinline__ void sync_extract(SyncSmem& sm, const SyncSearch& S, con
         base = __shfl_sync(0xFFFFFFFFu, base, 31);
         sm.wpre[lane] = base + incl - x;
     }
-    if (FROM_KEYS) {
+    if (KIND != kFromBits) {
         verts = __reduce_add_sync(0xFFFFFFFFu, verts);
         entries = __reduce_add_sync(0xFFFFFFFFu, entries);
         if (lane == 0 && verts) {

@@ -246,6 +246,19 @@ __device__ __forceinline__ uint32_t wide_next(SyncSmem& sm, const SyncSearch& S,
     return kActSlice;
 }
 
+// Thread 0 of a CTA that is done with a search: the last one to leave sets the
+// status and clears the barrier's words for the next search.
+__device__ __forceinline__ void sync_leave(const SyncSearch& S, const Team& T) {
+    __threadfence();
+    if (atomicInc(&S.bar->exited, T.size - 1) != T.size - 1) return;
+    __threadfence();
+    for (int b = 0; b < 2; ++b) {
+        S.bar->word[b] = S.bar->aux[b] = 0;
+        S.bar->lcnt[b] = 0;
+    }
+    S.ctl->status = ld_relaxed(&S.ctl->err) ? kFailed : kDone;
+}
+
 // Runs one search on this team.  The outputs and the control block are written
 // when it returns (to be read after the kernel).
 //
@@ -323,13 +336,13 @@ __device__ __forceinline__ void sync_search(SyncSmem& sm, const SyncSearch& S, c
             if (up) {
                 sync_bottom_up(sm, S, T, k);
             } else {
-                wide_expand<SIG>(sm, S, T, k, sm.items);
+                wide_expand<SIG ? kWideCounts : kWidePlain>(sm, S, T, k, sm.items);
                 if (!team_sync(sm, S, T)) {
                     act = kActFailed;
                     break;
                 }
                 sync_trace(S, T, kPhExtract, k, 0u, 0u, 0u, 0u);
-                sync_extract<true>(sm, S, T, k);
+                sync_extract<kFromKeys>(sm, S, T, k);
             }
             __syncthreads();
             if (lead) {
@@ -350,7 +363,7 @@ __device__ __forceinline__ void sync_search(SyncSmem& sm, const SyncSearch& S, c
             act = sm.act;
             if (up && act == kActWide) {
                 // back to top-down levels: the list of the frontier bitmap
-                sync_extract<false>(sm, S, T, k - 1);
+                sync_extract<kFromBits>(sm, S, T, k - 1);
                 __syncthreads();
                 const uint32_t c = sm.app[0][0];
                 if (!team_sync(sm, S, T, c)) act = kActFailed;
@@ -374,17 +387,7 @@ __device__ __forceinline__ void sync_search(SyncSmem& sm, const SyncSearch& S, c
         if (sm.st_verts) atomicAdd(&c->reached, (uint32_t)sm.st_verts);
         atomicMax(&c->levels, sm.levels);
         if (T.rank == 0 && wide_levels) atomicAdd(&c->wide_levels, wide_levels);
-        // the last CTA to leave sets the status and clears the barrier's words
-        // for the next search
-        __threadfence();
-        if (atomicInc(&S.bar->exited, T.size - 1) == T.size - 1) {
-            __threadfence();
-            for (int b = 0; b < 2; ++b) {
-                S.bar->word[b] = S.bar->aux[b] = 0;
-                S.bar->lcnt[b] = 0;
-            }
-            c->status = ld_relaxed(&c->err) ? kFailed : kDone;
-        }
+        sync_leave(S, T);
     }
 }
 

@@ -76,3 +76,68 @@ def test_default_engine_at_its_edges(name, shift):
     assert np.array_equal(sig.cpu().numpy().view(np.uint64), oracle.path_counts(g, s)), name
     assert st["entries_read"] == st["nnz_reached"]
     G.destroy()
+
+
+def test_batch_teams_and_queue():
+    """One launch in which large searches run on teams of several CTAs and small
+    ones are taken from the queue, replayed; then the same with path counts."""
+    hosts = [synth.rmat(17, 16.0, seed=21), synth.er(60000, 9.0, seed=22), synth.grid(70, 53),
+             synth.from_arcs(1, [], [], directed=False), synth.rgg_knn(5000, 4, seed=23),
+             synth.rmat(15, 8.0, seed=24)] + [synth.er(900 + 31 * i, 5.0, seed=30 + i) for i in range(200)]
+    dev = [abfs.graph_create(g.colptr, g.rowidx, directed=g.directed) for g in hosts]
+    srcs = [int(np.argmax(g.degrees())) if g.nnz else 0 for g in hosts]
+    want = [oracle.bfs(g, s) for g, s in zip(hosts, srcs)]
+    plan = abfs.BatchPlan(dev, srcs)
+    for rep in range(3):
+        for t in plan.levels + plan.parents:
+            t.fill_(9)
+        plan.launch()
+        assert plan.status() == [0] * len(dev)
+        for i, (lo, po) in enumerate(want):
+            assert np.array_equal(plan.levels[i].cpu().numpy(), lo), (rep, i)
+            assert np.array_equal(plan.parents[i].cpu().numpy(), po), (rep, i)
+    plan.destroy()
+    plan = abfs.BatchPlan(dev[:12], srcs[:12], counts=True)
+    plan.launch()
+    assert plan.status() == [0] * 12
+    for i in range(12):
+        assert np.array_equal(plan.levels[i].cpu().numpy(), want[i][0])
+        assert np.array_equal(plan.sigmas[i].cpu().numpy().view(np.uint64), oracle.path_counts(hosts[i], srcs[i]))
+    plan.destroy()
+    for G in dev:
+        G.destroy()
+
+
+@pytest.mark.parametrize("leaves,count", [(2047, 5), (2049, 64), (9000, 63), (20000, 64)])
+def test_multi_source_long_columns(leaves, count):
+    """A hub whose column is scanned by a whole CTA: sources are leaves on both
+    sides of the lane, warp and round boundaries of that scan (their bits reach
+    the hub from exactly one entry each), and the other way round."""
+    g = synth.from_arcs(leaves + 1, [0] * leaves, list(range(1, leaves + 1)), directed=False)
+    edge = [1, 16, 17, 32, 33, 128, 129, 144, 145, 2047, 4096, 4097, 4112, 4113, 8192, 8193, leaves]
+    srcs = [s for s in edge if s <= leaves][:count - 1]
+    rng = np.random.default_rng(leaves)
+    srcs += [int(x) for x in rng.integers(leaves + 1, size=count - len(srcs))]
+    G = abfs.graph_create(g.colptr, g.rowidx, directed=False)
+    levels, parents, st = abfs.run_batch([G] * count, srcs)
+    torch.cuda.synchronize()
+    assert all(x == 0 for x in st)
+    for s, L, P in zip(srcs, levels, parents):
+        lo, po = oracle.bfs(g, s)
+        assert np.array_equal(L.cpu().numpy(), lo) and np.array_equal(P.cpu().numpy(), po), s
+    G.destroy()
+
+
+def test_multi_source_on_a_skewed_graph():
+    """64 sources on a graph with hubs and thousands of unreached vertices:
+    pushed and pulled levels."""
+    g = synth.rmat(16, 16.0, seed=31)
+    G = abfs.graph_create(g.colptr, g.rowidx, directed=False)
+    srcs = [int(x) for x in synth.sources_with_degree(g, 64, seed=3)]
+    levels, parents, st = abfs.run_batch([G] * 64, srcs)
+    torch.cuda.synchronize()
+    assert all(x == 0 for x in st)
+    for s, L, P in zip(srcs, levels, parents):
+        lo, po = oracle.bfs(g, s)
+        assert np.array_equal(L.cpu().numpy(), lo) and np.array_equal(P.cpu().numpy(), po), s
+    G.destroy()
