@@ -74,12 +74,13 @@ typedef enum {
 /* Tunable launch parameters.  abfs_default_params() fills sound values;
  * abfs_tune() measures and picks them for a graph.
  *
- * Two engines run single searches, with the same results.  With the default
- * values of the scheduling knobs (tile, unit_entries, narrow_*, ctas_per_sm,
- * claim_scan, cluster_*), submatrix searches without a physical shrink run on
- * the level-synchronous engine, which takes one search at a time and none of
- * those knobs.  A search that sets any of them, the comparator, shrinks,
- * abfs_run_static and serving run on the unit scheduler, whose knobs they
+ * Two engines run searches, with the same results.  With the default values
+ * of the scheduling knobs (tile, unit_entries, narrow_*, ctas_per_sm,
+ * claim_scan, cluster_*), submatrix searches without a physical shrink --
+ * single ones, batches and serving -- run on the level-synchronous engine,
+ * where a team of CTAs runs one search at a time and none of those knobs
+ * means anything.  A search that sets any of them, the comparator, shrinks and
+ * abfs_run_static run on the unit scheduler, whose knobs they
  * are. */
 typedef struct {
     uint32_t mode;            /* ABFS_MODE_SUBMATRIX or ABFS_MODE_PLAIN */
@@ -308,8 +309,9 @@ int abfs_run_trace(abfs_graph_t g, uint32_t source, int32_t* level, int32_t* par
 
 /*
  * Batched search: `count` independent searches (graph g[i], source
- * sources[i]) in ONE persistent launch with per-instance frontier queues;
- * each CTA takes work units from any instance that has them.  level[i] and
+ * sources[i]) in ONE persistent launch with per-instance frontier queues:
+ * teams of CTAs for the large searches, one CTA each for the others (with
+ * non-default scheduling knobs, work units that any CTA takes).  level[i] and
  * parent[i] are caller-owned DEVICE buffers of g[i]'s n int32 each.
  * status_per_query (host, count entries, may be NULL) receives each search's
  * abfs_status.  Synchronises `stream`.  Results equal abfs_run's, bit for
@@ -378,8 +380,8 @@ int abfs_batch_tune(const abfs_graph_t* g, const uint32_t* sources, uint32_t cou
  * admission thread moves them into free device slots as soon as a slot and
  * enough workspace memory (abfs_graph_footprint of the query's graph, carved
  * from a memory budget) are free, while other queries are running; their
- * work overlaps on the device in one persistent launch, which any CTA serves
- * unit by unit.  The launch ends after idle_exit_ms without work and is
+ * work overlaps on the device in one persistent launch, whose CTAs form a team
+ * for each query as they come free.  The launch ends after idle_exit_ms without work and is
  * relaunched on demand.  Each query's result equals abfs_run's, bit for bit.
  * The paper has no counterpart (it evaluates single searches).
  */

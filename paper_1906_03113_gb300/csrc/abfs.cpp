@@ -217,6 +217,19 @@ bool sync_applies(uint32_t n, uint64_t nnz, const abfs_params& p) {
            p.cluster_max == d.cluster_max && p.cluster_edges == d.cluster_edges;
 }
 
+// One CTA's time for a search: 0.9 ns an entry and 1.5 ns a vertex; a
+// multi-source search (ms sources) 2 ns an entry and 0.06 ns more per source.
+double sync_work_us(uint32_t n, uint64_t nnz, uint32_t ms) {
+    return (ms ? 2e-3 + 6e-5 * ms : 0.9e-3) * (double)nnz + 1.5e-3 * n * (ms ? 1.0 + ms / 8.0 : 1.0);
+}
+
+// The largest useful team of a search: a few thousand entries per CTA.  Up to
+// 16 384 entries one CTA, without barriers between CTAs, is fastest.
+int sync_team_cap(uint64_t nnz, int most) {
+    const uint64_t want = nnz <= 16384 ? 1 : (nnz + 4095) / 4096;
+    return (int)std::min<uint64_t>((uint64_t)most, std::max<uint64_t>(want, 1));
+}
+
 // ---------------------------------------------------------------------------
 // per-search workspace layout
 // ---------------------------------------------------------------------------
@@ -574,12 +587,6 @@ SyncSearch make_sync(const abfs_graph_s* g, char* base, const Layout& L, SyncBar
     return S;
 }
 
-// CTAs of a search's team: enough that each has a few thousand entries.
-int sync_ctas(const abfs_graph_s* g, int most) {
-    const uint64_t want = g->nnz <= 16384 ? 1 : (g->nnz + 4095) / 4096;
-    return (int)std::min<uint64_t>((uint64_t)most, std::max<uint64_t>(want, 1));
-}
-
 // Enqueues one search into g's workspace; caller holds g->mu.
 int enqueue_single(abfs_graph_s* g, uint32_t source, int32_t* level, int32_t* parent,
                    cudaStream_t s, const abfs_params& p, uint4* trace = nullptr,
@@ -606,7 +613,7 @@ int enqueue_single(abfs_graph_s* g, uint32_t source, int32_t* level, int32_t* pa
         S.trace_cap = trace_cap;
         S.bu_alpha = bu_ok ? p.bottom_up_alpha : 0u;
         S.bu_beta = p.bottom_up_beta;
-        CK(launch_sync(S, sync_ctas(g, most), s));
+        CK(launch_sync(S, sync_team_cap(g->nnz, most), s));
         CK(cudaEventRecord(g->last_use, s));
         g->used = true;
         return ABFS_OK;
@@ -655,6 +662,15 @@ int finish_stats(abfs_graph_s* g, cudaStream_t s, abfs_stats* stats) {
 }  // namespace
 
 namespace abfs {
+SyncSearch serve_search(abfs_graph_t g, char* base, const Layout& L, SyncBar* bar, InstCtl* ctl,
+                        uint32_t source, int32_t* level, int32_t* parent, const abfs_params& p) {
+    SyncSearch S = make_sync(g, base, L, bar, source, false, p);
+    S.level = level;
+    S.parent = reinterpret_cast<uint32_t*>(parent);
+    S.ctl = ctl;
+    S.hold_units = 0;
+    return S;
+}
 int graph_arrays(abfs_graph_t g, const uint32_t** colptr, const uint32_t** rowidx, uint32_t* n,
                  uint64_t* nnz, int* device, int* sms) {
     if (!g) return ABFS_ERR_INVALID_ARG;
@@ -1347,15 +1363,12 @@ int batch_create(const abfs_graph_t* g, const uint32_t* sources, uint32_t count,
     std::memset(&sb, 0, sizeof(sb));
     int sync_grid = 0;
     if (sync) {
-        // one CTA's time for a search: 0.9 ns an entry and 1.5 ns a vertex; a
-        // multi-source search 2 ns an entry and 0.06 ns more for each source
         std::vector<double> work(ninst);
         std::vector<uint32_t> cap(ninst);
         for (uint32_t t = 0; t < ninst; ++t) {
             const abfs_graph_s* gt = g[inst[t].gi];
-            const double per = hI[t].ms ? 2e-3 + 6e-5 * hI[t].ms : 0.9e-3;
-            work[t] = per * (double)gt->nnz + 1.5e-3 * gt->n * (hI[t].ms ? 1.0 + hI[t].ms / 8.0 : 1.0);
-            cap[t] = (uint32_t)sync_ctas(gt, most);
+            work[t] = sync_work_us(gt->n, gt->nnz, hI[t].ms);
+            cap[t] = (uint32_t)sync_team_cap(gt->nnz, most);
         }
         const TeamPlan plan = plan_teams(work, cap, most);
         sync_grid = plan.ctas;

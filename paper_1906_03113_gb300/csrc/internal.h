@@ -102,6 +102,7 @@ enum InstStatus : uint32_t { kIdle = 0, kRunning = 1, kDone = 2, kFailed = 3 };
 
 // Serving slot states (device array, one word per slot).
 enum SlotState : uint32_t { kSlotFree = 0, kSlotSubmitted = 1, kSlotRunning = 2 };
+constexpr uint32_t kSlotWorkShift = 8;  // (level-synchronous engine)
 
 // A block of the frontier: nv consecutive vertices at fq[vb..], whose column
 // entries occupy [eb, eb + sum of their weights) of the level's entry space.
@@ -305,6 +306,26 @@ struct SyncBatch {
     uint32_t* next;           // [0] taken from the queue, [1] CTAs that have left
 };
 
+// Serving on the level-synchronous engine: a query in a slot of the device's
+// table.
+struct SyncSlot {
+    SyncSearch search;
+    unsigned long long ticket;
+    unsigned long long* notify;  // host-mapped word that receives ticket << 8 | status
+    uint32_t cap;                // largest team it can use
+};
+struct SyncServe {
+    const SyncSlot* slots;
+    uint32_t* state;             // per slot: SlotState in 8 bits, above it the query's work in units
+    uint32_t* claim;             // 1 while a CTA claims a query and opens its team
+    // per slot, the team being formed: [sequence : 32][open : 1][wanted : 8][joined : 8]
+    unsigned long long* join;
+    const uint32_t* stop_flag;
+    unsigned long long* heartbeat;
+    uint32_t nslots;
+    unsigned long long idle_exit_ns;
+};
+
 // Cycle accounting of the engine's CTAs (profiling runs only).
 enum ProfSlot : int {
     kProfIdle = 0,     // no unit available
@@ -360,6 +381,12 @@ bool sync_applies(uint32_t n, uint64_t nnz, const abfs_params& p);
 Inst make_inst_raw(const uint32_t* colptr, const uint32_t* rowidx, uint32_t n, char* base,
                    const Layout& L, uint32_t src, int32_t* level, int32_t* parent);
 int grid_for(int sms, const abfs_params& p);
+// The search of a query served in slot buffers (base, bar, ctl), top-down; the
+// microseconds it takes on one CTA; the largest team it can use.
+SyncSearch serve_search(abfs_graph_t g, char* base, const Layout& L, SyncBar* bar, InstCtl* ctl,
+                        uint32_t source, int32_t* level, int32_t* parent, const abfs_params& p);
+double sync_work_us(uint32_t n, uint64_t nnz, uint32_t ms);
+int sync_team_cap(uint64_t nnz, int most);
 int graph_arrays(abfs_graph_t g, const uint32_t** colptr, const uint32_t** rowidx, uint32_t* n,
                  uint64_t* nnz, int* device, int* sms);
 
@@ -394,6 +421,7 @@ cudaError_t engine_max_clusters(uint32_t mode, uint32_t cluster, int* clusters);
 // Level-synchronous engine (sync_engine.cu).
 int sync_max_ctas(int device, int sms);
 cudaError_t launch_sync(const SyncSearch& S, int ctas, cudaStream_t s);
+cudaError_t launch_sync_serve(const SyncServe& A, int ctas, cudaStream_t s);
 cudaError_t launch_sync_batch(const SyncBatch& B, bool sigma, int ctas, cudaStream_t s);
 
 }  // namespace abfs

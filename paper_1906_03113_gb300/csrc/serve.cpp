@@ -96,6 +96,14 @@ struct abfs_server_s {
     int device = 0, sms = 0;
     // device
     Inst* d_slots = nullptr;
+    // queries on the level-synchronous engine (cfg.params permitting): their
+    // slots, barriers (256 bytes each) and teams being formed
+    int ctas = 0;                 // CTAs of its launch, 0: the unit scheduler serves
+    SyncSlot* d_sync = nullptr;
+    char* d_bars = nullptr;
+    unsigned long long* d_join = nullptr;
+    SyncSlot* h_sync = nullptr;
+    std::vector<uint32_t> work;   // per graph: eighths of a microsecond on one CTA
     InstCtl* d_ctl = nullptr;
     uint32_t* d_state = nullptr;
     uint32_t* d_stop = nullptr;
@@ -106,7 +114,7 @@ struct abfs_server_s {
     unsigned long long* h_notify = nullptr;
     unsigned long long* d_notify = nullptr;
     Inst* h_stage = nullptr;
-    uint32_t* h_words = nullptr;  // [0] = kSlotSubmitted, [1] = 1 (stop)
+    uint32_t* h_words = nullptr;  // [1] = 1 (stop), [2 + i]: slot i's state when submitted
     cudaStream_t kstream = nullptr, cstream = nullptr;
     // bookkeeping
     std::mutex mu;
@@ -135,6 +143,10 @@ void release_server(abfs_server_s* S) {
     cudaFree(S->d_done);
     cudaFree(S->d_beat);
     cudaFree(S->d_arena);
+    cudaFree(S->d_sync);
+    cudaFree(S->d_bars);
+    cudaFree(S->d_join);
+    if (S->h_sync) cudaFreeHost(S->h_sync);
     if (S->h_notify) cudaFreeHost(S->h_notify);
     if (S->h_stage) cudaFreeHost(S->h_stage);
     if (S->h_words) cudaFreeHost(S->h_words);
@@ -154,6 +166,51 @@ EngineArgs serve_args(abfs_server_s* S) {
     a.idle_exit_ns = (unsigned long long)S->cfg.idle_exit_ms * 1000000ull;
     a.p = engine_params(S->cfg.params);
     return a;
+}
+
+// Device launch that serves the slots.
+cudaError_t serve_launch(abfs_server_s* S) {
+    if (!S->ctas) return launch_engine(serve_args(S), grid_for(S->sms, S->cfg.params), S->kstream);
+    SyncServe A;
+    A.slots = S->d_sync;
+    A.state = S->d_state;
+    A.claim = S->d_done;
+    A.join = S->d_join;
+    A.stop_flag = S->d_stop;
+    A.heartbeat = S->d_beat;
+    A.nslots = S->cfg.max_slots;
+    A.idle_exit_ns = (unsigned long long)S->cfg.idle_exit_ms * 1000000ull;
+    return launch_sync_serve(A, S->ctas, S->kstream);
+}
+
+// Writes request rq, admitted to slot i with the workspace at `off`, into the
+// slot's descriptor (copied on cstream).  Caller holds S->mu.
+cudaError_t serve_describe(abfs_server_s* S, uint32_t i, const Request& rq, size_t off) {
+    if (S->ctas) {
+        SyncSlot& q = S->h_sync[i];
+        q.search = serve_search(S->graphs[rq.g], S->d_arena + off, S->layouts[rq.g],
+                                reinterpret_cast<SyncBar*>(S->d_bars + 256 * (size_t)i), S->d_ctl + i, rq.src,
+                                rq.level, rq.parent, S->cfg.params);
+        q.ticket = rq.ticket;
+        q.notify = S->d_notify + i;
+        q.cap = (uint32_t)sync_team_cap(q.search.nnz, S->ctas);
+        S->h_words[2 + i] = kSlotSubmitted | S->work[rq.g] << kSlotWorkShift;
+        return cudaMemcpyAsync(S->d_sync + i, &q, sizeof(SyncSlot), cudaMemcpyHostToDevice, S->cstream);
+    }
+    const uint32_t* cp;
+    const uint32_t* ri;
+    uint32_t n;
+    uint64_t nnz;
+    int dev, sms;
+    graph_arrays(S->graphs[rq.g], &cp, &ri, &n, &nnz, &dev, &sms);
+    Inst I = make_inst_raw(cp, ri, n, S->d_arena + off, S->layouts[rq.g], rq.src, rq.level, rq.parent);
+    I.ctl = S->d_ctl + i;  // fixed per slot, so a scan of slot i always reads its own block
+    I.slot = i;
+    I.ticket = rq.ticket;
+    I.notify = S->d_notify + i;
+    S->h_words[2 + i] = kSlotSubmitted;
+    S->h_stage[i] = I;
+    return cudaMemcpyAsync(S->d_slots + i, S->h_stage + i, sizeof(Inst), cudaMemcpyHostToDevice, S->cstream);
 }
 
 // The admission thread.
@@ -194,24 +251,11 @@ void serve_loop(abfs_server_s* S) {
                 const Layout& L = S->layouts[rq.g];
                 size_t off = 0;
                 if (!S->arena.alloc(L.total, &off)) break;
-                const uint32_t* cp;
-                const uint32_t* ri;
-                uint32_t n;
-                uint64_t nnz;
-                int dev, sms;
-                graph_arrays(S->graphs[rq.g], &cp, &ri, &n, &nnz, &dev, &sms);
-                Inst I = make_inst_raw(cp, ri, n, S->d_arena + off, L, rq.src, rq.level, rq.parent);
-                I.ctl = S->d_ctl + i;  // fixed per slot, so a scan of slot i always reads its own block
-                I.slot = i;
-                I.ticket = rq.ticket;
-                I.notify = S->d_notify + i;
-                S->h_stage[i] = I;
                 // the descriptor first, then the state word: the device reads the
                 // state, then (after an acquire) the descriptor
-                cudaError_t e = cudaMemcpyAsync(S->d_slots + i, S->h_stage + i, sizeof(Inst),
-                                                cudaMemcpyHostToDevice, S->cstream);
+                cudaError_t e = serve_describe(S, i, rq, off);
                 if (e == cudaSuccess)
-                    e = cudaMemcpyAsync(S->d_state + i, S->h_words, 4, cudaMemcpyHostToDevice,
+                    e = cudaMemcpyAsync(S->d_state + i, S->h_words + 2 + i, 4, cudaMemcpyHostToDevice,
                                         S->cstream);
                 if (e != cudaSuccess) {
                     S->fatal = ABFS_ERR_CUDA;
@@ -233,8 +277,7 @@ void serve_loop(abfs_server_s* S) {
             const bool running = launched && cudaStreamQuery(S->kstream) == cudaErrorNotReady;
             if (!running) {
                 cudaGetLastError();
-                const EngineArgs a = serve_args(S);
-                if (launch_engine(a, grid_for(S->sms, S->cfg.params), S->kstream) != cudaSuccess) {
+                if (serve_launch(S) != cudaSuccess) {
                     S->fatal = ABFS_ERR_CUDA;
                 } else {
                     launched = true;
@@ -301,7 +344,9 @@ extern "C" int abfs_serve_start(const abfs_graph_t* g, uint32_t ngraphs, const a
             delete S;
             return ABFS_ERR_INVALID_ARG;
         }
-        S->layouts.push_back(layout_for(n, nnz, c.params));
+        if (i == 0 && sync_applies(n, nnz, c.params)) S->ctas = sync_max_ctas(dev, sms);
+        S->layouts.push_back(layout_for(n, nnz, c.params, 0, false, S->ctas > 0));
+        S->work.push_back((uint32_t)std::min(8.0 * sync_work_us(n, nnz, 0) + 1.0, 16777215.0));
         largest = std::max(largest, S->layouts.back().total);
     }
     if (largest + 256 > c.memory_budget) {
@@ -322,13 +367,20 @@ extern "C" int abfs_serve_start(const abfs_graph_t* g, uint32_t ngraphs, const a
     ck(cudaMalloc((void**)&S->d_arena, c.memory_budget));
     ck(cudaHostAlloc((void**)&S->h_notify, 8 * ns, cudaHostAllocMapped));
     ck(cudaHostAlloc((void**)&S->h_stage, sizeof(Inst) * ns, cudaHostAllocDefault));
-    ck(cudaHostAlloc((void**)&S->h_words, 64, cudaHostAllocDefault));
+    ck(cudaHostAlloc((void**)&S->h_words, 4 * (size_t)ns + 64, cudaHostAllocDefault));
+    if (S->ctas) {
+        ck(cudaMalloc((void**)&S->d_sync, sizeof(SyncSlot) * ns));
+        ck(cudaMalloc((void**)&S->d_bars, 256 * (size_t)ns));
+        ck(cudaMalloc((void**)&S->d_join, 8 * (size_t)ns));
+        ck(cudaHostAlloc((void**)&S->h_sync, sizeof(SyncSlot) * ns, cudaHostAllocDefault));
+        if (e == cudaSuccess) ck(cudaMemset(S->d_bars, 0, 256 * (size_t)ns));
+        if (e == cudaSuccess) ck(cudaMemset(S->d_join, 0, 8 * (size_t)ns));
+    }
     if (e == cudaSuccess) ck(cudaHostGetDevicePointer((void**)&S->d_notify, S->h_notify, 0));
     ck(cudaStreamCreateWithFlags(&S->kstream, cudaStreamNonBlocking));
     ck(cudaStreamCreateWithFlags(&S->cstream, cudaStreamNonBlocking));
     if (e == cudaSuccess) {
         std::memset(S->h_notify, 0, 8 * ns);
-        S->h_words[0] = kSlotSubmitted;
         S->h_words[1] = 1u;
         ck(cudaMemset(S->d_slots, 0, sizeof(Inst) * ns));
         ck(cudaMemset(S->d_ctl, 0, sizeof(InstCtl) * ns));

@@ -74,6 +74,190 @@ __global__ void __launch_bounds__(kSyncThreads, 1) sync_batch_kernel(const __gri
     }
 }
 
+// ---------------------------------------------------------------------------
+// serving: a long-lived launch over a table of slots
+// ---------------------------------------------------------------------------
+// A CTA without a search first joins a team that is being formed, else claims a
+// newly submitted query.  The query gets a share of the CTAs in proportion to
+// its part of the work at hand (all of them when it is alone): the claiming CTA
+// opens a team of that size, waits for others to come free, a quarter of the
+// time the query then takes and at most kJoinWaitNs, closes the team and runs
+// the query with whoever came.  Only CTAs that have joined are waited for
+// afterwards, so the launch needs no co-residency of all its CTAs, and a CTA
+// that idles out is never missed.  Claims are made one at a time, so that CTAs
+// that come free together do not each open a team that nobody is left to join.
+// (Counting on free CTAs alone left large queries on one CTA whenever the
+// launch was busy: 256 queries on 16 graphs 3.6 -> 6.7 ms.)
+constexpr unsigned long long kJoinOpen = 1ull << 16;
+constexpr unsigned long long kJoinWaitNs = 150000, kJoinWaitMinNs = 5000;
+constexpr uint64_t kMemberWaitNs = 1000000000ull;
+
+struct ServeCmd {
+    uint32_t what;  // 0: nothing to do, 1: run slot q, 2: leave
+    uint32_t q, rank, size;
+};
+
+// One lane, having joined or opened the team of slot q with the word `word`:
+// waits until the leader has closed it and returns its size.
+__device__ __forceinline__ uint32_t team_form(const SyncServe& A, uint32_t q, unsigned long long word,
+                                              bool leader, unsigned long long wait_ns) {
+    const uint64_t t0 = globaltimer();
+    for (;;) {
+        const unsigned long long w = ld_relaxed64(A.join + q);
+        if ((w >> 32) != (word >> 32) || !(w & kJoinOpen)) return (uint32_t)w & 0xFFu;
+        const bool full = (w & 0xFFu) >= ((w >> 8) & 0xFFu);
+        const uint64_t dt = globaltimer() - t0;
+        if (leader && (full || dt > wait_ns)) return (uint32_t)atomicAnd(A.join + q, ~kJoinOpen) & 0xFFu;
+        // (the leader closes the team well before this; the search's own
+        // barriers are bounded too)
+        if (!leader && dt > wait_ns) return (uint32_t)(w >> 8) & 0xFFu;
+    }
+}
+
+// Warp 0: something to do, or nothing.
+__device__ __forceinline__ ServeCmd serve_poll(const SyncServe& A, uint32_t cursor) {
+    const uint32_t lane = threadIdx.x & 31;
+    ServeCmd c = {0, 0, 0, 0};
+    unsigned long long work = 0;  // of all queries submitted or running
+    uint32_t near = ~0u;          // submitted query nearest after the cursor: its distance
+    for (uint32_t b = 0; b < A.nslots; b += 32) {
+        const uint32_t q = b + lane;
+        unsigned long long w = 0;
+        uint32_t st = 0;
+        if (q < A.nslots) {
+            w = ld_relaxed64(A.join + q);
+            st = ld_relaxed(A.state + q);
+        }
+        uint32_t m = __ballot_sync(0xFFFFFFFFu, (w & kJoinOpen) && (w & 0xFFu) < ((w >> 8) & 0xFFu));
+        while (m) {
+            const uint32_t l = __ffs(m) - 1;
+            m &= m - 1;
+            uint32_t rank = 0, size = 0;
+            if (lane == l) {
+                for (int tries = 0; tries < 8; ++tries) {
+                    if (!(w & kJoinOpen) || (w & 0xFFu) >= ((w >> 8) & 0xFFu)) break;
+                    const unsigned long long seen = atomicCAS(A.join + q, w, w + 1);
+                    if (seen == w) {
+                        rank = (uint32_t)w & 0xFFu;
+                        __threadfence();  // acquire: the slot's descriptor
+                        size = team_form(A, q, w, false, kMemberWaitNs);
+                        break;
+                    }
+                    w = seen;
+                }
+            }
+            size = __shfl_sync(0xFFFFFFFFu, size, l);
+            if (size) {
+                c.what = 1;
+                c.q = b + l;
+                c.rank = __shfl_sync(0xFFFFFFFFu, rank, l);
+                c.size = size;
+                return c;
+            }
+        }
+        if (st & 0xFFu) work += st >> kSlotWorkShift;
+        if ((st & 0xFFu) == kSlotSubmitted) near = min(near, q >= cursor ? q - cursor : q + A.nslots - cursor);
+    }
+    near = __reduce_min_sync(0xFFFFFFFFu, near);
+    if (near == ~0u) return c;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) work += __shfl_xor_sync(0xFFFFFFFFu, work, d);
+    const uint32_t q = (near + cursor) % A.nslots;
+    uint32_t size = 0;
+    if (lane == 0) {
+        if (atomicCAS(A.claim, 0u, 1u) == 0u) {
+            const uint32_t st = ld_relaxed(A.state + q);
+            const uint32_t run = (st & ~0xFFu) | kSlotRunning;
+            unsigned long long w = 0, wait = 0;
+            if ((st & 0xFFu) == kSlotSubmitted && atomicCAS(A.state + q, st, run) == st) {
+                __threadfence();  // acquire: the descriptor the host wrote before the state
+                atomicAdd(A.heartbeat, 1ull);
+                const unsigned long long mine = max(st >> kSlotWorkShift, 1u);
+                const unsigned long long part = (mine * gridDim.x + work - 1) / max(work, 1ull);
+                size = max(1u, (uint32_t)min(part, (unsigned long long)ld_l2(&A.slots[q].cap)));
+                if (size > 1) {
+                    // (work is in eighths of a microsecond)
+                    wait = min(kJoinWaitNs, max(kJoinWaitMinNs, 125ull * mine / (4 * size)));
+                    const unsigned long long seq = (ld_relaxed64(A.join + q) >> 32) + 1;
+                    w = seq << 32 | kJoinOpen | (unsigned long long)size << 8 | 1ull;
+                    __threadfence();
+                    st_relaxed64(A.join + q, w);
+                }
+            }
+            // (the team is open before the next claim can be made)
+            __threadfence();
+            st_relaxed(A.claim, 0u);
+            if (w) size = team_form(A, q, w, true, wait);
+        }
+    }
+    size = __shfl_sync(0xFFFFFFFFu, size, 0);
+    if (size) {
+        c.what = 1;
+        c.q = q;
+        c.size = size;
+    }
+    return c;
+}
+
+__global__ void __launch_bounds__(kSyncThreads, 1) sync_serve_kernel(const __grid_constant__ SyncServe A) {
+    __shared__ SyncSmem sm;
+    __shared__ SyncSlot slot;
+    __shared__ ServeCmd cmd;
+    uint64_t idle_since = 0;
+    unsigned long long last_beat = ~0ull;
+    uint32_t backoff = 64;
+    for (;;) {
+        if (threadIdx.x < 32) {
+            ServeCmd c = {2, 0, 0, 0};
+            if (ld_relaxed(A.stop_flag) == 0) {
+                c = serve_poll(A, blockIdx.x * 7u % A.nslots);
+                if (c.what == 0) {
+                    // nothing to do: sleep, or leave after idle_exit_ns without
+                    // progress anywhere (the host relaunches on demand)
+                    const unsigned long long beat = ld_relaxed64(A.heartbeat);
+                    const uint64_t now = globaltimer();
+                    if (beat != last_beat) {
+                        last_beat = beat;
+                        idle_since = now;
+                    } else if (now - idle_since > A.idle_exit_ns) {
+                        c.what = 2;
+                    }
+                    if (c.what == 0) __nanosleep(backoff);
+                    if (backoff < 1024) backoff <<= 1;
+                } else {
+                    backoff = 64;
+                    last_beat = ~0ull;
+                }
+            }
+            if (threadIdx.x == 0) cmd = c;
+        }
+        __syncthreads();
+        const ServeCmd c = cmd;
+        if (c.what == 2) break;
+        if (c.what == 1) {
+            // read through L2: the slot held another query before
+            const uint32_t* src = reinterpret_cast<const uint32_t*>(A.slots + c.q);
+            uint32_t* dst = reinterpret_cast<uint32_t*>(&slot);
+            for (uint32_t w = threadIdx.x; w < sizeof(SyncSlot) / 4; w += kSyncThreads) dst[w] = ld_l2(src + w);
+            Team T;
+            T.rank = c.rank;
+            T.size = T.expect = c.size;
+            __syncthreads();
+            const bool last = sync_search<false>(sm, slot.search, T);
+            if (threadIdx.x == 0 && last) {
+                // ticket and status reach the host's word after every write of
+                // the search (each CTA fenced its own before it left)
+                st_relaxed(A.state + c.q, kSlotFree);
+                atomicAdd(A.heartbeat, 1ull);
+                __threadfence_system();
+                const unsigned long long word = slot.ticket << 8 | (ld_relaxed(&slot.search.ctl->err) & 0xFFu);
+                asm volatile("st.release.sys.global.u64 [%0], %1;" ::"l"(slot.notify), "l"(word) : "memory");
+            }
+        }
+        __syncthreads();
+    }
+}
+
 static_assert(sizeof(SyncSmem) <= 31 * 1024, "two lists under the 32 KB shared-memory split");
 
 namespace {
@@ -106,7 +290,7 @@ int sync_max_ctas(int device, int sms) {
     int c = std::min(sms, 240);
     if (prepare(sync_kernel<false>, sms, &c) != cudaSuccess || prepare(sync_kernel<true>, sms, &c) != cudaSuccess ||
         prepare(sync_batch_kernel<false>, sms, &c) != cudaSuccess ||
-        prepare(sync_batch_kernel<true>, sms, &c) != cudaSuccess) {
+        prepare(sync_batch_kernel<true>, sms, &c) != cudaSuccess || prepare(sync_serve_kernel, sms, &c) != cudaSuccess) {
         cudaGetLastError();
         c = 0;
     }
@@ -133,6 +317,11 @@ cudaError_t launch_sync(const SyncSearch& S, int ctas, cudaStream_t s) {
     cudaError_t e = S.sigma ? cudaLaunchKernelEx(&cfg, sync_kernel<true>, S)
                             : cudaLaunchKernelEx(&cfg, sync_kernel<false>, S);
     return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+cudaError_t launch_sync_serve(const SyncServe& A, int ctas, cudaStream_t s) {
+    sync_serve_kernel<<<ctas, kSyncThreads, 0, s>>>(A);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_sync_batch(const SyncBatch& B, bool sigma, int ctas, cudaStream_t s) {

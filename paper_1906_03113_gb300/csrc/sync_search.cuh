@@ -247,16 +247,17 @@ __device__ __forceinline__ uint32_t wide_next(SyncSmem& sm, const SyncSearch& S,
 }
 
 // Thread 0 of a CTA that is done with a search: the last one to leave sets the
-// status and clears the barrier's words for the next search.
-__device__ __forceinline__ void sync_leave(const SyncSearch& S, const Team& T) {
+// status, clears the barrier's words for the next search and returns true.
+__device__ __forceinline__ bool sync_leave(const SyncSearch& S, const Team& T) {
     __threadfence();
-    if (atomicInc(&S.bar->exited, T.size - 1) != T.size - 1) return;
+    if (atomicInc(&S.bar->exited, T.size - 1) != T.size - 1) return false;
     __threadfence();
     for (int b = 0; b < 2; ++b) {
         S.bar->word[b] = S.bar->aux[b] = 0;
         S.bar->lcnt[b] = 0;
     }
     S.ctl->status = ld_relaxed(&S.ctl->err) ? kFailed : kDone;
+    return true;
 }
 
 // Runs one search on this team.  The outputs and the control block are written
@@ -267,8 +268,9 @@ __device__ __forceinline__ void sync_leave(const SyncSearch& S, const Team& T) {
 // of that (each thin -> wide switch rebuilds the bitmap, 8 bytes per vertex).
 // After a barrier thread 0 alone decides what follows: the same decision made
 // by every thread took 1.3 us a level on 32 warps.
+// Returns, in thread 0, whether this CTA was the last to leave.
 template <bool SIG>
-__device__ __forceinline__ void sync_search(SyncSmem& sm, const SyncSearch& S, const Team& T) {
+__device__ __forceinline__ bool sync_search(SyncSmem& sm, const SyncSearch& S, const Team& T) {
     const bool lead = threadIdx.x == 0;
     unsigned long long items;
     uint32_t k = 0, wide_levels = 0, act = kActThin;
@@ -387,8 +389,9 @@ __device__ __forceinline__ void sync_search(SyncSmem& sm, const SyncSearch& S, c
         if (sm.st_verts) atomicAdd(&c->reached, (uint32_t)sm.st_verts);
         atomicMax(&c->levels, sm.levels);
         if (T.rank == 0 && wide_levels) atomicAdd(&c->wide_levels, wide_levels);
-        sync_leave(S, T);
+        return sync_leave(S, T);
     }
+    return false;
 }
 
 }  // namespace abfs

@@ -141,3 +141,39 @@ def test_multi_source_on_a_skewed_graph():
         lo, po = oracle.bfs(g, s)
         assert np.array_equal(L.cpu().numpy(), lo) and np.array_equal(P.cpu().numpy(), po), s
     G.destroy()
+
+
+@pytest.mark.parametrize("slots", [1, 3, 40])
+def test_serving_teams(slots):
+    """Queries large enough for teams of CTAs beside small ones, few slots (each
+    reused) and many, two bursts with the device launch ended in between."""
+    import time
+    hosts = [synth.rmat(17, 16.0, seed=41), synth.er(20000, 10.0, seed=42), synth.er(700, 5.0, seed=43),
+             synth.grid(60, 41)]
+    dev = [abfs.graph_create(g.colptr, g.rowidx, directed=g.directed) for g in hosts]
+    srcs = [synth.sources_with_degree(g, 8, seed=5) for g in hosts]
+    want = {}
+    srv = abfs.Server(dev, abfs.serve_default_cfg(max_slots=slots, memory_budget=1 << 30, idle_exit_ms=1))
+    for burst in range(2):
+        jobs = []
+        for i in range(48):
+            gi = i % len(hosts)
+            s = int(srcs[gi][(i // 4 + burst) % 8])
+            lev, par = (torch.full((hosts[gi].n,), 7, dtype=torch.int32, device="cuda") for _ in range(2))
+            jobs.append([gi, s, lev, par])
+        # the fills are done before a query may write (the server has its own stream)
+        torch.cuda.synchronize()
+        for job in jobs:
+            job.append(srv.submit(*job))
+        for gi, s, lev, par, t in jobs:
+            assert srv.wait(t) == 0
+        for gi, s, lev, par, t in jobs:
+            if (gi, s) not in want:
+                want[gi, s] = oracle.bfs(hosts[gi], s)
+            lo, po = want[gi, s]
+            assert np.array_equal(lev.cpu().numpy(), lo) and np.array_equal(par.cpu().numpy(), po), (gi, s)
+        time.sleep(0.05)
+    rep = srv.stop()
+    assert rep["completed"] == 96 and rep["failed"] == 0
+    for G in dev:
+        G.destroy()
