@@ -353,6 +353,34 @@ __device__ __noinline__ void sync_bitmaps(const SyncSearch& S, const Team& T, ui
     }
 }
 
+// Writes the items of this warp's columns (lane l's: [cb, cb + len), label j;
+// none if empty) from position `at` of the global list on; returns their number.
+// The lanes share the items: a hub's 400 written by its own lane held its warp,
+// and with it the level, for 25 us.  Whole warp.
+__device__ __noinline__ uint32_t list_put_long(const SyncSearch& S, uint32_t p, uint32_t at, uint32_t j,
+                                               uint32_t cb, uint32_t len) {
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t ns = items_of(cb, len), incl = warp_incl_scan(ns);
+    const uint32_t tot = __shfl_sync(0xFFFFFFFFu, incl, 31);
+#pragma unroll 1
+    for (uint32_t x0 = 0; x0 < tot; x0 += 32) {
+        const uint32_t x = x0 + lane;
+        uint32_t own = 0;  // the first lane whose inclusive count exceeds x
+#pragma unroll
+        for (uint32_t d = 16; d > 0; d >>= 1)
+            if (x >= __shfl_sync(0xFFFFFFFFu, incl, own + d - 1)) own += d;
+        const uint32_t oj = __shfl_sync(0xFFFFFFFFu, j, own), ob = __shfl_sync(0xFFFFFFFFu, cb, own);
+        const uint32_t ol = __shfl_sync(0xFFFFFFFFu, len, own);
+        const uint32_t of = __shfl_sync(0xFFFFFFFFu, incl - ns, own);
+        if (x < tot) {
+            uint32_t b, l;
+            item_at(ob, ol, x - of, b, l);
+            list_put(S, p, (unsigned long long)at + x, oj, b, l);
+        }
+    }
+    return tot;
+}
+
 // The frontier list of level k + 1.  kFromKeys: after a wide level, its new
 // vertices are those outside the bitmap whose key has a parent; they get their
 // level, join the bitmap (each word has one writer) and make up the frontier
@@ -380,6 +408,7 @@ __device__ __noinline__ void sync_extract(SyncSmem& sm, const SyncSearch& S, con
     const uint32_t g0 = (warp * T.size + T.rank) * Q;  // groups of Q words, round robin
     uint32_t* const khi = reinterpret_cast<uint32_t*>(S.key) + 1;
     uint32_t verts = 0, entries = 0, mine = 0;
+#pragma unroll 1
     for (uint32_t wb = g0; wb < S.nwords; wb += Q * W) {
         const bool own = lane < Q && wb + lane < S.nwords;
         uint32_t word = 0, seen = 0, add = 0;
@@ -445,6 +474,7 @@ __device__ __noinline__ void sync_extract(SyncSmem& sm, const SyncSearch& S, con
     __syncthreads();
     if (!wt) return;
     uint32_t at = sm.wpre[warp];
+#pragma unroll 1
     for (uint32_t wb = g0; wb < S.nwords; wb += Q * W) {
         // (this lane's own words of the first pass)
         const uint32_t word = lane < Q && wb + lane < S.nwords ? ld_l2(S.fbm[pn] + wb + lane) : 0u;
@@ -464,17 +494,15 @@ __device__ __noinline__ void sync_extract(SyncSmem& sm, const SyncSearch& S, con
         for (uint32_t q = 0; q < Q; ++q) {
             const uint32_t ns = items_of(cb[q], len[q]);
             if (!__any_sync(0xFFFFFFFFu, ns != 0)) continue;
-            const uint32_t incl = warp_incl_scan(ns);
-            if (ns) {
-                const unsigned long long v = v0 + 32 * q;
-                const uint32_t j = S.lab ? ld_ro(S.lab + v) : (uint32_t)v;
-                for (uint32_t i = 0; i < ns; ++i) {
-                    uint32_t b, l;
-                    item_at(cb[q], len[q], i, b, l);
-                    list_put(S, pn, (unsigned long long)at + incl - ns + i, j, b, l);
-                }
+            const unsigned long long v = v0 + 32 * q;
+            const uint32_t j = ns && S.lab ? ld_ro(S.lab + v) : (uint32_t)v;
+            if (!__any_sync(0xFFFFFFFFu, ns > 1)) {
+                const uint32_t m = __ballot_sync(0xFFFFFFFFu, ns != 0);
+                if (ns) list_put(S, pn, (unsigned long long)at + __popc(m & lanemask_lt()), j, cb[q], len[q]);
+                at += __popc(m);
+            } else {
+                at += list_put_long(S, pn, at, j, cb[q], len[q]);
             }
-            at += __shfl_sync(0xFFFFFFFFu, incl, 31);
         }
     }
 }
