@@ -65,7 +65,8 @@ struct SyncSmem {
     uint32_t act;                     // SyncAct after the last barrier
     unsigned long long items;         // the next level's items
     // thread 0's state of the search
-    uint32_t lim_items, lim_ent;      // a list above either is heavy
+    uint32_t lim;                     // a list of more weight is heavy
+    float weight;                     // of the current level's lists
     uint32_t bu;
     unsigned long long nf, entries, seen;
     unsigned long long st_read, st_unmasked, st_verts, st_ent;
@@ -115,9 +116,9 @@ __device__ __forceinline__ void red_add_release64(unsigned long long* p, unsigne
     asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-// Thread 0 of each CTA: adds `add` and the arrival to the barrier's word, waits
-// until the team has arrived and returns the totals, or ~0 when the bounded
-// wait ran out.  The wait itself delivers the totals: no further read follows
+// One thread of each CTA: adds `add` and the arrival to the barrier's word
+// (bar_arrive), waits until the team has arrived and returns the totals, or ~0
+// when the bounded wait ran out (bar_poll).  The wait itself delivers the totals: no further read follows
 // unless `aux` is wanted.
 //
 // FULL: what the CTAs wrote before the barrier can be read after it.  Without
@@ -127,19 +128,25 @@ __device__ __forceinline__ void red_add_release64(unsigned long long* p, unsigne
 // word is another atomic or a strong load there.  The release and the acquire
 // cost 1.1 + 0.8 thousand cycles of a thin level's 8.4.
 template <bool FULL>
-__device__ __forceinline__ unsigned long long bar_wait(SyncSmem& sm, const SyncSearch& S, const Team& T,
+__device__ __forceinline__ void bar_arrive(SyncSmem& sm, const SyncSearch& S, const Team& T,
+                                           unsigned long long add, unsigned long long aux) {
+    if (T.expect == 1) return;
+    const uint32_t b = sm.step & 1u;
+    if (FULL) {
+        if (aux) red_add64(&S.bar->aux[b], aux);
+        red_add_release64(&S.bar->word[b], add + (1ull << kArriveShift));
+    } else {
+        red_add64(&S.bar->word[b], add + (1ull << kArriveShift));
+    }
+}
+template <bool FULL>
+__device__ __forceinline__ unsigned long long bar_poll(SyncSmem& sm, const SyncSearch& S, const Team& T,
                                                        unsigned long long add, unsigned long long& aux) {
     if (T.expect == 1) return add;
     const uint32_t b = sm.step & 1u;
     ++sm.step;
     unsigned long long* w = &S.bar->word[b];
     const unsigned long long before = sm.word[b];
-    if (FULL) {
-        if (aux) red_add64(&S.bar->aux[b], aux);
-        red_add_release64(w, add + (1ull << kArriveShift));
-    } else {
-        red_add64(w, add + (1ull << kArriveShift));
-    }
     unsigned long long v;
     uint64_t t0 = 0;
     for (uint32_t spin = 0;; ++spin) {
@@ -164,6 +171,12 @@ __device__ __forceinline__ unsigned long long bar_wait(SyncSmem& sm, const SyncS
         sm.aux[b] = x;
     }
     return (v - before) & ((1ull << kArriveShift) - 1);
+}
+template <bool FULL>
+__device__ __forceinline__ unsigned long long bar_wait(SyncSmem& sm, const SyncSearch& S, const Team& T,
+                                                       unsigned long long add, unsigned long long& aux) {
+    bar_arrive<FULL>(sm, S, T, add, aux);
+    return bar_poll<FULL>(sm, S, T, add, aux);
 }
 
 // A plain full barrier; the sums of `add` and `ent` (thread 0's) reach sm.items
@@ -222,8 +235,8 @@ __device__ __noinline__ void list_dump(SyncSmem& sm, const SyncSearch& S, uint32
 // at most kThinCap per CTA) into its list `q`.  Whole CTA.
 __device__ __noinline__ void list_slice(SyncSmem& sm, const SyncSearch& S, const Team& T, uint32_t q,
                                         uint32_t p, unsigned long long items) {
-    const unsigned long long lo = items * T.rank / T.size, hi = items * (T.rank + 1) / T.size;
-    const uint32_t c = (uint32_t)(hi - lo);
+    const uint32_t n = (uint32_t)items, lo = n * T.rank / T.size, hi = n * (T.rank + 1) / T.size;
+    const uint32_t c = hi - lo;
     for (uint32_t i = threadIdx.x; i < c && lo + i < S.icap; i += kSyncThreads) {
         sm.ij[q][i] = ld_l2(S.lj[p] + lo + i);
         sm.ib[q][i] = ld_l2(S.lb[p] + lo + i);

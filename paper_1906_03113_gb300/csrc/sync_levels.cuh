@@ -15,51 +15,22 @@ namespace abfs {
 // is row index, atomicMin, barrier.  The lists are evened out only when a few
 // CTAs hold much more than their share (see sync_search).
 
-// Appends the rows won by this warp's lanes (row r, column [cb, ce)) to the
-// CTA's list `q` (level k + 1); what does not fit goes to the global list.
-// Whole warp.
-__device__ __forceinline__ void thin_append(SyncSmem& sm, const SyncSearch& S, uint32_t k, uint32_t q,
-                                            bool win, uint32_t r, uint32_t cb, uint32_t ce) {
-    if (!__any_sync(0xFFFFFFFFu, win)) return;
+// The general case of thin_append: the warp's `tot` items (lane l's: the column
+// [cb, cb + len) of label j; inclusive counts incl) go to positions at... of the
+// list, those from kThinCap on to the global list, written by the warp together.
+__device__ __noinline__ void thin_append_long(SyncSmem& sm, const SyncSearch& S, uint32_t k, uint32_t q,
+                                              uint32_t at, uint32_t tot, uint32_t incl, uint32_t j,
+                                              uint32_t cb, uint32_t len) {
     const uint32_t lane = threadIdx.x & 31;
-    const uint32_t len = win ? ce - cb : 0u;
-    const uint32_t ns = items_of(cb, len);
-    const uint32_t ent = __reduce_add_sync(0xFFFFFFFFu, len);
-    const uint32_t j = ns && S.lab ? ld_ro(S.lab + r) : r;
-    // the next level starts with these row indices
-    if (ns) asm volatile("prefetch.global.L2 [%0];" ::"l"(S.rowidx + cb));
-    const bool longs = __any_sync(0xFFFFFFFFu, ns > 1);
-    uint32_t incl = 0, pre = 0, tot;
-    if (longs) {
-        incl = warp_incl_scan(ns);
-        tot = __shfl_sync(0xFFFFFFFFu, incl, 31);
-    } else {
-        const uint32_t m = __ballot_sync(0xFFFFFFFFu, ns != 0);
-        tot = __popc(m);
-        pre = __popc(m & lanemask_lt());
-    }
-    // lane 0 reserves the items, lane 1 counts the entries
-    uint32_t at = 0;
-    if (lane < 2) at = atomicAdd(&sm.app[q][lane], lane ? ent : tot);
-    at = __shfl_sync(0xFFFFFFFFu, at, 0);
-    if (!longs && at + tot <= kThinCap) {
-        if (ns) {
-            sm.ij[q][at + pre] = j;
-            sm.ib[q][at + pre] = cb;
-            sm.il[q][at + pre] = len;
-        }
-        return;
-    }
-    // long columns or a full list: the warp writes the items together, those
-    // from position `room` on to the global list
-    if (!longs) incl = pre + (ns != 0);
     const uint32_t p = (k + 1) & 1;
+    const uint32_t before = incl - items_of(cb, len);
     const uint32_t room = at < kThinCap ? min(kThinCap - at, tot) : 0u;
     uint32_t spill = 0;
     if (room < tot) {
         if (lane == 0) spill = atomicAdd(&S.bar->lcnt[p], tot - room);
         spill = __shfl_sync(0xFFFFFFFFu, spill, 0);
     }
+#pragma unroll 1
     for (uint32_t x0 = 0; x0 < tot; x0 += 32) {
         const uint32_t x = x0 + lane;
         uint32_t own = 0;  // the first lane whose inclusive count exceeds x
@@ -68,7 +39,7 @@ __device__ __forceinline__ void thin_append(SyncSmem& sm, const SyncSearch& S, u
             if (x >= __shfl_sync(0xFFFFFFFFu, incl, own + d - 1)) own += d;
         const uint32_t oj = __shfl_sync(0xFFFFFFFFu, j, own), ob = __shfl_sync(0xFFFFFFFFu, cb, own);
         const uint32_t ol = __shfl_sync(0xFFFFFFFFu, len, own);
-        const uint32_t of = __shfl_sync(0xFFFFFFFFu, incl - ns, own);
+        const uint32_t of = __shfl_sync(0xFFFFFFFFu, before, own);
         if (x < tot) {
             uint32_t b, l;
             item_at(ob, ol, x - of, b, l);
@@ -83,91 +54,165 @@ __device__ __forceinline__ void thin_append(SyncSmem& sm, const SyncSearch& S, u
     }
 }
 
+// Appends the rows won by this warp's lanes (row r, column [cb, ce)) to the
+// CTA's list `q` (level k + 1); what does not fit goes to the global list.
+// Whole warp.
+__device__ __forceinline__ void thin_append(SyncSmem& sm, const SyncSearch& S, uint32_t k, uint32_t q,
+                                            bool win, uint32_t r, uint32_t cb, uint32_t ce) {
+    if (!__any_sync(0xFFFFFFFFu, win)) return;
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t len = win ? ce - cb : 0u;
+    const uint32_t ns = items_of(cb, len);
+    const uint32_t ent = __reduce_add_sync(0xFFFFFFFFu, len);
+    const uint32_t j = ns && S.lab ? ld_ro(S.lab + r) : r;
+    // the next level starts with these row indices
+    if (ns) asm volatile("prefetch.global.L2 [%0];" ::"l"(S.rowidx + cb));
+    const bool longs = __any_sync(0xFFFFFFFFu, ns > 1);
+    uint32_t incl, tot;
+    if (longs) {
+        incl = warp_incl_scan(ns);
+        tot = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    } else {
+        const uint32_t m = __ballot_sync(0xFFFFFFFFu, ns != 0);
+        tot = __popc(m);
+        incl = __popc(m & lanemask_lt()) + ns;
+    }
+    // lane 0 reserves the items, lane 1 counts the entries
+    uint32_t at = 0;
+    if (lane < 2) at = atomicAdd(&sm.app[q][lane], lane ? ent : tot);
+    at = __shfl_sync(0xFFFFFFFFu, at, 0);
+    if (longs || at + tot > kThinCap) {
+        thin_append_long(sm, S, k, q, at, tot, incl, j, cb, len);
+    } else if (ns) {
+        sm.ij[q][at + incl - 1] = j;
+        sm.ib[q][at + incl - 1] = cb;
+        sm.il[q][at + incl - 1] = len;
+    }
+}
+
 // Expands the columns of this CTA's list of level k (list k & 1) into its list
 // of level k + 1.  The warps share the list's batches of 32 items evenly; the
 // warps of a batch take its groups of 32 entries in turn, one entry per lane
 // and kThinIlp groups in flight, so that one hub or a handful of columns keeps
-// all of them busy.  Whole CTA.
+// all of them busy.
+//
+// A warp's first groups are staged while the team's barrier is under way: the
+// row indices (and, where a CTA has few entries and the level is bound by
+// latency, the rows' columns; their key words are brought to the L2) depend on
+// this CTA's list alone.  The chain from one barrier to the next is then claim,
+// append, arrive: 4096^2 grid 19.7 -> 15.4 ms, RGG 2^22 10.8 -> 8.7 ms.
 constexpr int kThinIlp = 2;
+// Entries per CTA up to which the columns of all rows are staged instead of
+// looked up for the rows that are won, and the key words prefetched (the grid
+// 16.5 ms without the prefetch), and up to which a list is staged before the
+// barrier at all: a longer list is bound by its claims, and often the next
+// level turns out to be wide (R-MAT-20 5 us slower with every list staged).
+constexpr uint32_t kThinEarly = 1024, kThinPrefetch = 512, kThinAhead = 2048;
 
-template <bool SIG>
-__device__ __forceinline__ void thin_level(SyncSmem& sm, const SyncSearch& S, uint32_t k, SyncTally& t) {
-    const uint32_t cur = k & 1;
+struct ThinStage {
+    uint32_t r[kThinIlp], jj[kThinIlp], cb[kThinIlp], ce[kThinIlp];
+    uint32_t j, first, shift;  // this lane's item: column, first entry, its position less that
+    uint32_t e0, total, step;  // the warp's next group, the batch's entries, entries between groups
+    bool early;                // cb and ce are there
+};
+
+// The rows and columns of kThinIlp groups from st.e0 on.
+__device__ __forceinline__ void thin_groups(const SyncSearch& S, ThinStage& st) {
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t le_mask = (2u << lane) - 1u;
+#pragma unroll
+    for (int u = 0; u < kThinIlp; ++u) {
+        const uint32_t g = st.e0 + u * st.step;
+        st.r[u] = kUnset;
+        st.jj[u] = 0;
+        if (g < st.total) {
+            const uint32_t rel = st.first - g;
+            const uint32_t before = __popc(__ballot_sync(0xFFFFFFFFu, st.first < g));
+            const uint32_t w = __reduce_or_sync(0xFFFFFFFFu, rel < 32u ? 1u << rel : 0u);
+            // the item of entry g + lane
+            const uint32_t own = (before + __popc(w & le_mask) - 1u) & 31u;
+            const uint32_t pos = __shfl_sync(0xFFFFFFFFu, st.shift, own) + g + lane;
+            st.jj[u] = __shfl_sync(0xFFFFFFFFu, st.j, own);
+            if (g + lane < st.total) st.r[u] = ld_ro(S.rowidx + pos);
+        }
+    }
+}
+
+// Whole CTA.
+__device__ __forceinline__ void thin_stage(const SyncSmem& sm, const SyncSearch& S, uint32_t cur, ThinStage& st) {
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t cnt = min(sm.app[cur][0], kThinCap);
     // batches of 32 items, rounded up to a power of two (at most one per warp)
     const uint32_t lb = cnt > 32 ? 32 - __clz((cnt - 1) / 32) : 0;
     const uint32_t batch = warp & ((1u << lb) - 1u), nth = warp >> lb;
     const uint32_t i0 = 32 * batch;
-    if (i0 >= cnt || (lb == 0 && 32 * nth >= sm.app[cur][1])) return;
-    const uint32_t step = (32 * kSyncWarps) >> lb;  // entries between a warp's groups
-    const uint32_t le_mask = (2u << lane) - 1u;
-    const unsigned long long hi = (unsigned long long)(k + 1) << 32;
-    const uint32_t m = min(32u, cnt - i0);
-    uint32_t j = 0, beg = 0, len = 0;
-    if (lane < m) {
-        j = sm.ij[cur][i0 + lane];
+    st.e0 = 32 * nth;
+    st.total = 0;
+    if (i0 >= cnt || (lb == 0 && st.e0 >= sm.app[cur][1])) return;
+    st.step = (32 * kSyncWarps) >> lb;
+    uint32_t beg = 0, len = 0;
+    st.j = 0;
+    if (lane < cnt - i0) {
+        st.j = sm.ij[cur][i0 + lane];
         beg = sm.ib[cur][i0 + lane];
         len = sm.il[cur][i0 + lane];
     }
-    if (nth == 0) t.read += len;
     const uint32_t incl = warp_incl_scan(len);
-    const uint32_t total = __shfl_sync(0xFFFFFFFFu, incl, 31);
-    const uint32_t first = incl - len;  // this item's first entry
-    const uint32_t shift = beg - first;
-    // a warp with a group or two is bound by latency: the columns of all rows
-    // are looked up beside the claims instead of after them
-    const bool early = total <= kThinIlp * step;
-    for (uint32_t e0 = 32 * nth; e0 < total; e0 += kThinIlp * step) {
-        uint32_t r[kThinIlp], jj[kThinIlp];
+    st.total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    // (lanes without an item are past every group)
+    st.first = lane < cnt - i0 ? incl - len : kUnset;
+    st.shift = beg - st.first;
+    st.early = (st.total << lb) <= kThinEarly;
+    thin_groups(S, st);
+    if (!st.early) return;
+    const bool far = (st.total << lb) <= kThinPrefetch;
 #pragma unroll
-        for (int u = 0; u < kThinIlp; ++u) {
-            const uint32_t g = e0 + u * step;
-            r[u] = kUnset;
-            jj[u] = 0;
-            if (g < total) {
-                const uint32_t rel = first - g;
-                const uint32_t before = __popc(__ballot_sync(0xFFFFFFFFu, lane < m && first < g));
-                const uint32_t w =
-                    __reduce_or_sync(0xFFFFFFFFu, (lane < m && rel < 32u) ? 1u << rel : 0u);
-                // the item of entry g + lane
-                const uint32_t own = (before + __popc(w & le_mask) - 1u) & 31u;
-                const uint32_t pos = __shfl_sync(0xFFFFFFFFu, shift, own) + g + lane;
-                jj[u] = __shfl_sync(0xFFFFFFFFu, j, own);
-                if (g + lane < total) r[u] = ld_ro(S.rowidx + pos);
-            }
-        }
+    for (int u = 0; u < kThinIlp; ++u) {
+        if (st.r[u] == kUnset) continue;
+        if (far) asm volatile("prefetch.global.L2 [%0];" ::"l"(S.key + st.r[u]));
+        st.cb[u] = ld_ro(S.colptr + st.r[u]);
+        st.ce[u] = ld_ro(S.colptr + st.r[u] + 1);
+    }
+}
+
+// Whole CTA.
+template <bool SIG>
+__device__ __forceinline__ void thin_claims(SyncSmem& sm, const SyncSearch& S, uint32_t k, ThinStage& st,
+                                            SyncTally& t) {
+    const uint32_t cur = k & 1;
+    const unsigned long long hi = (unsigned long long)(k + 1) << 32;
+#pragma unroll 1
+    while (st.e0 < st.total) {
         unsigned long long old[kThinIlp];
-        uint32_t cb[kThinIlp], ce[kThinIlp];
 #pragma unroll
         for (int u = 0; u < kThinIlp; ++u) {
             old[u] = 0;
-            cb[u] = ce[u] = 0;
-            if (r[u] != kUnset) {
-                old[u] = atomicMin(S.key + r[u], hi | jj[u]);
-                if (early) {
-                    cb[u] = ld_ro(S.colptr + r[u]);
-                    ce[u] = ld_ro(S.colptr + r[u] + 1);
-                }
-            }
+            if (st.r[u] != kUnset) old[u] = atomicMin(S.key + st.r[u], hi | st.jj[u]);
         }
 #pragma unroll
         for (int u = 0; u < kThinIlp; ++u) {
-            if (e0 + u * step >= total) break;
-            const bool pass = r[u] != kUnset && (uint32_t)(old[u] >> 32) > k;
+            if (st.e0 + u * st.step >= st.total) break;
+            const bool have = st.r[u] != kUnset;
+            const bool pass = have && (uint32_t)(old[u] >> 32) > k;
             const bool win = pass && old[u] == kKeyUnset;
+            t.read += have;
             t.unmasked += pass;
             if (win) {
                 ++t.verts;
                 t.levels = k + 2;
             }
-            if (SIG && pass) red_add64(S.sigma + r[u], ld_l2(S.sigma + jj[u]));
-            if (win && !early) {
-                cb[u] = ld_ro(S.colptr + r[u]);
-                ce[u] = ld_ro(S.colptr + r[u] + 1);
+            if (SIG && pass) red_add64(S.sigma + st.r[u], ld_l2(S.sigma + st.jj[u]));
+            uint32_t cb = 0, ce = 0;
+            if (win) {
+                cb = st.early ? st.cb[u] : ld_ro(S.colptr + st.r[u]);
+                ce = st.early ? st.ce[u] : ld_ro(S.colptr + st.r[u] + 1);
             }
-            thin_append(sm, S, k, cur ^ 1, win, r[u], cb[u], ce[u]);
+            thin_append(sm, S, k, cur ^ 1, win, st.r[u], cb, ce);
         }
+        st.e0 += kThinIlp * st.step;
+        if (st.e0 >= st.total) break;
+        st.early = false;
+        thin_groups(S, st);
     }
 }
 
@@ -532,11 +577,12 @@ __device__ __noinline__ void sync_extract(SyncSmem& sm, const SyncSearch& S, con
 constexpr uint32_t kBuWords = 4;
 
 __device__ __noinline__ void sync_bottom_up(SyncSmem& sm, const SyncSearch& S, const Team& T, uint32_t k) {
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t lane = threadIdx.x & 31;
     const uint32_t p = k & 1, pn = p ^ 1;
     const uint32_t* const fbm = S.fbm[p];
     SyncTally t;
     uint32_t verts = 0, entries = 0;
+#pragma unroll 1
     for (;;) {
         uint32_t x = 0;
         if (lane == 0) x = atomicAdd(&sm.tick, 1u);

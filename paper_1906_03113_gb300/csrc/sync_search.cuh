@@ -92,7 +92,8 @@ __device__ __forceinline__ void sync_source(SyncSmem& sm, const SyncSearch& S, c
     const uint32_t cb = ld_ro(S.colptr + S.src);
     const uint32_t len = ld_ro(S.colptr + S.src + 1) - cb;
     items = items_of(cb, len);
-    const uint32_t lo = (uint32_t)(items * T.rank / T.size), hi = (uint32_t)(items * (T.rank + 1) / T.size);
+    const uint32_t ni = (uint32_t)items;  // (at most 2^24: 32 bits hold the products)
+    const uint32_t lo = ni * T.rank / T.size, hi = ni * (T.rank + 1) / T.size;
     // a column too long for the team's lists starts in the global list
     const bool global = items > (unsigned long long)T.size * kThinCap;
     for (uint32_t i = lo + threadIdx.x; i < hi; i += kSyncThreads) {
@@ -113,8 +114,8 @@ __device__ __forceinline__ void sync_source(SyncSmem& sm, const SyncSearch& S, c
         sm.app[0][1] = ~0u;  // entries: not known
         sm.app[1][0] = sm.app[1][1] = 0;
         sm.verts = sm.ent = 0;
-        sm.lim_items = 64;
-        sm.lim_ent = 2048;
+        sm.lim = 1024;
+        sm.weight = (float)len + 4.f * (float)items + 1.f;
         sm.bu = 0;
         sm.nf = 1;
         sm.seen = sm.entries = len;
@@ -125,13 +126,18 @@ __device__ __forceinline__ void sync_source(SyncSmem& sm, const SyncSearch& S, c
     }
 }
 
-// A list is heavy above twice an even share of the current level and what a
-// CTA expands without queueing (64 items: two per warp; 2048 entries: two
-// groups per warp).
-__device__ __forceinline__ void heavy_limits(SyncSmem& sm, const Team& T, float items, float ent) {
-    const float share = 2.f / (float)T.size;
-    sm.lim_items = 64u + (uint32_t)(items * share);
-    sm.lim_ent = 2048u + (uint32_t)(ent * share);
+// A list's cost to its CTA, in entries: a claim each, and per item its append
+// and look-up.  A list is heavy above what a CTA expands in about a microsecond
+// and twice an even share of the next level if that grows as this one did
+// (capped, so that a hub's list is noticed): evening the lists out costs 5 us.
+// (Without the growth, ER 2^16 of degree 8 pays for it once more just before its
+// largest level, when some lists pass the limit by chance: 52 -> 59 us.)
+__device__ __forceinline__ uint32_t list_weight(uint32_t items, uint32_t ent) { return ent + 4 * items; }
+__device__ __forceinline__ void heavy_limit(SyncSmem& sm, const Team& T, float items, float ent) {
+    const float w = ent + 4.f * items;
+    const float next = w * fminf(8.f, fmaxf(1.f, __fdividef(w, sm.weight)));
+    sm.lim = 1024u + (uint32_t)__fdividef(2.f * next, (float)T.size);
+    sm.weight = fmaxf(w, 1.f);
 }
 __device__ __forceinline__ uint32_t tot_items(unsigned long long tot) {
     return (uint32_t)(tot >> kItemShift) & ((1u << (kHeavyShift - kItemShift)) - 1u);
@@ -167,13 +173,10 @@ __device__ __forceinline__ uint32_t thin_next(SyncSmem& sm, const SyncSearch& S,
         }
     }
     if (ent >= wide_line(S, items, ent) || items > T.size * kThinCap) return kActWide;
-    // a list is full, or a few CTAs hold much more than the others (but when
-    // the frontier has outgrown the limits, lists above them say nothing)
+    // a list is full, or a few CTAs hold much more than the others
     const uint32_t heavy = flags & 0xFFu;
-    const float n2 = 2.f / (float)T.size;
-    const bool grown = (float)sm.lim_items < n2 * (float)items && (float)sm.lim_ent < n2 * (float)ent;
-    if ((flags >> 8) || (heavy && 2 * heavy <= T.size && !grown)) {
-        heavy_limits(sm, T, (float)items, (float)ent);
+    if ((flags >> 8) || (heavy && 2 * heavy <= T.size)) {
+        heavy_limit(sm, T, (float)items, (float)ent);
         return kActEven;
     }
     return kActThin;
@@ -186,32 +189,45 @@ __device__ __forceinline__ uint32_t thin_next(SyncSmem& sm, const SyncSearch& S,
 template <bool SIG>
 __device__ __noinline__ uint32_t thin_run(SyncSmem& sm, const SyncSearch& S, const Team& team, uint32_t k) {
     const Team T = team;
-    const bool lead = threadIdx.x == 0;
+    // the barrier and the decision fall to the warp that has work of its own
+    // only when all of them have
+    const bool lead = threadIdx.x == kSyncThreads - 32;
     const bool want_aux = S.bu_alpha != 0 || S.trace != nullptr;
     SyncTally t;
+    ThinStage st;
     uint32_t act;
+    bool staged = false;
+    __syncthreads();
     do {
+        if (!staged) thin_stage(sm, S, k & 1, st);
         if (S.trace) sync_trace(S, T, kPhLevel, k, 4u, (uint32_t)sm.items, (uint32_t)sm.nf, (uint32_t)sm.entries);
-        thin_level<SIG>(sm, S, k, t);
+        thin_claims<SIG>(sm, S, k, st, t);
         __syncthreads();
-        unsigned long long tot = 0, aux = 0;
+        const uint32_t cur = k & 1;
+        unsigned long long add = 0, aux = 0;
         if (lead) {
-            const uint32_t cur = k & 1;
             const uint32_t c = sm.app[cur ^ 1][0], e = sm.app[cur ^ 1][1];
-            unsigned long long add =
-                (unsigned long long)min(c, kItemClamp) << kItemShift | min(e / kEntUnit, kEntClamp);
-            if (c > sm.lim_items || e > sm.lim_ent) add += 1ull << kHeavyShift;
+            add = (unsigned long long)min(c, kItemClamp) << kItemShift | min(e / kEntUnit, kEntClamp);
+            if (list_weight(c, e) > sm.lim) add += 1ull << kHeavyShift;
             if (c > kThinCap) add += 1ull << kFullShift;
+            aux = e;
+            if (SIG || want_aux) bar_arrive<true>(sm, S, T, add, aux);
+            else bar_arrive<false>(sm, S, T, add, aux);
             sm.app[cur][0] = sm.app[cur][1] = 0;
             sm.st_ent += e;
-            aux = e;
-            tot = SIG || want_aux ? bar_wait<true>(sm, S, T, add, aux) : bar_wait<false>(sm, S, T, add, aux);
+        }
+        __syncwarp();
+        staged = sm.app[cur ^ 1][1] <= kThinAhead;
+        if (staged) thin_stage(sm, S, cur ^ 1, st);
+        unsigned long long tot = 0;
+        if (lead) {
+            tot = SIG || want_aux ? bar_poll<true>(sm, S, T, add, aux) : bar_poll<false>(sm, S, T, add, aux);
             sm.act = thin_next(sm, S, T, tot, aux, want_aux);
         }
         __syncthreads();
         ++k;
         act = sm.act;
-        if (lead && act == kActThin) heavy_limits(sm, T, (float)tot_items(tot), (float)tot_ent(tot));
+        if (lead && act == kActThin) heavy_limit(sm, T, (float)tot_items(tot), (float)tot_ent(tot));
     } while (act == kActThin);
     tally_add(sm, t.read, t.unmasked);
     t.verts = __reduce_add_sync(0xFFFFFFFFu, t.verts);
@@ -242,7 +258,7 @@ __device__ __forceinline__ uint32_t wide_next(SyncSmem& sm, const SyncSearch& S,
     if (bottom_up || tot > (unsigned long long)T.size * kThinCap ||
         sm.entries >= wide_line(S, tot, sm.entries) / 2)
         return kActWide;
-    heavy_limits(sm, T, (float)tot, (float)sm.entries);
+    heavy_limit(sm, T, (float)tot, (float)sm.entries);
     return kActSlice;
 }
 
