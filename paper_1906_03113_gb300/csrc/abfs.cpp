@@ -223,10 +223,14 @@ double sync_work_us(uint32_t n, uint64_t nnz, uint32_t ms) {
     return (ms ? 2e-3 + 6e-5 * ms : 0.9e-3) * (double)nnz + 1.5e-3 * n * (ms ? 1.0 + ms / 8.0 : 1.0);
 }
 
+// Whether one CTA can hold a search whole (sync_local.cuh): its keys in shared
+// memory, its graph in the L1.
+bool sync_local(uint32_t n, uint64_t nnz) { return n <= kLocalN && nnz <= kLocalNnz; }
+
 // The largest useful team of a search: a few thousand entries per CTA.  Up to
 // 16 384 entries one CTA, without barriers between CTAs, is fastest.
-int sync_team_cap(uint64_t nnz, int most) {
-    const uint64_t want = nnz <= 16384 ? 1 : (nnz + 4095) / 4096;
+int sync_team_cap(const SyncSearch& S, int most) {
+    const uint64_t want = S.local || S.nnz <= 16384 ? 1 : (S.nnz + 4095) / 4096;
     return (int)std::min<uint64_t>((uint64_t)most, std::max<uint64_t>(want, 1));
 }
 
@@ -600,9 +604,11 @@ int enqueue_single(abfs_graph_s* g, uint32_t source, int32_t* level, int32_t* pa
     // those that may take bottom-up levels: their scans need each column in
     // ascending input-label order, which only the input numbering has
     const bool bu_wanted = p.bottom_up_alpha && !g->directed && g->sorted;
-    const bool rel = w.relabel && p.mode == ABFS_MODE_SUBMATRIX && !sigma && !bu_wanted;
-    const uint32_t bu_ok = (!rel && !g->directed && g->sorted && !sigma) ? 1u : 0u;
     const int most = sync_applies(g->n, g->nnz, p) ? sync_max_ctas(g->device, g->sms) : 0;
+    // (a graph that fits one CTA gains nothing from its relabelled copy)
+    const bool rel = w.relabel && p.mode == ABFS_MODE_SUBMATRIX && !sigma && !bu_wanted &&
+                     !(most > 0 && sync_local(g->n, g->nnz));
+    const uint32_t bu_ok = (!rel && !g->directed && g->sorted && !sigma) ? 1u : 0u;
     if (most > 0) {
         SyncBar* bar = reinterpret_cast<SyncBar*>(reinterpret_cast<char*>(w.d_done) + kBarAt);
         SyncSearch S = make_sync(g, w.base, w.L, bar, source, rel, p);
@@ -613,7 +619,8 @@ int enqueue_single(abfs_graph_s* g, uint32_t source, int32_t* level, int32_t* pa
         S.trace_cap = trace_cap;
         S.bu_alpha = bu_ok ? p.bottom_up_alpha : 0u;
         S.bu_beta = p.bottom_up_beta;
-        CK(launch_sync(S, sync_team_cap(g->nnz, most), s));
+        S.local = !rel && !sigma && !trace && !S.bu_alpha && sync_local(g->n, g->nnz);
+        CK(launch_sync(S, sync_team_cap(S, most), s));
         CK(cudaEventRecord(g->last_use, s));
         g->used = true;
         return ABFS_OK;
@@ -669,6 +676,7 @@ SyncSearch serve_search(abfs_graph_t g, char* base, const Layout& L, SyncBar* ba
     S.parent = reinterpret_cast<uint32_t*>(parent);
     S.ctl = ctl;
     S.hold_units = 0;
+    S.local = sync_local(g->n, g->nnz);
     return S;
 }
 int graph_arrays(abfs_graph_t g, const uint32_t** colptr, const uint32_t** rowidx, uint32_t* n,
@@ -1365,10 +1373,27 @@ int batch_create(const abfs_graph_t* g, const uint32_t* sources, uint32_t count,
     if (sync) {
         std::vector<double> work(ninst);
         std::vector<uint32_t> cap(ninst);
+        std::vector<SyncSearch> searches(ninst);
         for (uint32_t t = 0; t < ninst; ++t) {
             const abfs_graph_s* gt = g[inst[t].gi];
+            SyncSearch& S = searches[t];
+            S = make_sync(gt, b->ws + base[t], L[t], nullptr, hI[t].src, false, p);
+            S.level = hI[t].level;
+            S.parent = hI[t].parent;
+            S.sigma = hI[t].sigma;
+            S.bu_alpha = hI[t].bu_ok ? p.bottom_up_alpha : 0u;
+            S.bu_beta = p.bottom_up_beta;
+            S.ms = hI[t].ms;
+            S.ms_vis = hI[t].ms_vis;
+            S.ms_fr[0] = hI[t].ms_fr[0];
+            S.ms_fr[1] = hI[t].ms_fr[1];
+            S.ms_nx = hI[t].ms_nx;
+            S.ms_src = hI[t].ms_src;
+            S.ms_level = hI[t].ms_level;
+            S.ms_parent = hI[t].ms_parent;
+            S.local = !S.sigma && !S.bu_alpha && !S.ms && sync_local(gt->n, gt->nnz);
             work[t] = sync_work_us(gt->n, gt->nnz, hI[t].ms);
-            cap[t] = (uint32_t)sync_team_cap(gt->nnz, most);
+            cap[t] = (uint32_t)sync_team_cap(S, most);
         }
         const TeamPlan plan = plan_teams(work, cap, most);
         sync_grid = plan.ctas;
@@ -1391,23 +1416,8 @@ int batch_create(const abfs_graph_t* g, const uint32_t* sources, uint32_t count,
         // barriers and the queue's counters start at zero
         std::vector<char> h(o, 0);
         for (uint32_t t = 0; t < ninst; ++t) {
-            const abfs_graph_s* gt = g[inst[t].gi];
-            SyncBar* bar = reinterpret_cast<SyncBar*>(b->d_sync + at_bar + 256 * (size_t)t);
-            SyncSearch S = make_sync(gt, b->ws + base[t], L[t], bar, hI[t].src, false, p);
-            S.level = hI[t].level;
-            S.parent = hI[t].parent;
-            S.sigma = hI[t].sigma;
-            S.bu_alpha = hI[t].bu_ok ? p.bottom_up_alpha : 0u;
-            S.bu_beta = p.bottom_up_beta;
-            S.ms = hI[t].ms;
-            S.ms_vis = hI[t].ms_vis;
-            S.ms_fr[0] = hI[t].ms_fr[0];
-            S.ms_fr[1] = hI[t].ms_fr[1];
-            S.ms_nx = hI[t].ms_nx;
-            S.ms_src = hI[t].ms_src;
-            S.ms_level = hI[t].ms_level;
-            S.ms_parent = hI[t].ms_parent;
-            std::memcpy(h.data() + at_search + sizeof(SyncSearch) * t, &S, sizeof(S));
+            searches[t].bar = reinterpret_cast<SyncBar*>(b->d_sync + at_bar + 256 * (size_t)t);
+            std::memcpy(h.data() + at_search + sizeof(SyncSearch) * t, &searches[t], sizeof(SyncSearch));
         }
         std::memcpy(h.data() + at_off, plan.off.data(), 4 * plan.off.size());
         std::memcpy(h.data() + at_steps, plan.steps.data(), sizeof(SyncStep) * plan.steps.size());

@@ -59,6 +59,10 @@ constexpr uint32_t kChunk = 4;
 constexpr int kStartWords = kUnitMax / kChunk / 32 + 2;
 // Column entries per item of the level-synchronous engine's lists.
 constexpr uint32_t kSyncSeg = 256;
+// Graphs whose searches one CTA holds whole (sync_local.cuh): keys and queue of
+// kLocalN vertices take the 24 KB of its lists; the row indices, 160 KB, and the
+// column pointers fit the L1 beside them.
+constexpr uint32_t kLocalN = 4096, kLocalNnz = 40960;
 // Marker of an unset parent / unclaimed vertex (reads as -1 through int32).
 constexpr uint32_t kUnset = 0xFFFFFFFFu;
 // Weight of a frontier vertex in its level's work space: the chunks that hold
@@ -281,6 +285,7 @@ struct SyncSearch {
     int32_t* const* ms_level;
     int32_t* const* ms_parent;
     uint32_t hold_units;         // test control: arrivals that never come
+    uint32_t local;              // one CTA holds the whole search in shared memory
     // a level of this many entries is wide; the same for frontiers whose items
     // average hub_avg entries or more
     unsigned long long wide_min, wide_hub;
@@ -386,7 +391,8 @@ int grid_for(int sms, const abfs_params& p);
 SyncSearch serve_search(abfs_graph_t g, char* base, const Layout& L, SyncBar* bar, InstCtl* ctl,
                         uint32_t source, int32_t* level, int32_t* parent, const abfs_params& p);
 double sync_work_us(uint32_t n, uint64_t nnz, uint32_t ms);
-int sync_team_cap(uint64_t nnz, int most);
+int sync_team_cap(const SyncSearch& S, int most);
+bool sync_local(uint32_t n, uint64_t nnz);
 int graph_arrays(abfs_graph_t g, const uint32_t** colptr, const uint32_t** rowidx, uint32_t* n,
                  uint64_t* nnz, int* device, int* sms);
 

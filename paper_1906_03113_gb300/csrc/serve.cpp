@@ -193,7 +193,7 @@ cudaError_t serve_describe(abfs_server_s* S, uint32_t i, const Request& rq, size
                                 rq.level, rq.parent, S->cfg.params);
         q.ticket = rq.ticket;
         q.notify = S->d_notify + i;
-        q.cap = (uint32_t)sync_team_cap(q.search.nnz, S->ctas);
+        q.cap = (uint32_t)sync_team_cap(q.search, S->ctas);
         S->h_words[2 + i] = kSlotSubmitted | S->work[rq.g] << kSlotWorkShift;
         return cudaMemcpyAsync(S->d_sync + i, &q, sizeof(SyncSlot), cudaMemcpyHostToDevice, S->cstream);
     }

@@ -2,7 +2,7 @@
 // Part of sync_engine.cu, split by topic; included in order.
 #pragma once
 
-#include "sync_levels.cuh"
+#include "sync_local.cuh"
 
 namespace abfs {
 
@@ -288,6 +288,10 @@ __device__ __forceinline__ bool sync_leave(const SyncSearch& S, const Team& T) {
 template <bool SIG>
 __device__ __forceinline__ bool sync_search(SyncSmem& sm, const SyncSearch& S, const Team& T) {
     const bool lead = threadIdx.x == 0;
+    if (!SIG && S.local && T.expect == 1) {
+        local_search(sm, S);
+        return lead && sync_leave(S, T);
+    }
     unsigned long long items;
     uint32_t k = 0, wide_levels = 0, act = kActThin;
     sync_init(S, T);

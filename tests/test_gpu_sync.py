@@ -177,3 +177,53 @@ def test_serving_teams(slots):
     assert rep["completed"] == 96 and rep["failed"] == 0
     for G in dev:
         G.destroy()
+
+
+def _path(n, extra, seed):
+    """A path over all n vertices in a shuffled order (as many levels as
+    vertices) with `extra` directed chords backwards along it."""
+    rng = np.random.default_rng(seed)
+    order = rng.permutation(n)
+    a = rng.integers(1, n, size=extra)
+    b = (a * rng.random(extra)).astype(np.int64)
+    src = np.concatenate([order[:-1], order[a]])
+    dst = np.concatenate([order[1:], order[b]])
+    return order, synth.from_arcs(n, src.tolist(), dst.tolist(), directed=True)
+
+
+# around the largest graph that one CTA holds whole (4096 vertices, 40960 entries)
+@pytest.mark.parametrize("n,entries", [(1, 0), (2, 1), (33, 70), (1023, 9000), (4095, 40960), (4096, 40960),
+                                       (4096, 40961), (4097, 40000), (1500, 41000)])
+def test_searches_held_by_one_cta(n, entries):
+    if n == 1:
+        g, srcs = synth.from_arcs(1, [], [], directed=False), [0]
+    elif n == 2:
+        g, srcs = synth.from_arcs(2, [0], [1], directed=True), [0, 1]
+    else:
+        order, g = _path(n, 2 * entries, 51)
+        while g.nnz > entries:  # duplicates merge: thin out to the exact count
+            keep = np.sort(np.random.default_rng(52).permutation(g.nnz)[:entries])
+            col = np.repeat(np.arange(n), g.degrees())[keep]
+            g = synth.from_arcs(n, col.tolist(), np.asarray(g.rowidx)[keep].tolist(), directed=True)
+        assert g.nnz == entries or entries > 40960 or n < 1024
+        srcs = [int(order[0]), int(order[n // 2]), int(order[-1])]
+    G = abfs.graph_create(g.colptr, g.rowidx, directed=g.directed)
+    deg = g.degrees()
+    chain = _path(n, 0, 53) if n > 2 else None
+    for s in srcs:
+        lo, po = oracle.bfs(g, s)
+        lev, par, st = abfs.run(G, s, stats=True)
+        assert np.array_equal(lev.cpu().numpy(), lo) and np.array_equal(par.cpu().numpy(), po), s
+        assert st["reached"] == int((lo >= 0).sum()) and st["levels"] == int(lo.max()) + 1
+        assert st["nnz_reached"] == int(deg[lo >= 0].sum()) == st["entries_read"]
+    G.destroy()
+    if chain:
+        order, g = chain
+        G = abfs.graph_create(g.colptr, g.rowidx, directed=True)
+        lo, po = oracle.bfs(g, int(order[0]))
+        levels, parents, status = abfs.run_batch([G, G], [int(order[0])] * 2)
+        torch.cuda.synchronize()
+        assert status == [0, 0] and int(lo.max()) == n - 1
+        for lev, par in zip(levels, parents):
+            assert np.array_equal(lev.cpu().numpy(), lo) and np.array_equal(par.cpu().numpy(), po)
+        G.destroy()
