@@ -86,31 +86,41 @@ __device__ __noinline__ void sync_outputs(const SyncSearch& S, const Team& T) {
     }
 }
 
-// The team's share of level 0's list: the items of the source's column.
+// The team's share of level 0's list: an even part of the source's column each,
+// so that the rows it wins -- often hubs, on an R-MAT graph -- are spread over
+// the CTAs from the start (they were one CTA's, and evened out before level 1).
 __device__ __forceinline__ void sync_source(SyncSmem& sm, const SyncSearch& S, const Team& T,
                                             unsigned long long& items) {
     const uint32_t cb = ld_ro(S.colptr + S.src);
     const uint32_t len = ld_ro(S.colptr + S.src + 1) - cb;
     items = items_of(cb, len);
-    const uint32_t ni = (uint32_t)items;  // (at most 2^24: 32 bits hold the products)
-    const uint32_t lo = ni * T.rank / T.size, hi = ni * (T.rank + 1) / T.size;
-    // a column too long for the team's lists starts in the global list
-    const bool global = items > (unsigned long long)T.size * kThinCap;
-    for (uint32_t i = lo + threadIdx.x; i < hi; i += kSyncThreads) {
-        uint32_t b, l;
-        item_at(cb, len, i, b, l);
-        if (global) {
+    // a column too long for the team's lists starts in the global list, in
+    // items shared out evenly
+    const bool global = items > (unsigned long long)T.size * (kThinCap - 1);
+    uint32_t mine = 0;
+    if (global) {
+        const uint32_t ni = (uint32_t)items;  // (at most 2^24: 32 bits hold the products)
+        for (uint32_t i = ni * T.rank / T.size + threadIdx.x; i < ni * (T.rank + 1) / T.size; i += kSyncThreads) {
+            uint32_t b, l;
+            item_at(cb, len, i, b, l);
             list_put(S, 0, i, S.src_label, b, l);
-        } else {
-            sm.ij[0][i - lo] = S.src_label;
-            sm.ib[0][i - lo] = b;
-            sm.il[0][i - lo] = l;
+        }
+    } else {
+        const uint32_t per = (len + T.size - 1) / T.size;
+        const uint32_t lo = min(len, per * T.rank), part = min(len - lo, per);
+        mine = items_of(cb + lo, part);
+        for (uint32_t i = threadIdx.x; i < mine; i += kSyncThreads) {
+            uint32_t b, l;
+            item_at(cb + lo, part, i, b, l);
+            sm.ij[0][i] = S.src_label;
+            sm.ib[0][i] = b;
+            sm.il[0][i] = l;
         }
     }
     if (threadIdx.x == 0) {
         sm.step = sm.tick = 0;
         sm.word[0] = sm.word[1] = sm.aux[0] = sm.aux[1] = 0;
-        sm.app[0][0] = global ? 0u : hi - lo;
+        sm.app[0][0] = mine;
         sm.app[0][1] = ~0u;  // entries: not known
         sm.app[1][0] = sm.app[1][1] = 0;
         sm.verts = sm.ent = 0;
@@ -298,7 +308,7 @@ __device__ __forceinline__ bool sync_search(SyncSmem& sm, const SyncSearch& S, c
     sync_source(sm, S, T, items);
     if (!team_sync(sm, S, T)) act = kActFailed;
     else if (items == 0) act = kActDone;
-    else if (items > (unsigned long long)T.size * kThinCap) {
+    else if (items > (unsigned long long)T.size * (kThinCap - 1)) {
         sync_bitmaps(S, T, 0);
         act = team_sync(sm, S, T) ? kActWide : kActFailed;
         if (lead) sm.items = items;
