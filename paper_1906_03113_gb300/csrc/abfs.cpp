@@ -576,15 +576,6 @@ SyncSearch make_sync(const abfs_graph_s* g, char* base, const Layout& L, SyncBar
     }
     S.ctl = reinterpret_cast<InstCtl*>(base + L.ctl);
     S.bar = bar;
-    // A wide level costs a bitmap (8 bytes per vertex), an extraction and a
-    // barrier more than a thin one and saves a returned 64-bit atomic per entry.
-    // Those atomics queue where many columns share hub rows, which a frontier
-    // of columns well above the mean is a sign of (undirected graphs): R-MAT of scale 16, 1.2 M
-    // entries, 150 us with its hub levels thin, 75 us wide.  Without hubs thin
-    // levels stay ahead longer: ER of 2^18 vertices of degree 8, 85 us thin, 100 us
-    // with the lower line.
-    S.wide_min = (3ull << 19) + g->n;
-    S.wide_hub = (1ull << 18) + g->n / 4;
     S.hub_avg = (uint32_t)std::max<uint64_t>(8, 3 * g->nnz / (2ull * g->n));
     S.timeout_ns = (unsigned long long)p.timeout_ms * 1000000ull;
     S.hold_units = test_hold_units();

@@ -286,10 +286,7 @@ struct SyncSearch {
     int32_t* const* ms_parent;
     uint32_t hold_units;         // test control: arrivals that never come
     uint32_t local;              // one CTA holds the whole search in shared memory
-    // a level of this many entries is wide; the same for frontiers whose items
-    // average hub_avg entries or more
-    unsigned long long wide_min, wide_hub;
-    uint32_t hub_avg;
+    uint32_t hub_avg;            // a frontier whose items average this many entries has hubs
     unsigned long long timeout_ns;
 };
 

@@ -36,7 +36,7 @@ constexpr unsigned long long kKeyUnset = ~0ull;
 // exact totals follow with the next barrier where they matter).  Beside it,
 // for the hybrid and traces: [vertices : 31][column entries : 33].
 constexpr uint32_t kArriveShift = 56, kFullShift = 48, kHeavyShift = 40, kItemShift = 19;
-constexpr uint32_t kEntUnit = 64, kEntClamp = 2184, kItemClamp = 8191;
+constexpr uint32_t kEntUnit = 64, kItemClamp = 8191;
 constexpr uint32_t kAuxShift = 33;
 
 // What a level is followed by; the team's CTAs agree on it because they decide
@@ -67,6 +67,7 @@ struct SyncSmem {
     // thread 0's state of the search
     uint32_t lim;                     // a list of more weight is heavy
     float weight;                     // of the current level's lists
+    uint32_t ent_clamp;               // a CTA's largest part of a thin word's entries
     uint32_t bu;
     unsigned long long nf, entries, seen;
     unsigned long long st_read, st_unmasked, st_verts, st_ent;

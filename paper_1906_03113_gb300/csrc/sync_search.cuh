@@ -125,6 +125,7 @@ __device__ __forceinline__ void sync_source(SyncSmem& sm, const SyncSearch& S, c
         sm.app[1][0] = sm.app[1][1] = 0;
         sm.verts = sm.ent = 0;
         sm.lim = 1024;
+        sm.ent_clamp = ((1u << kItemShift) - 1u) / T.size;
         sm.weight = (float)len + 4.f * (float)items + 1.f;
         sm.bu = 0;
         sm.nf = 1;
@@ -156,10 +157,23 @@ __device__ __forceinline__ uint32_t tot_ent(unsigned long long tot) {
     return ((uint32_t)tot & ((1u << kItemShift) - 1u)) * kEntUnit;
 }
 
-// Entries from which the level of a frontier of `items` items is wide.
-__device__ __forceinline__ unsigned long long wide_line(const SyncSearch& S, unsigned long long items,
-                                                        unsigned long long ent) {
-    return ent >= S.hub_avg * items ? S.wide_hub : S.wide_min;
+// Entries from which the level of a frontier of `items` items is wide.  A wide
+// level costs a bitmap (8 bytes per vertex), an extraction and a barrier more
+// than a thin one, about 10 us and a part in n, and saves a returned 64-bit
+// atomic per entry, so the line grows with the team (a line fixed for the whole
+// GPU: a batch of 32 graphs on teams of a few CTAs, 340 us instead of 317).  Those
+// atomics queue where many columns share hub rows, which a frontier of columns
+// well above the mean is a sign of (undirected graphs): R-MAT of scale 16, 1.2 M
+// entries, 150 us with its hub levels thin, 75 us wide.  Without hubs thin levels
+// stay ahead longer: ER of 150 000 vertices, degree 16, 82 us, 98 us with half
+// the line.
+constexpr uint32_t kWidePerCta = 10240, kHubPerCta = 1728;
+__device__ __forceinline__ uint32_t hub_line(const SyncSearch& S, const Team& T) {
+    return kHubPerCta * T.size + S.n / 4;
+}
+__device__ __forceinline__ uint32_t wide_line(const SyncSearch& S, const Team& T, unsigned long long items,
+                                              unsigned long long ent) {
+    return ent >= S.hub_avg * items ? hub_line(S, T) : kWidePerCta * T.size + S.n;
 }
 
 // Thread 0 after the barrier that ended a thin level (tot: the barrier's
@@ -170,7 +184,7 @@ __device__ __forceinline__ uint32_t thin_next(SyncSmem& sm, const SyncSearch& S,
     const uint32_t items = tot_items(tot), ent = tot_ent(tot);
     sm.items = items;
     if (items == 0) return kActDone;
-    if (flags == 0 && ent < S.wide_hub && !want_aux) return kActThin;
+    if (flags == 0 && ent < hub_line(S, T) && !want_aux) return kActThin;
     if (tot == ~0ull) return kActFailed;
     if (want_aux) {
         sm.nf = items;
@@ -182,7 +196,7 @@ __device__ __forceinline__ uint32_t thin_next(SyncSmem& sm, const SyncSearch& S,
             if (sm.bu) return kActBottomUp;
         }
     }
-    if (ent >= wide_line(S, items, ent) || items > T.size * kThinCap) return kActWide;
+    if (ent >= wide_line(S, T, items, ent) || items > T.size * kThinCap) return kActWide;
     // a list is full, or a few CTAs hold much more than the others
     const uint32_t heavy = flags & 0xFFu;
     if ((flags >> 8) || (heavy && 2 * heavy <= T.size)) {
@@ -217,7 +231,7 @@ __device__ __noinline__ uint32_t thin_run(SyncSmem& sm, const SyncSearch& S, con
         unsigned long long add = 0, aux = 0;
         if (lead) {
             const uint32_t c = sm.app[cur ^ 1][0], e = sm.app[cur ^ 1][1];
-            add = (unsigned long long)min(c, kItemClamp) << kItemShift | min(e / kEntUnit, kEntClamp);
+            add = (unsigned long long)min(c, kItemClamp) << kItemShift | min(e / kEntUnit, sm.ent_clamp);
             if (list_weight(c, e) > sm.lim) add += 1ull << kHeavyShift;
             if (c > kThinCap) add += 1ull << kFullShift;
             aux = e;
@@ -266,7 +280,7 @@ __device__ __forceinline__ uint32_t wide_next(SyncSmem& sm, const SyncSearch& S,
         if (sm.bu) return kActBottomUp;
     }
     if (bottom_up || tot > (unsigned long long)T.size * kThinCap ||
-        sm.entries >= wide_line(S, tot, sm.entries) / 2)
+        sm.entries >= wide_line(S, T, tot, sm.entries) / 2)
         return kActWide;
     heavy_limit(sm, T, (float)tot, (float)sm.entries);
     return kActSlice;
@@ -329,7 +343,7 @@ __device__ __forceinline__ bool sync_search(SyncSmem& sm, const SyncSearch& S, c
                 } else if (act == kActEven) {
                     // exact totals now: the thin level's were clamped per CTA
                     const unsigned long long all = sm.items, entries = sm.entries;
-                    if (all <= (unsigned long long)T.size * kThinCap && entries < wide_line(S, all, entries)) {
+                    if (all <= (unsigned long long)T.size * kThinCap && entries < wide_line(S, T, all, entries)) {
                         list_slice(sm, S, T, p, p, all);
                         // a failed append leaves the list incomplete
                         if (lead) sm.act = ld_relaxed(&S.ctl->err) ? kActFailed : kActThin;
