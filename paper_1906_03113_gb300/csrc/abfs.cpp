@@ -217,15 +217,20 @@ bool sync_applies(uint32_t n, uint64_t nnz, const abfs_params& p) {
            p.cluster_max == d.cluster_max && p.cluster_edges == d.cluster_edges;
 }
 
-// One CTA's time for a search: 0.9 ns an entry and 1.5 ns a vertex; a
-// multi-source search (ms sources) 2 ns an entry and 0.06 ns more per source.
-double sync_work_us(uint32_t n, uint64_t nnz, uint32_t ms) {
-    return (ms ? 2e-3 + 6e-5 * ms : 0.9e-3) * (double)nnz + 1.5e-3 * n * (ms ? 1.0 + ms / 8.0 : 1.0);
-}
-
 // Whether one CTA can hold a search whole (sync_local.cuh): its keys in shared
 // memory, its graph in the L1.
 bool sync_local(uint32_t n, uint64_t nnz) { return n <= kLocalN && nnz <= kLocalNnz; }
+
+// One CTA's time for a search: 0.9 ns an entry and 4 ns a vertex (fitted to the
+// searches of a batch of 128), half an entry's where the visited bitmap is held in
+// shared memory, less where the whole search is; a multi-source search (ms
+// sources) 2 ns an entry and 0.06 ns more per source.  (With 1.5 ns a vertex the
+// batch waited for one sparse graph on two CTAs: 826 us instead of 611.)
+double sync_work_us(uint32_t n, uint64_t nnz, uint32_t ms) {
+    if (ms) return (2e-3 + 6e-5 * ms) * (double)nnz + 1.5e-3 * n * (1.0 + ms / 8.0);
+    if (sync_local(n, nnz)) return 5.0 + 0.3e-3 * (double)nnz;
+    return (n <= kBitsN ? 0.45e-3 : 0.9e-3) * (double)nnz + 4e-3 * n;
+}
 
 // The largest useful team of a search: a few thousand entries per CTA.  Up to
 // 16 384 entries one CTA, without barriers between CTAs, is fastest.

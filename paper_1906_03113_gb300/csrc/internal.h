@@ -63,6 +63,8 @@ constexpr uint32_t kSyncSeg = 256;
 // kLocalN vertices take the 24 KB of its lists; the row indices, 160 KB, and the
 // column pointers fit the L1 beside them.
 constexpr uint32_t kLocalN = 4096, kLocalNnz = 40960;
+// Graphs whose visited bitmap takes the place of those lists in wide levels.
+constexpr uint32_t kBitsN = 32 * 6144;
 // Marker of an unset parent / unclaimed vertex (reads as -1 through int32).
 constexpr uint32_t kUnset = 0xFFFFFFFFu;
 // Weight of a frontier vertex in its level's work space: the chunks that hold

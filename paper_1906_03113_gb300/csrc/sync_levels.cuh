@@ -243,7 +243,12 @@ enum WideKind : int {
                       // that it lacks, in the next-bit masks
 };
 
-template <int KIND>
+// BITS: the graph has at most kBitsN vertices, and its bitmap is copied into the
+// place of the thin levels' lists, which a wide level does not need: a test then
+// costs a bank conflict or two instead of a cycle per entry for its cache line.
+static_assert(kBitsN / 8 == sizeof(SyncSmem::ij) + sizeof(SyncSmem::ib) + sizeof(SyncSmem::il), "the lists' bytes");
+
+template <int KIND, bool BITS>
 __device__ __noinline__ void wide_expand(SyncSmem& sm, const SyncSearch& S, const Team& T, uint32_t k,
                                          unsigned long long items) {
     const uint32_t lane = threadIdx.x & 31;
@@ -262,7 +267,11 @@ __device__ __noinline__ void wide_expand(SyncSmem& sm, const SyncSearch& S, cons
     const uint32_t run = max(1u, min(min(32u, four), n / (4u * W)));
     const uint32_t runs = (n + run - 1) / run;
     const uint64_t pol = evict_first_policy();
-    const uint32_t* const bm = S.bm;
+    const uint32_t* const bm = BITS ? &sm.ij[0][0] : S.bm;
+    if (BITS) {
+        for (uint32_t w = threadIdx.x; w < S.nwords; w += kSyncThreads) (&sm.ij[0][0])[w] = ld_l2(S.bm + w);
+        __syncthreads();
+    }
     uint32_t* const klo = reinterpret_cast<uint32_t*>(S.key);
     SyncTally t;
     // the items of the run after the current one

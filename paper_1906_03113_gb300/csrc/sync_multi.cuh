@@ -301,7 +301,7 @@ __device__ __forceinline__ void ms_search(SyncSmem& sm, const SyncSearch& S, con
             if (T.rank == 0 && lead) st_relaxed(&S.bar->lcnt[k & 1], 0u);
             if (lead) sm.entries = ent;
             __syncthreads();
-            wide_expand<kWideMulti>(sm, S, T, k, items);
+            wide_expand<kWideMulti, false>(sm, S, T, k, items);
             ok = team_sync(sm, S, T);
             if (!ok) break;
             if (lead) sm.tick = 0;

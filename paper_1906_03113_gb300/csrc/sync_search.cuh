@@ -382,7 +382,9 @@ __device__ __forceinline__ bool sync_search(SyncSmem& sm, const SyncSearch& S, c
             if (up) {
                 sync_bottom_up(sm, S, T, k);
             } else {
-                wide_expand<SIG ? kWideCounts : kWidePlain>(sm, S, T, k, sm.items);
+                constexpr int kind = SIG ? kWideCounts : kWidePlain;
+                if (S.n <= kBitsN) wide_expand<kind, true>(sm, S, T, k, sm.items);
+                else wide_expand<kind, false>(sm, S, T, k, sm.items);
                 if (!team_sync(sm, S, T)) {
                     act = kActFailed;
                     break;
