@@ -227,3 +227,27 @@ def test_searches_held_by_one_cta(n, entries):
         for lev, par in zip(levels, parents):
             assert np.array_equal(lev.cpu().numpy(), lo) and np.array_equal(par.cpu().numpy(), po)
         G.destroy()
+
+
+@pytest.mark.parametrize("n", [196607, 196608, 196609])
+def test_bitmap_in_shared_memory_at_its_limit(n):
+    """Wide levels around the largest graph whose bitmap fits beside the lists,
+    on a large team, on the small teams of a batch, and with path counts."""
+    rng = np.random.default_rng(n)
+    # two dense halves of the vertex range, bridged: rows on the first and last words
+    src = rng.integers(n, size=6 * n)
+    dst = np.concatenate([rng.integers(n, size=5 * n), n - 1 - rng.integers(64, size=n)])
+    g = synth.from_arcs(n, src.tolist(), dst.tolist(), directed=False)
+    G = abfs.graph_create(g.colptr, g.rowidx, directed=False)
+    lo, po = oracle.bfs(g, n - 1)
+    lev, par = abfs.run(G, n - 1)
+    assert np.array_equal(lev.cpu().numpy(), lo) and np.array_equal(par.cpu().numpy(), po)
+    lev, par, sig = abfs.run_counts(G, n - 1)
+    assert np.array_equal(lev.cpu().numpy(), lo) and np.array_equal(par.cpu().numpy(), po)
+    assert np.array_equal(sig.cpu().numpy().view(np.uint64), oracle.path_counts(g, n - 1))
+    levels, parents, status = abfs.run_batch([G] * 7, [n - 1] * 7)
+    torch.cuda.synchronize()
+    assert status == [0] * 7
+    for lev, par in zip(levels, parents):
+        assert np.array_equal(lev.cpu().numpy(), lo) and np.array_equal(par.cpu().numpy(), po)
+    G.destroy()
