@@ -478,20 +478,20 @@ __device__ __noinline__ void sync_extract(SyncSmem& sm, const SyncSearch& S, con
     const uint32_t g0 = (warp * T.size + T.rank) * Q;  // groups of Q words, round robin
     uint32_t* const khi = reinterpret_cast<uint32_t*>(S.key) + 1;
     uint32_t verts = 0, entries = 0, mine = 0;
+    // this lane's word of the group at wb, loaded a group ahead (a batch of 128
+    // graphs 608 -> 598 us)
+    auto load = [&](const uint32_t* bits, uint32_t wb) {
+        return lane < Q && wb < S.nwords && lane < S.nwords - wb ? ld_l2(bits + wb + lane) : 0u;
+    };
+    const uint32_t* const from = FROM_KEYS ? S.bm : S.fbm[pn];
+    uint32_t ahead = MASKS ? 0u : load(from, g0);
 #pragma unroll 1
     for (uint32_t wb = g0; wb < S.nwords; wb += Q * W) {
         const bool own = lane < Q && wb + lane < S.nwords;
-        uint32_t word = 0, seen = 0, add = 0;
-        if (own) {
-            if (FROM_KEYS) {
-                seen = ld_l2(S.bm + wb + lane);
-                word = ~seen & word_mask(S, wb + lane);
-            } else if (MASKS) {
-                word = word_mask(S, wb + lane);
-            } else {
-                word = ld_l2(S.fbm[pn] + wb + lane);
-            }
-        }
+        const uint32_t seen = ahead;
+        uint32_t word = 0, add = 0;
+        if (!MASKS) ahead = load(from, wb + Q * W);
+        if (own) word = FROM_KEYS ? ~seen & word_mask(S, wb + lane) : MASKS ? word_mask(S, wb + lane) : seen;
         const unsigned long long v0 = (unsigned long long)wb * 32 + lane;
         bool fresh[Q];
 #pragma unroll
@@ -544,10 +544,12 @@ __device__ __noinline__ void sync_extract(SyncSmem& sm, const SyncSearch& S, con
     __syncthreads();
     if (!wt) return;
     uint32_t at = sm.wpre[warp];
+    // (this lane's own words of the first pass)
+    ahead = load(S.fbm[pn], g0);
 #pragma unroll 1
     for (uint32_t wb = g0; wb < S.nwords; wb += Q * W) {
-        // (this lane's own words of the first pass)
-        const uint32_t word = lane < Q && wb + lane < S.nwords ? ld_l2(S.fbm[pn] + wb + lane) : 0u;
+        const uint32_t word = ahead;
+        ahead = load(S.fbm[pn], wb + Q * W);
         if (!__any_sync(0xFFFFFFFFu, word != 0)) continue;
         const unsigned long long v0 = (unsigned long long)wb * 32 + lane;
         uint32_t cb[Q], len[Q];
