@@ -168,6 +168,12 @@ EngineArgs serve_args(abfs_server_s* S) {
     return a;
 }
 
+// Servers with a graph above either size run on the unit scheduler: a team holds
+// its CTAs for a whole search, so a few large or long searches keep the others
+// waiting, where the scheduler's CTAs move from search to search.
+constexpr uint32_t kTeamServeN = 1u << 20;
+constexpr uint64_t kTeamServeNnz = 1ull << 25;
+
 // Device launch that serves the slots.
 cudaError_t serve_launch(abfs_server_s* S) {
     if (!S->ctas) return launch_engine(serve_args(S), grid_for(S->sms, S->cfg.params), S->kstream);
@@ -345,6 +351,15 @@ extern "C" int abfs_serve_start(const abfs_graph_t* g, uint32_t ngraphs, const a
             return ABFS_ERR_INVALID_ARG;
         }
         if (i == 0 && sync_applies(n, nnz, c.params)) S->ctas = sync_max_ctas(dev, sms);
+        if (n > kTeamServeN || nnz > kTeamServeNnz) S->ctas = 0;
+    }
+    for (uint32_t i = 0; i < ngraphs; ++i) {
+        const uint32_t* cp;
+        const uint32_t* ri;
+        uint32_t n;
+        uint64_t nnz;
+        int dev, sms;
+        graph_arrays(g[i], &cp, &ri, &n, &nnz, &dev, &sms);
         S->layouts.push_back(layout_for(n, nnz, c.params, 0, false, S->ctas > 0));
         S->work.push_back((uint32_t)std::min(8.0 * sync_work_us(n, nnz, 0) + 1.0, 16777215.0));
         largest = std::max(largest, S->layouts.back().total);
