@@ -77,8 +77,8 @@ typedef enum {
  * Two engines run searches, with the same results.  With the default values
  * of the scheduling knobs (tile, unit_entries, narrow_*, ctas_per_sm,
  * claim_scan, cluster_*), submatrix searches without a physical shrink --
- * single ones, batches and serving -- run on the level-synchronous engine,
- * where a team of CTAs runs one search at a time and none of those knobs
+ * single ones, batches, and serving of graphs of up to 2^20 vertices and 2^25
+ * entries -- run on the level-synchronous engine, where a team of CTAs runs one search at a time and none of those knobs
  * means anything.  A search that sets any of them, the comparator, shrinks and
  * abfs_run_static run on the unit scheduler, whose knobs they
  * are. */
