@@ -492,6 +492,16 @@ int abfs_set_allocator(void* (*alloc)(size_t bytes, void* ctx), void (*free_fn)(
  */
 int abfs_test_hold_first_phase(uint32_t extra_units);
 
+/*
+ * The same control for a later wait of the level-synchronous engine: a search
+ * passes its first `barriers` team barriers and then waits, at the next one,
+ * for extra_arrivals more arrivals than it has CTAs (at most 255 in all), so
+ * that the time-out of every wait of a search can be tested.  A search with
+ * fewer barriers ends normally.  On the unit scheduler `barriers` means
+ * nothing.  abfs_test_hold_first_phase(x) is abfs_test_hold_barrier(x, 0).
+ */
+int abfs_test_hold_barrier(uint32_t extra_arrivals, uint32_t barriers);
+
 /* On-chip ceilings of the expand step, measured on the current device. */
 typedef struct {
     uint32_t words;     /* array size in 32-bit words (2^words_log2) */

@@ -584,6 +584,7 @@ SyncSearch make_sync(const abfs_graph_s* g, char* base, const Layout& L, SyncBar
     S.hub_avg = (uint32_t)std::max<uint64_t>(8, 3 * g->nnz / (2ull * g->n));
     S.timeout_ns = (unsigned long long)p.timeout_ms * 1000000ull;
     S.hold_units = test_hold_units();
+    S.hold_from = test_hold_from();
     return S;
 }
 
@@ -1744,19 +1745,25 @@ extern "C" int abfs_set_allocator(void* (*alloc)(size_t, void*), void (*free_fn)
 extern "C" const char* abfs_last_cuda_error(void) { return g_last_cuda_error.c_str(); }
 
 // ---------------------------------------------------------------------------
-// test control: a first phase that never completes
+// test controls: a first phase, or a barrier, that never completes
 // ---------------------------------------------------------------------------
 
 namespace {
-std::atomic<uint32_t> g_hold_units{0};
+std::atomic<uint32_t> g_hold_units{0}, g_hold_from{0};
 }  // namespace
 
 namespace abfs {
 uint32_t test_hold_units() { return g_hold_units.load(std::memory_order_relaxed); }
+uint32_t test_hold_from() { return g_hold_from.load(std::memory_order_relaxed); }
 }  // namespace abfs
 
 extern "C" int abfs_test_hold_first_phase(uint32_t extra_units) {
-    g_hold_units.store(extra_units, std::memory_order_relaxed);
+    return abfs_test_hold_barrier(extra_units, 0);
+}
+
+extern "C" int abfs_test_hold_barrier(uint32_t extra_arrivals, uint32_t barriers) {
+    g_hold_from.store(barriers, std::memory_order_relaxed);
+    g_hold_units.store(extra_arrivals, std::memory_order_relaxed);
     return ABFS_OK;
 }
 

@@ -286,7 +286,8 @@ struct SyncSearch {
     const uint32_t* ms_src;
     int32_t* const* ms_level;
     int32_t* const* ms_parent;
-    uint32_t hold_units;         // test control: arrivals that never come
+    uint32_t hold_units;         // test control: arrivals that never come ...
+    uint32_t hold_from;          // ... at barriers from this one on
     uint32_t local;              // one CTA holds the whole search in shared memory
     uint32_t hub_avg;            // a frontier whose items average this many entries has hubs
     unsigned long long timeout_ns;
@@ -395,8 +396,11 @@ bool sync_local(uint32_t n, uint64_t nnz);
 int graph_arrays(abfs_graph_t g, const uint32_t** colptr, const uint32_t** rowidx, uint32_t* n,
                  uint64_t* nnz, int* device, int* sms);
 
-// Test control set by abfs_test_hold_first_phase (abfs.cpp).
+// Test control set by abfs_test_hold_first_phase and abfs_test_hold_barrier (abfs.cpp).
 uint32_t test_hold_units();
+// Barriers a held search of the level-synchronous engine passes first
+// (abfs_test_hold_barrier).
+uint32_t test_hold_from();
 
 // Launch helpers implemented in engine.cu.
 cudaError_t launch_put_inst(const Inst& inst, Inst* dst, cudaStream_t s);

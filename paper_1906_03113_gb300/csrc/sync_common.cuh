@@ -63,6 +63,7 @@ struct SyncSmem {
     uint32_t base;
     uint32_t wsum[kSyncWarps], wpre[kSyncWarps];
     uint32_t act;                     // SyncAct after the last barrier
+    uint32_t passed;                  // whether the last team_sync was passed (written there only)
     unsigned long long items;         // the next level's items
     // thread 0's state of the search
     uint32_t lim;                     // a list of more weight is heavy
@@ -84,7 +85,7 @@ struct SyncSmem {
 // A CTA's place in its team.
 struct Team {
     uint32_t rank, size;
-    uint32_t expect;  // arrivals a barrier waits for (more than size only in the held test)
+    uint32_t expect;  // arrivals a barrier waits for (more than size only in the held tests)
 };
 
 // Counters of a thread over a whole search.
@@ -145,6 +146,8 @@ __device__ __forceinline__ unsigned long long bar_poll(SyncSmem& sm, const SyncS
                                                        unsigned long long add, unsigned long long& aux) {
     if (T.expect == 1) return add;
     const uint32_t b = sm.step & 1u;
+    // (held tests: from barrier hold_from on)
+    const uint32_t expect = T.expect != T.size && sm.step < S.hold_from ? T.size : T.expect;
     ++sm.step;
     unsigned long long* w = &S.bar->word[b];
     const unsigned long long before = sm.word[b];
@@ -152,7 +155,7 @@ __device__ __forceinline__ unsigned long long bar_poll(SyncSmem& sm, const SyncS
     uint64_t t0 = 0;
     for (uint32_t spin = 0;; ++spin) {
         v = ld_relaxed64(w);
-        if ((uint32_t)((v - before) >> kArriveShift) == T.expect) break;
+        if ((uint32_t)((v - before) >> kArriveShift) == expect) break;
         // reading %globaltimer is slow: the clock starts after 4096 polls
         if ((spin & 4095u) == 4095u) {
             const uint64_t now = globaltimer();
@@ -182,16 +185,20 @@ __device__ __forceinline__ unsigned long long bar_wait(SyncSmem& sm, const SyncS
 
 // A plain full barrier; the sums of `add` and `ent` (thread 0's) reach sm.items
 // and sm.entries.
-// Returns false when the bounded wait ran out.  Whole CTA.
+// Returns false when the bounded wait ran out.  The verdict has a word of its
+// own: callers go on to write sm.items without another __syncthreads, and every
+// thread has to read the same verdict.  Whole CTA.
 __device__ __forceinline__ bool team_sync(SyncSmem& sm, const SyncSearch& S, const Team& T,
                                           unsigned long long add = 0, unsigned long long ent = 0) {
     __syncthreads();
     if (threadIdx.x == 0) {
-        sm.items = bar_wait<true>(sm, S, T, add, ent);
+        const unsigned long long tot = bar_wait<true>(sm, S, T, add, ent);
+        sm.items = tot;
         sm.entries = ent;
+        sm.passed = tot != ~0ull;
     }
     __syncthreads();
-    return sm.items != ~0ull;
+    return sm.passed != 0;
 }
 
 // Items of the column [beg, beg + len).
