@@ -128,7 +128,10 @@ __device__ __forceinline__ void red_add_release64(unsigned long long* p, unsigne
 // a key word whose returned value its CTA has used before it arrived, so it
 // has been performed at the L2, and everything the next level does with a key
 // word is another atomic or a strong load there.  The release and the acquire
-// cost 1.1 + 0.8 thousand cycles of a thin level's 8.4.
+// cost 1.1 + 0.8 thousand cycles of a thin level's 8.4.  The same holds for the
+// list counters lcnt: a thin level reserves in them by atomics, and whoever
+// resets one does it before a FULL barrier or by an atomic whose result it has
+// used.
 template <bool FULL>
 __device__ __forceinline__ void bar_arrive(SyncSmem& sm, const SyncSearch& S, const Team& T,
                                            unsigned long long add, unsigned long long aux) {
@@ -253,8 +256,11 @@ __device__ __noinline__ void list_slice(SyncSmem& sm, const SyncSearch& S, const
     if (threadIdx.x == 0) {
         sm.app[q][0] = c;
         sm.app[q][1] = ~0u;  // entries: not known
-        // every reservation in this list was made before the last barrier
-        if (T.rank == 0) st_relaxed(&S.bar->lcnt[p], 0u);
+        // Every reservation in this list was made before the last barrier.  The
+        // next barrier may be a thin level's, which orders no stores: the reset
+        // is an atomic whose returned value this thread has stored before the
+        // CTA's arrival, so it is performed before any CTA reserves again.
+        if (T.rank == 0) sm.base = atomicExch(&S.bar->lcnt[p], 0u);
     }
     __syncthreads();
 }

@@ -135,3 +135,25 @@ def test_each_wait_of_a_multi_source_search_times_out(lib):
 
     _hold_each_barrier(lib, search, exact, 4)
     G.destroy()
+
+
+@pytest.mark.parametrize("layers,mids", [(400, 1500), (150, 5000), (3, 60000)])
+def test_lists_that_overflow_right_after_a_slice(lib, layers, mids):
+    """Layers of one hub, its `mids` rows and the next hub: the hub's rows
+    overflow one CTA's list and are evened out through the global list, and the
+    level after that, behind a thin level's barrier, the next hub's rows
+    overflow into the same list again."""
+    step = mids + 1
+    hub = np.arange(layers, dtype=np.int64) * step
+    mid = hub[:, None] + np.arange(1, step)
+    src = np.concatenate([np.repeat(hub, mids), mid[:-1].ravel()])
+    dst = np.concatenate([mid.ravel(), np.repeat(hub[1:], mids)])
+    g = synth.from_arcs(layers * step, src.tolist(), dst.tolist(), directed=True)
+    G = abfs.graph_create(g.colptr, g.rowidx, directed=True)
+    lo, po = oracle.bfs(g, 0)
+    want = torch.from_numpy(lo).cuda(), torch.from_numpy(po).cuda()
+    for rep in range(10):
+        lev, par, st = abfs.run(G, 0, stats=True)
+        assert torch.equal(lev, want[0]) and torch.equal(par, want[1]), rep
+        assert st["reached"] == g.n and st["nnz_reached"] == g.nnz
+    G.destroy()
