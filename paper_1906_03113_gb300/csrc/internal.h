@@ -323,7 +323,7 @@ struct SyncServe {
     const SyncSlot* slots;
     uint32_t* state;             // per slot: SlotState in 8 bits, above it the query's work in units
     uint32_t* claim;             // 1 while a CTA claims a query and opens its team
-    // per slot, the team being formed: [sequence : 32][open : 1][wanted : 8][joined : 8]
+    // per slot, the team being formed (serve_team.h)
     unsigned long long* join;
     const uint32_t* stop_flag;
     unsigned long long* heartbeat;

@@ -20,6 +20,7 @@
 
 #include "sync_multi.cuh"
 #include "internal.h"
+#include "serve_team.h"
 
 namespace abfs {
 
@@ -88,31 +89,21 @@ __global__ void __launch_bounds__(kSyncThreads, 1) sync_batch_kernel(const __gri
 // that come free together do not each open a team that nobody is left to join.
 // (Counting on free CTAs alone left large queries on one CTA whenever the
 // launch was busy: 256 queries on 16 graphs 3.6 -> 6.7 ms.)
-constexpr unsigned long long kJoinOpen = 1ull << 16;
 constexpr unsigned long long kJoinWaitNs = 150000, kJoinWaitMinNs = 5000;
-constexpr uint64_t kMemberWaitNs = 1000000000ull;
+constexpr unsigned long long kMemberWaitNs = 1000000000ull;
 
 struct ServeCmd {
     uint32_t what;  // 0: nothing to do, 1: run slot q, 2: leave
     uint32_t q, rank, size;
 };
 
-// One lane, having joined or opened the team of slot q with the word `word`:
-// waits until the leader has closed it and returns its size.
-__device__ __forceinline__ uint32_t team_form(const SyncServe& A, uint32_t q, unsigned long long word,
-                                              bool leader, unsigned long long wait_ns) {
-    const uint64_t t0 = globaltimer();
-    for (;;) {
-        const unsigned long long w = ld_relaxed64(A.join + q);
-        if ((w >> 32) != (word >> 32) || !(w & kJoinOpen)) return (uint32_t)w & 0xFFu;
-        const bool full = (w & 0xFFu) >= ((w >> 8) & 0xFFu);
-        const uint64_t dt = globaltimer() - t0;
-        if (leader && (full || dt > wait_ns)) return (uint32_t)atomicAnd(A.join + q, ~kJoinOpen) & 0xFFu;
-        // (the leader closes the team well before this; the search's own
-        // barriers are bounded too)
-        if (!leader && dt > wait_ns) return (uint32_t)(w >> 8) & 0xFFu;
-    }
-}
+// The accesses of a slot's word (serve_team.h).
+struct JoinIo {
+    unsigned long long* word;
+    __device__ __forceinline__ unsigned long long load() { return ld_relaxed64(word); }
+    __device__ __forceinline__ unsigned long long close() { return atomicAnd(word, ~kJoinOpen); }
+    __device__ __forceinline__ unsigned long long now() { return globaltimer(); }
+};
 
 // Warp 0: something to do, or nothing.
 __device__ __forceinline__ ServeCmd serve_poll(const SyncServe& A, uint32_t cursor) {
@@ -128,19 +119,20 @@ __device__ __forceinline__ ServeCmd serve_poll(const SyncServe& A, uint32_t curs
             w = ld_relaxed64(A.join + q);
             st = ld_relaxed(A.state + q);
         }
-        uint32_t m = __ballot_sync(0xFFFFFFFFu, (w & kJoinOpen) && (w & 0xFFu) < ((w >> 8) & 0xFFu));
+        uint32_t m = __ballot_sync(0xFFFFFFFFu, join_room(w));
         while (m) {
             const uint32_t l = __ffs(m) - 1;
             m &= m - 1;
             uint32_t rank = 0, size = 0;
             if (lane == l) {
                 for (int tries = 0; tries < 8; ++tries) {
-                    if (!(w & kJoinOpen) || (w & 0xFFu) >= ((w >> 8) & 0xFFu)) break;
+                    if (!join_room(w)) break;
                     const unsigned long long seen = atomicCAS(A.join + q, w, w + 1);
                     if (seen == w) {
-                        rank = (uint32_t)w & 0xFFu;
+                        rank = join_count(w);
                         __threadfence();  // acquire: the slot's descriptor
-                        size = team_form(A, q, w, false, kMemberWaitNs);
+                        JoinIo io{A.join + q};
+                        size = team_form(io, false, kMemberWaitNs);
                         break;
                     }
                     w = seen;
@@ -178,8 +170,7 @@ __device__ __forceinline__ ServeCmd serve_poll(const SyncServe& A, uint32_t curs
                 if (size > 1) {
                     // (work is in eighths of a microsecond)
                     wait = min(kJoinWaitNs, max(kJoinWaitMinNs, 125ull * mine / (4 * size)));
-                    const unsigned long long seq = (ld_relaxed64(A.join + q) >> 32) + 1;
-                    w = seq << 32 | kJoinOpen | (unsigned long long)size << 8 | 1ull;
+                    w = join_opened(ld_relaxed64(A.join + q), size);
                     __threadfence();
                     st_relaxed64(A.join + q, w);
                 }
@@ -187,7 +178,10 @@ __device__ __forceinline__ ServeCmd serve_poll(const SyncServe& A, uint32_t curs
             // (the team is open before the next claim can be made)
             __threadfence();
             st_relaxed(A.claim, 0u);
-            if (w) size = team_form(A, q, w, true, wait);
+            if (w) {
+                JoinIo io{A.join + q};
+                size = team_form(io, true, wait);
+            }
         }
     }
     size = __shfl_sync(0xFFFFFFFFu, size, 0);
