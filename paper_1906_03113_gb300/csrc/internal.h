@@ -251,6 +251,7 @@ struct SyncBar {
     unsigned long long aux[2];   // vertices and entries beside them
     uint32_t lcnt[2];            // items appended to the global list, by level parity
     uint32_t exited;             // CTAs that have left (wraps to 0)
+    uint32_t err;                // abfs_status of the first CTA that failed
 };
 
 // One search of the level-synchronous engine (a kernel argument).

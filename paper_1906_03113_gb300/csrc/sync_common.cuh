@@ -118,10 +118,19 @@ __device__ __forceinline__ void red_add_release64(unsigned long long* p, unsigne
     asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
+// A CTA fails its search.  The status stands beside the barrier words and, like
+// them, is cleared by the last CTA to leave, which copies it to the control
+// block: a member that has waited in vain may fail before rank 0, busy in
+// another search of the batch, has begun this one and cleared its control block.
+__device__ __forceinline__ void sync_fail(const SyncSearch& S, uint32_t code) {
+    atomicCAS(&S.bar->err, 0u, code);
+}
+
 // One thread of each CTA: adds `add` and the arrival to the barrier's word
 // (bar_arrive), waits until the team has arrived and returns the totals, or ~0
-// when the bounded wait ran out (bar_poll).  The wait itself delivers the totals: no further read follows
-// unless `aux` is wanted.
+// when the bounded wait ran out or, after a FULL barrier, a CTA has failed the
+// search (bar_poll).  The wait itself delivers the totals: no further read
+// follows unless `aux` is wanted.
 //
 // FULL: what the CTAs wrote before the barrier can be read after it.  Without
 // it the barrier orders only the claims of a thin level: each was an atomic on
@@ -165,7 +174,7 @@ __device__ __forceinline__ unsigned long long bar_poll(SyncSmem& sm, const SyncS
             if (t0 == 0) {
                 t0 = now;
             } else if (now - t0 > S.timeout_ns) {
-                fail(S.ctl, 5 /* ABFS_ERR_TIMEOUT */);
+                sync_fail(S, 5 /* ABFS_ERR_TIMEOUT */);
                 return ~0ull;
             }
         }
@@ -174,8 +183,10 @@ __device__ __forceinline__ unsigned long long bar_poll(SyncSmem& sm, const SyncS
     if (FULL) {
         __threadfence();  // acquire: what the others wrote before they arrived
         const unsigned long long x = ld_relaxed64(&S.bar->aux[b]);
+        const uint32_t err = ld_relaxed(&S.bar->err);
         aux = x - sm.aux[b];
         sm.aux[b] = x;
+        if (err) return ~0ull;
     }
     return (v - before) & ((1ull << kArriveShift) - 1);
 }
@@ -224,7 +235,7 @@ __device__ __forceinline__ void list_put(const SyncSearch& S, uint32_t p, unsign
         S.lb[p][at] = b;
         S.ll[p][at] = l;
     } else {
-        fail(S.ctl, 7 /* ABFS_ERR_DEVICE */);
+        sync_fail(S, 7 /* ABFS_ERR_DEVICE */);
     }
 }
 

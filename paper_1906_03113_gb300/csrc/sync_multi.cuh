@@ -317,7 +317,7 @@ __device__ __forceinline__ void ms_search(SyncSmem& sm, const SyncSearch& S, con
         if (lead) {
             sm.tick = sm.nlong = sm.verts = sm.ent = 0;
             sm.open = 0;
-            sm.act = ld_relaxed(&S.ctl->err);  // a failed append
+            sm.act = ld_relaxed(&S.bar->err);  // a failed append
         }
         if (!push) open = sm.items;
         const uint32_t nv = (uint32_t)(sm.entries >> kAuxShift);

@@ -296,7 +296,10 @@ __device__ __forceinline__ bool sync_leave(const SyncSearch& S, const Team& T) {
         S.bar->word[b] = S.bar->aux[b] = 0;
         S.bar->lcnt[b] = 0;
     }
-    S.ctl->status = ld_relaxed(&S.ctl->err) ? kFailed : kDone;
+    const uint32_t err = ld_relaxed(&S.bar->err);
+    S.bar->err = 0;
+    S.ctl->err = err;
+    S.ctl->status = err ? kFailed : kDone;
     return true;
 }
 
@@ -346,7 +349,7 @@ __device__ __forceinline__ bool sync_search(SyncSmem& sm, const SyncSearch& S, c
                     if (all <= (unsigned long long)T.size * kThinCap && entries < wide_line(S, T, all, entries)) {
                         list_slice(sm, S, T, p, p, all);
                         // a failed append leaves the list incomplete
-                        if (lead) sm.act = ld_relaxed(&S.ctl->err) ? kActFailed : kActThin;
+                        if (lead) sm.act = ld_relaxed(&S.bar->err) ? kActFailed : kActThin;
                         __syncthreads();
                         act = sm.act;
                     } else {
@@ -404,7 +407,7 @@ __device__ __forceinline__ bool sync_search(SyncSmem& sm, const SyncSearch& S, c
                 const unsigned long long tot = bar_wait<true>(sm, S, T, c, aux);
                 sm.act = wide_next(sm, S, T, up, tot, aux);
                 // a failed append leaves a list incomplete: nothing reads it
-                if (sm.act < kActDone && ld_relaxed(&S.ctl->err)) sm.act = kActFailed;
+                if (sm.act < kActDone && T.expect == 1 && ld_relaxed(&S.bar->err)) sm.act = kActFailed;
             }
             __syncthreads();
             ++k;

@@ -157,3 +157,39 @@ def test_lists_that_overflow_right_after_a_slice(lib, layers, mids):
         assert torch.equal(lev, want[0]) and torch.equal(par, want[1]), rep
         assert st["reached"] == g.n and st["nnz_reached"] == g.nnz
     G.destroy()
+
+
+def _deep_batch(n_deep, count, n_mid):
+    """A path, whose search takes far longer than a batch plan (which knows
+    vertices and entries only) expects, and `count` graphs of four entries per
+    column but vertex 0's, which is empty: their teams are made up of CTAs that
+    the path's search holds and of CTAs that are free at once."""
+    path = synth.from_arcs(n_deep, list(range(n_deep - 1)), list(range(1, n_deep)), directed=True)
+    rng = np.random.default_rng(n_mid)
+    col = np.repeat(np.arange(1, n_mid), 4)
+    row = rng.integers(n_mid, size=col.size)
+    mid = synth.from_arcs(n_mid, col.tolist(), row.tolist(), directed=True)
+    P, M = (abfs.graph_create(g.colptr, g.rowidx, directed=True) for g in (path, mid))
+    return path, mid, P, M
+
+
+@pytest.mark.parametrize("source", [0, 1])
+def test_members_that_wait_for_a_search_elsewhere(lib, source):
+    """A search whose members wait longer than timeout_ms for one that is still
+    busy with a deep search never ends as done with outputs that were not
+    written, whoever comes last."""
+    path, mid, P, M = _deep_batch(100000, 90, 60000)
+    lo, po = (torch.from_numpy(x).cuda() for x in oracle.bfs(mid, source))
+    p = abfs.default_params(timeout_ms=2, multi_source=0)
+    graphs = [P] + [M] * 90
+    lv, pr = ([torch.full((G.n,), 7, dtype=torch.int32, device="cuda") for G in graphs] for _ in range(2))
+    _, _, st = abfs.run_batch(graphs, [0] + [source] * 90, lv, pr, params=p)
+    torch.cuda.synchronize()
+    for q, s in enumerate(st):
+        assert s in (0, binding.ERR_TIMEOUT)
+        if s == 0 and q == 0:
+            assert torch.equal(lv[0], torch.arange(P.n, dtype=torch.int32, device="cuda"))
+        elif s == 0:
+            assert torch.equal(lv[q], lo) and torch.equal(pr[q], po), q
+    P.destroy()
+    M.destroy()
