@@ -581,6 +581,8 @@ SyncSearch make_sync(const abfs_graph_s* g, char* base, const Layout& L, SyncBar
     }
     S.ctl = reinterpret_cast<InstCtl*>(base + L.ctl);
     S.bar = bar;
+    S.bars = reinterpret_cast<const char*>(bar);
+    S.nbars = 1;
     S.hub_avg = (uint32_t)std::max<uint64_t>(8, 3 * g->nnz / (2ull * g->n));
     S.timeout_ns = (unsigned long long)p.timeout_ms * 1000000ull;
     S.hold_units = test_hold_units();
@@ -1400,11 +1402,10 @@ int batch_create(const abfs_graph_t* g, const uint32_t* sources, uint32_t count,
             o = align_up(o + bytes, 256);
             return at;
         };
-        const size_t at_search = part(sizeof(SyncSearch) * ninst), at_bar = part(256 * (size_t)ninst);
+        const size_t at_search = part(sizeof(SyncSearch) * ninst), at_bar = part(kBarStride * (size_t)ninst);
         const size_t at_off = part(4 * plan.off.size());
         const size_t at_steps = part(sizeof(SyncStep) * std::max<size_t>(plan.steps.size(), 1));
         const size_t at_queue = part(4 * std::max<size_t>(plan.queue.size(), 1)), at_next = part(8);
-        static_assert(sizeof(SyncBar) <= 256, "a barrier per 256 bytes");
         rc = dev_alloc((void**)&b->d_sync, o);
         if (rc) {
             abfs_batch_destroy(b);
@@ -1413,7 +1414,9 @@ int batch_create(const abfs_graph_t* g, const uint32_t* sources, uint32_t count,
         // barriers and the queue's counters start at zero
         std::vector<char> h(o, 0);
         for (uint32_t t = 0; t < ninst; ++t) {
-            searches[t].bar = reinterpret_cast<SyncBar*>(b->d_sync + at_bar + 256 * (size_t)t);
+            searches[t].bar = reinterpret_cast<SyncBar*>(b->d_sync + at_bar + kBarStride * (size_t)t);
+            searches[t].bars = b->d_sync + at_bar;
+            searches[t].nbars = ninst;
             std::memcpy(h.data() + at_search + sizeof(SyncSearch) * t, &searches[t], sizeof(SyncSearch));
         }
         std::memcpy(h.data() + at_off, plan.off.data(), 4 * plan.off.size());

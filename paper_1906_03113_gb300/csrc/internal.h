@@ -252,7 +252,11 @@ struct SyncBar {
     uint32_t lcnt[2];            // items appended to the global list, by level parity
     uint32_t exited;             // CTAs that have left (wraps to 0)
     uint32_t err;                // abfs_status of the first CTA that failed
+    uint32_t pad[20];
+    unsigned long long beat;     // progress between barriers (a cache line of its own, never reset)
 };
+constexpr uint32_t kBarStride = 256;
+static_assert(sizeof(SyncBar) == 136 && sizeof(SyncBar) <= kBarStride, "the count starts a cache line");
 
 // One search of the level-synchronous engine (a kernel argument).
 struct SyncSearch {
@@ -275,6 +279,8 @@ struct SyncSearch {
     uint32_t* parent;
     InstCtl* ctl;
     SyncBar* bar;
+    const char* bars;            // the barriers of all searches of the launch, kBarStride
+    uint32_t nbars;              // bytes apart: its progress, for the bounded waits
     uint4* trace;
     uint32_t trace_cap;
     uint32_t bu_alpha, bu_beta;  // hybrid thresholds (0: off or not allowed)

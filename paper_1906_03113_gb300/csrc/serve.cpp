@@ -97,7 +97,7 @@ struct abfs_server_s {
     // device
     Inst* d_slots = nullptr;
     // queries on the level-synchronous engine (cfg.params permitting): their
-    // slots, barriers (256 bytes each) and teams being formed
+    // slots, barriers (kBarStride bytes each) and teams being formed
     int ctas = 0;                 // CTAs of its launch, 0: the unit scheduler serves
     SyncSlot* d_sync = nullptr;
     char* d_bars = nullptr;
@@ -197,7 +197,7 @@ cudaError_t serve_describe(abfs_server_s* S, uint32_t i, const Request& rq, size
     if (S->ctas) {
         SyncSlot& q = S->h_sync[i];
         q.search = serve_search(S->graphs[rq.g], S->d_arena + off, S->layouts[rq.g],
-                                reinterpret_cast<SyncBar*>(S->d_bars + 256 * (size_t)i), S->d_ctl + i, rq.src,
+                                reinterpret_cast<SyncBar*>(S->d_bars + kBarStride * (size_t)i), S->d_ctl + i, rq.src,
                                 rq.level, rq.parent, S->cfg.params);
         q.ticket = rq.ticket;
         q.notify = S->d_notify + i;
@@ -387,10 +387,10 @@ extern "C" int abfs_serve_start(const abfs_graph_t* g, uint32_t ngraphs, const a
     ck(cudaHostAlloc((void**)&S->h_words, 4 * (size_t)ns + 64, cudaHostAllocDefault));
     if (S->ctas) {
         ck(cudaMalloc((void**)&S->d_sync, sizeof(SyncSlot) * ns));
-        ck(cudaMalloc((void**)&S->d_bars, 256 * (size_t)ns));
+        ck(cudaMalloc((void**)&S->d_bars, kBarStride * (size_t)ns));
         ck(cudaMalloc((void**)&S->d_join, 8 * (size_t)ns));
         ck(cudaHostAlloc((void**)&S->h_sync, sizeof(SyncSlot) * ns, cudaHostAllocDefault));
-        if (e == cudaSuccess) ck(cudaMemset(S->d_bars, 0, 256 * (size_t)ns));
+        if (e == cudaSuccess) ck(cudaMemset(S->d_bars, 0, kBarStride * (size_t)ns));
         if (e == cudaSuccess) ck(cudaMemset(S->d_join, 0, 8 * (size_t)ns));
     }
     if (e == cudaSuccess) ck(cudaHostGetDevicePointer((void**)&S->d_notify, S->h_notify, 0));

@@ -80,6 +80,7 @@ struct SyncSmem {
     unsigned long long wm[2][kSyncWarps];
     uint32_t step;                            // barriers passed
     unsigned long long word[2], aux[2];       // the barrier words as last seen
+    unsigned long long wait_from, wait_seen;  // bar_late's clock and the progress it saw
 };
 
 // A CTA's place in its team.
@@ -118,12 +119,50 @@ __device__ __forceinline__ void red_add_release64(unsigned long long* p, unsigne
     asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
+// Progress, for the waits of the other CTAs of the launch: in a batch a member
+// may wait for one that is busy in another search, for as long as that search
+// takes.  Barriers show it by themselves (bar_late reads the words of all
+// searches of the launch); a step between two barriers that can outlast a
+// millisecond counts its search's beat up once in a while: one lane, at each
+// `every`-th (a power of two) piece of work, of which `n` counts.  Passes over
+// the vertices, which the CTAs share evenly, do at each step of the team's first
+// thread if a CTA has a million vertices or more.  (A count shared by a batch of
+// 128, moved at every step of those passes and in every 16th thin level:
+// 593 -> 606 us, 4096^2 grid 14.3 -> 14.5 ms.)
+__device__ __forceinline__ void sync_beat(const SyncSearch& S, uint32_t n, uint32_t every) {
+    if ((n & (every - 1)) == every - 1) red_add64(&S.bar->beat, 1ull);
+}
+__device__ __forceinline__ bool sync_long_pass(const SyncSearch& S, const Team& T) {
+    return T.rank == 0 && threadIdx.x == 0 && (S.n >> 20) >= T.size;
+}
+
 // A CTA fails its search.  The status stands beside the barrier words and, like
 // them, is cleared by the last CTA to leave, which copies it to the control
 // block: a member that has waited in vain may fail before rank 0, busy in
 // another search of the batch, has begun this one and cleared its control block.
 __device__ __forceinline__ void sync_fail(const SyncSearch& S, uint32_t code) {
     atomicCAS(&S.bar->err, 0u, code);
+}
+
+// A waiting thread, now and then: whether its wait has run out, which fails the
+// search.  The clock starts at the first look and again whenever the launch has
+// made progress since the last one.
+__device__ __noinline__ bool bar_late(SyncSmem& sm, const SyncSearch& S, bool first) {
+    const unsigned long long now = globaltimer();
+    unsigned long long seen = 0;
+#pragma unroll 4
+    for (uint32_t i = 0; i < S.nbars; ++i) {
+        const SyncBar* const b = reinterpret_cast<const SyncBar*>(S.bars + (size_t)kBarStride * i);
+        // (a sum that each new arrival and each beat changes)
+        seen += ld_relaxed64(&b->word[0]) + 3 * ld_relaxed64(&b->word[1]) + 5 * ld_relaxed64(&b->beat);
+    }
+    if (first || seen != sm.wait_seen) {
+        sm.wait_from = now;
+        sm.wait_seen = seen;
+    }
+    if (now - sm.wait_from <= S.timeout_ns) return false;
+    sync_fail(S, 5 /* ABFS_ERR_TIMEOUT */);
+    return true;
 }
 
 // One thread of each CTA: adds `add` and the arrival to the barrier's word
@@ -164,20 +203,11 @@ __device__ __forceinline__ unsigned long long bar_poll(SyncSmem& sm, const SyncS
     unsigned long long* w = &S.bar->word[b];
     const unsigned long long before = sm.word[b];
     unsigned long long v;
-    uint64_t t0 = 0;
     for (uint32_t spin = 0;; ++spin) {
         v = ld_relaxed64(w);
         if ((uint32_t)((v - before) >> kArriveShift) == expect) break;
-        // reading %globaltimer is slow: the clock starts after 4096 polls
-        if ((spin & 4095u) == 4095u) {
-            const uint64_t now = globaltimer();
-            if (t0 == 0) {
-                t0 = now;
-            } else if (now - t0 > S.timeout_ns) {
-                sync_fail(S, 5 /* ABFS_ERR_TIMEOUT */);
-                return ~0ull;
-            }
-        }
+        // reading %globaltimer is slow: the clock is looked at every 4096 polls
+        if ((spin & 4095u) == 4095u && bar_late(sm, S, spin == 4095u)) return ~0ull;
     }
     sm.word[b] = v;
     if (FULL) {

@@ -279,7 +279,10 @@ __device__ __noinline__ void wide_expand(SyncSmem& sm, const SyncSearch& S, cons
     uint32_t nj = 0, nbeg = 0, nlen = 0;
     auto fetch = [&]() {
         uint32_t x = 0;
-        if (lane == 0) x = atomicAdd(&sm.tick, 1u);
+        if (lane == 0) {
+            x = atomicAdd(&sm.tick, 1u);
+            sync_beat(S, x, 256);
+        }
         const unsigned long long c = (unsigned long long)__shfl_sync(0xFFFFFFFFu, x, 0) * T.size + T.rank;
         const unsigned long long at = c * run + lane;
         nj = nbeg = nlen = 0;
@@ -397,7 +400,9 @@ __device__ __noinline__ void sync_bitmaps(const SyncSearch& S, const Team& T, ui
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t W = T.size * kSyncWarps;
     constexpr int Q = kBitmapWords;
+    const bool slow = sync_long_pass(S, T);
     for (uint32_t w0 = (warp * T.size + T.rank) * Q; w0 < S.nwords; w0 += Q * W) {
+        if (slow) red_add64(&S.bar->beat, 1ull);
         uint32_t lv[Q];
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
@@ -478,6 +483,7 @@ __device__ __noinline__ void sync_extract(SyncSmem& sm, const SyncSearch& S, con
     const uint32_t g0 = (warp * T.size + T.rank) * Q;  // groups of Q words, round robin
     uint32_t* const khi = reinterpret_cast<uint32_t*>(S.key) + 1;
     uint32_t verts = 0, entries = 0, mine = 0;
+    const bool slow = sync_long_pass(S, T);
     // this lane's word of the group at wb, loaded a group ahead (a batch of 128
     // graphs 608 -> 598 us)
     auto load = [&](const uint32_t* bits, uint32_t wb) {
@@ -487,6 +493,7 @@ __device__ __noinline__ void sync_extract(SyncSmem& sm, const SyncSearch& S, con
     uint32_t ahead = MASKS ? 0u : load(from, g0);
 #pragma unroll 1
     for (uint32_t wb = g0; wb < S.nwords; wb += Q * W) {
+        if (slow) red_add64(&S.bar->beat, 1ull);
         const bool own = lane < Q && wb + lane < S.nwords;
         const uint32_t seen = ahead;
         uint32_t word = 0, add = 0;
@@ -548,6 +555,7 @@ __device__ __noinline__ void sync_extract(SyncSmem& sm, const SyncSearch& S, con
     ahead = load(S.fbm[pn], g0);
 #pragma unroll 1
     for (uint32_t wb = g0; wb < S.nwords; wb += Q * W) {
+        if (slow) red_add64(&S.bar->beat, 1ull);
         const uint32_t word = ahead;
         ahead = load(S.fbm[pn], wb + Q * W);
         if (!__any_sync(0xFFFFFFFFu, word != 0)) continue;
@@ -597,7 +605,10 @@ __device__ __noinline__ void sync_bottom_up(SyncSmem& sm, const SyncSearch& S, c
 #pragma unroll 1
     for (;;) {
         uint32_t x = 0;
-        if (lane == 0) x = atomicAdd(&sm.tick, 1u);
+        if (lane == 0) {
+            x = atomicAdd(&sm.tick, 1u);
+            sync_beat(S, x, 64);
+        }
         x = __shfl_sync(0xFFFFFFFFu, x, 0);
         const unsigned long long c = ((unsigned long long)x * T.size + T.rank) * kBuWords;
         if (c >= S.nwords) break;
@@ -637,6 +648,7 @@ __device__ __noinline__ void sync_bottom_up(SyncSmem& sm, const SyncSearch& S, c
                 const uint32_t lend = __shfl_sync(0xFFFFFFFFu, end, ldr);
                 uint32_t found = kUnset;
                 for (uint32_t x = le; x < lend; x += 32) {
+                    if (lane == 0) sync_beat(S, (x - le) / 32, 1024);
                     const uint32_t idx = x + lane;
                     const uint32_t j = idx < lend ? ld_ro(S.rowidx + idx) : kUnset;
                     const bool hit = j != kUnset && ((ld_frozen(fbm + (j >> 5)) >> (j & 31)) & 1u);

@@ -97,7 +97,10 @@ __device__ __noinline__ void ms_scan(SyncSmem& sm, const SyncSearch& S, const Te
     unsigned long long open = 0;
     for (;;) {
         uint32_t x = 0;
-        if (lane == 0) x = atomicAdd(&sm.tick, 1u);
+        if (lane == 0) {
+            x = atomicAdd(&sm.tick, 1u);
+            sync_beat(S, x, 32);
+        }
         x = __shfl_sync(0xFFFFFFFFu, x, 0);
         const unsigned long long w = (unsigned long long)x * T.size + T.rank;
         if (w >= S.nwords) break;
@@ -193,6 +196,7 @@ __device__ __noinline__ void ms_scan(SyncSmem& sm, const SyncSearch& S, const Te
     const uint32_t longs = min(sm.nlong, kThinCap);
     uint32_t round = 0;
     for (uint32_t i = 0; i < longs; ++i) {
+        if (threadIdx.x == 0) sync_beat(S, 0, 1);
         const uint32_t v = sm.ij[0][i];
         const unsigned long long want = (unsigned long long)sm.il[0][i] << 32 | sm.ib[0][i];
         const uint32_t cb = ld_ro(S.colptr + v), end = ld_ro(S.colptr + v + 1);
@@ -241,7 +245,9 @@ __device__ __noinline__ void ms_scan(SyncSmem& sm, const SyncSearch& S, const Te
 __device__ __forceinline__ void ms_search(SyncSmem& sm, const SyncSearch& S, const Team& T) {
     const bool lead = threadIdx.x == 0;
     const uint32_t stride = T.size * kSyncThreads, t0 = T.rank * kSyncThreads + threadIdx.x;
+    const bool slow = sync_long_pass(S, T);
     for (uint32_t v = t0; v < S.n; v += stride) {
+        if (slow) red_add64(&S.bar->beat, 1ull);
         S.ms_vis[v] = 0ull;
         S.ms_fr[0][v] = 0ull;
         S.ms_nx[v] = 0ull;
@@ -333,6 +339,7 @@ __device__ __forceinline__ void ms_search(SyncSmem& sm, const SyncSearch& S, con
         const unsigned long long all = S.ms == 64 ? ~0ull : (1ull << S.ms) - 1;
         const uint32_t lane = threadIdx.x & 31, W = T.size * kSyncWarps;
         for (uint32_t w = T.rank * kSyncWarps + (threadIdx.x >> 5); w < S.nwords; w += W) {
+            if (slow) red_add64(&S.bar->beat, 1ull);
             const uint32_t v = w * 32 + lane;
             const unsigned long long lack = v < S.n ? all & ~ld_l2(S.ms_vis + v) : 0ull;
             unsigned long long un = warp_or64(lack);

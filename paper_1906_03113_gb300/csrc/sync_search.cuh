@@ -23,9 +23,11 @@ __device__ __forceinline__ void sync_trace(const SyncSearch& S, const Team& T, u
 __device__ __forceinline__ void sync_init(const SyncSearch& S, const Team& T) {
     const uint32_t stride = T.size * kSyncThreads;
     const uint32_t t0 = T.rank * kSyncThreads + threadIdx.x;
+    const bool slow = sync_long_pass(S, T);
     // two keys per 16-byte store
     ulonglong2* const k2 = reinterpret_cast<ulonglong2*>(S.key);
     for (uint32_t i = t0; i < S.n / 2; i += stride) {
+        if (slow) red_add64(&S.bar->beat, 1ull);
         ulonglong2 x = make_ulonglong2(kKeyUnset, kKeyUnset);
         if (2 * i == S.src) x.x = S.src_label;
         if (2 * i + 1 == S.src) x.y = S.src_label;
@@ -33,7 +35,10 @@ __device__ __forceinline__ void sync_init(const SyncSearch& S, const Team& T) {
     }
     if ((S.n & 1) && t0 == 0) S.key[S.n - 1] = S.n - 1 == S.src ? S.src_label : kKeyUnset;
     if (S.sigma)
-        for (uint32_t v = t0; v < S.n; v += stride) S.sigma[v] = v == S.src ? 1ull : 0ull;
+        for (uint32_t v = t0; v < S.n; v += stride) {
+            if (slow) red_add64(&S.bar->beat, 1ull);
+            S.sigma[v] = v == S.src ? 1ull : 0ull;
+        }
     if (T.rank == 0) {
         uint32_t* c = reinterpret_cast<uint32_t*>(S.ctl);
         for (uint32_t w = threadIdx.x; w < sizeof(InstCtl) / 4; w += kSyncThreads) c[w] = 0u;
@@ -48,6 +53,7 @@ __device__ __noinline__ void sync_outputs(const SyncSearch& S, const Team& T) {
     const uint32_t stride = T.size * kSyncThreads;
     const uint32_t t0 = T.rank * kSyncThreads + threadIdx.x;
     const uint32_t quads = S.n / 4;
+    const bool slow = sync_long_pass(S, T);
     const bool vec = ((reinterpret_cast<uintptr_t>(S.level) | reinterpret_cast<uintptr_t>(S.parent)) & 15u) == 0;
     auto key_at = [&](uint32_t o) -> unsigned long long {
         if (!S.pos) return ld_relaxed64(S.key + o);
@@ -68,6 +74,7 @@ __device__ __noinline__ void sync_outputs(const SyncSearch& S, const Team& T) {
         }
     };
     for (uint32_t q = t0; q < quads; q += 2 * stride) {
+        if (slow) red_add64(&S.bar->beat, 1ull);
         const bool two = q + stride < quads;
         unsigned long long a[4], b[4];
 #pragma unroll

@@ -193,3 +193,21 @@ def test_members_that_wait_for_a_search_elsewhere(lib, source):
             assert torch.equal(lv[q], lo) and torch.equal(pr[q], po), q
     P.destroy()
     M.destroy()
+
+
+def test_a_deep_search_is_progress_for_those_who_wait(lib):
+    """timeout_ms bounds waits without progress: the members that wait for the
+    deep search (a thousand times longer than timeout_ms planned for) find their
+    own, and every search of the batch is exact."""
+    path, mid, P, M = _deep_batch(100000, 90, 60000)
+    lo, po = (torch.from_numpy(x).cuda() for x in oracle.bfs(mid, 1))
+    p = abfs.default_params(timeout_ms=1, multi_source=0)
+    lv, pr, st = abfs.run_batch([P] + [M] * 90, [0] + [1] * 90, params=p)
+    torch.cuda.synchronize()
+    assert st == [0] * 91
+    k = torch.arange(P.n, dtype=torch.int32, device="cuda")
+    assert torch.equal(lv[0], k) and torch.equal(pr[0], (k - 1).clamp_(min=0))
+    for q in range(1, 91):
+        assert torch.equal(lv[q], lo) and torch.equal(pr[q], po), q
+    P.destroy()
+    M.destroy()
