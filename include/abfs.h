@@ -381,8 +381,9 @@ int abfs_batch_tune(const abfs_graph_t* g, const uint32_t* sources, uint32_t cou
  * enough workspace memory (abfs_graph_footprint of the query's graph, carved
  * from a memory budget) are free, while other queries are running; their
  * work overlaps on the device in one persistent launch, whose CTAs form a team
- * for each query as they come free.  The launch ends after idle_exit_ms without work and is
- * relaunched on demand.  Each query's result equals abfs_run's, bit for bit.
+ * for each query as they come free.  The launch ends after idle_exit_ms in which
+ * no query was on the device and is relaunched on demand.  Each query's result
+ * equals abfs_run's, bit for bit.
  * The paper has no counterpart (it evaluates single searches).
  */
 typedef struct {

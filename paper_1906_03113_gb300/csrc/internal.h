@@ -333,7 +333,8 @@ struct SyncServe {
     // per slot, the team being formed (serve_team.h)
     unsigned long long* join;
     const uint32_t* stop_flag;
-    unsigned long long* heartbeat;
+    uint32_t* closed;            // number of the last launch that has been ended for want of queries
+    uint32_t launch;             // this launch's number, from 1
     uint32_t nslots;
     unsigned long long idle_exit_ns;
 };

@@ -176,6 +176,8 @@ EngineArgs serve_args(abfs_server_s* S) {
 constexpr uint32_t kTeamServeN = 1u << 20;
 constexpr uint64_t kTeamServeNnz = 1ull << 25;
 
+constexpr size_t kClosedAt = 32;  // words of d_done after the claimers' lock
+
 // Device launch that serves the slots.
 cudaError_t serve_launch(abfs_server_s* S) {
     if (!S->ctas) return launch_engine(serve_args(S), grid_for(S->sms, S->cfg.params), S->kstream);
@@ -185,7 +187,8 @@ cudaError_t serve_launch(abfs_server_s* S) {
     A.claim = S->d_done;
     A.join = S->d_join;
     A.stop_flag = S->d_stop;
-    A.heartbeat = S->d_beat;
+    A.closed = S->d_done + kClosedAt;
+    A.launch = (uint32_t)(S->launches + 1);
     A.nslots = S->cfg.max_slots;
     A.idle_exit_ns = (unsigned long long)S->cfg.idle_exit_ms * 1000000ull;
     return launch_sync_serve(A, S->ctas, S->kstream);

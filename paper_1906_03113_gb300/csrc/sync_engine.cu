@@ -95,6 +95,7 @@ constexpr unsigned long long kMemberWaitNs = 1000000000ull;
 struct ServeCmd {
     uint32_t what;  // 0: nothing to do, 1: run slot q, 2: leave
     uint32_t q, rank, size;
+    uint32_t busy;  // some slot holds a query that is submitted or running
 };
 
 // The accesses of a slot's word (serve_team.h).
@@ -108,7 +109,7 @@ struct JoinIo {
 // Warp 0: something to do, or nothing.
 __device__ __forceinline__ ServeCmd serve_poll(const SyncServe& A, uint32_t cursor) {
     const uint32_t lane = threadIdx.x & 31;
-    ServeCmd c = {0, 0, 0, 0};
+    ServeCmd c = {0, 0, 0, 0, 0};
     unsigned long long work = 0;  // of all queries submitted or running
     uint32_t near = ~0u;          // submitted query nearest after the cursor: its distance
     for (uint32_t b = 0; b < A.nslots; b += 32) {
@@ -147,10 +148,12 @@ __device__ __forceinline__ ServeCmd serve_poll(const SyncServe& A, uint32_t curs
                 return c;
             }
         }
+        c.busy |= st & 0xFFu;
         if (st & 0xFFu) work += st >> kSlotWorkShift;
         if ((st & 0xFFu) == kSlotSubmitted) near = min(near, q >= cursor ? q - cursor : q + A.nslots - cursor);
     }
     near = __reduce_min_sync(0xFFFFFFFFu, near);
+    c.busy = __any_sync(0xFFFFFFFFu, c.busy != 0);
     if (near == ~0u) return c;
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) work += __shfl_xor_sync(0xFFFFFFFFu, work, d);
@@ -161,9 +164,10 @@ __device__ __forceinline__ ServeCmd serve_poll(const SyncServe& A, uint32_t curs
             const uint32_t st = ld_relaxed(A.state + q);
             const uint32_t run = (st & ~0xFFu) | kSlotRunning;
             unsigned long long w = 0, wait = 0;
-            if ((st & 0xFFu) == kSlotSubmitted && atomicCAS(A.state + q, st, run) == st) {
+            // (a launch that has been closed claims nothing more)
+            if ((st & 0xFFu) == kSlotSubmitted && ld_relaxed(A.closed) != A.launch &&
+                atomicCAS(A.state + q, st, run) == st) {
                 __threadfence();  // acquire: the descriptor the host wrote before the state
-                atomicAdd(A.heartbeat, 1ull);
                 const unsigned long long mine = max(st >> kSlotWorkShift, 1u);
                 const unsigned long long part = (mine * gridDim.x + work - 1) / max(work, 1ull);
                 size = max(1u, (uint32_t)min(part, (unsigned long long)ld_l2(&A.slots[q].cap)));
@@ -193,34 +197,51 @@ __device__ __forceinline__ ServeCmd serve_poll(const SyncServe& A, uint32_t curs
     return c;
 }
 
+// Warp 0, having found no query for idle_exit_ns: closes the launch unless one
+// has come meanwhile.  Under the claimers' lock, so that no query is claimed by a
+// launch whose other CTAs are leaving.
+__device__ __forceinline__ bool serve_close(const SyncServe& A) {
+    const uint32_t lane = threadIdx.x & 31;
+    uint32_t locked = 0;
+    if (lane == 0) locked = atomicCAS(A.claim, 0u, 1u) == 0u;
+    if (!__shfl_sync(0xFFFFFFFFu, locked, 0)) return false;
+    __threadfence();
+    uint32_t busy = 0;
+    for (uint32_t q = lane; q < A.nslots; q += 32) busy |= ld_relaxed(A.state + q) & 0xFFu;
+    busy = __any_sync(0xFFFFFFFFu, busy != 0);
+    if (lane == 0) {
+        if (!busy) st_relaxed(A.closed, A.launch);
+        __threadfence();
+        st_relaxed(A.claim, 0u);
+    }
+    return !busy;
+}
+
 __global__ void __launch_bounds__(kSyncThreads, 1) sync_serve_kernel(const __grid_constant__ SyncServe A) {
     __shared__ SyncSmem sm;
     __shared__ SyncSlot slot;
     __shared__ ServeCmd cmd;
     uint64_t idle_since = 0;
-    unsigned long long last_beat = ~0ull;
     uint32_t backoff = 64;
     for (;;) {
         if (threadIdx.x < 32) {
-            ServeCmd c = {2, 0, 0, 0};
-            if (ld_relaxed(A.stop_flag) == 0) {
+            ServeCmd c = {2, 0, 0, 0, 0};
+            if (ld_relaxed(A.stop_flag) == 0 && ld_relaxed(A.closed) != A.launch) {
                 c = serve_poll(A, blockIdx.x * 7u % A.nslots);
                 if (c.what == 0) {
-                    // nothing to do: sleep, or leave after idle_exit_ns without
-                    // progress anywhere (the host relaunches on demand)
-                    const unsigned long long beat = ld_relaxed64(A.heartbeat);
+                    // Nothing to do: sleep, or end the launch after idle_exit_ns in
+                    // which no slot held a query (the host relaunches on demand).
+                    // While one runs, however long, every CTA stays for the next;
+                    // and the CTAs leave together, so that a launch that goes on
+                    // has the whole GPU.
                     const uint64_t now = globaltimer();
-                    if (beat != last_beat) {
-                        last_beat = beat;
-                        idle_since = now;
-                    } else if (now - idle_since > A.idle_exit_ns) {
-                        c.what = 2;
-                    }
+                    if (c.busy || idle_since == 0) idle_since = now;
+                    else if (now - idle_since > A.idle_exit_ns && serve_close(A)) c.what = 2;
                     if (c.what == 0) __nanosleep(backoff);
                     if (backoff < 1024) backoff <<= 1;
                 } else {
                     backoff = 64;
-                    last_beat = ~0ull;
+                    idle_since = 0;
                 }
             }
             if (threadIdx.x == 0) cmd = c;
@@ -242,7 +263,6 @@ __global__ void __launch_bounds__(kSyncThreads, 1) sync_serve_kernel(const __gri
                 // ticket and status reach the host's word after every write of
                 // the search (each CTA fenced its own before it left)
                 st_relaxed(A.state + c.q, kSlotFree);
-                atomicAdd(A.heartbeat, 1ull);
                 __threadfence_system();
                 const unsigned long long word = slot.ticket << 8 | (ld_relaxed(&slot.search.ctl->err) & 0xFFu);
                 asm volatile("st.release.sys.global.u64 [%0], %1;" ::"l"(slot.notify), "l"(word) : "memory");
