@@ -207,8 +207,15 @@ bool same_layout(const abfs_params& a, const abfs_params& b) {
 // The knobs of the unit scheduler (units, narrow and cluster runs, the grid and
 // the reduction threshold) mean nothing to the level-synchronous engine: a
 // search that sets any of them asks for the scheduler.
-bool sync_applies(uint32_t n, uint64_t nnz, const abfs_params& p) {
+//
+// Neither does it run searches (a batch's, together) of n vertices and nnz
+// entries in which the passes over the vertices are nearly everything: 24 bytes
+// a vertex, 8 on the scheduler, which only fills the outputs.  On 2^27 vertices
+// 16 384 entries take 557 us on teams and 344 on the scheduler, 2^20 entries 620
+// and 634; on 2^24 vertices 16 384 entries 117 and 165.
+bool sync_applies(uint64_t n, uint64_t nnz, const abfs_params& p) {
     const abfs_params d = default_params();
+    if (n > (1u << 25) && nnz < n / 128) return false;
     return p.mode == ABFS_MODE_SUBMATRIX && !shrink_enabled(p) && p.tile == d.tile &&
            p.unit_entries == d.unit_entries && p.narrow_max == d.narrow_max &&
            p.narrow_edges == d.narrow_edges && p.ctas_per_sm == d.ctas_per_sm &&
@@ -232,10 +239,14 @@ double sync_work_us(uint32_t n, uint64_t nnz, uint32_t ms) {
     return (n <= kBitsN ? 0.45e-3 : 0.9e-3) * (double)nnz + 4e-3 * n;
 }
 
-// The largest useful team of a search: a few thousand entries per CTA.  Up to
-// 16 384 entries one CTA, without barriers between CTAs, is fastest.
+// The largest useful team of a search: a few thousand entries per CTA, and as
+// many vertices, whose words the team clears, reads and writes out (16 384
+// entries on 2^24 vertices: one CTA 20 ms, 152 CTAs 0.12 ms; on 2^16 vertices 145
+// and, on 16 CTAs, 48 us; 8 or 4 CTAs there 50 and 60 us).  Up to 16 384 of both
+// one CTA, without barriers between CTAs.
 int sync_team_cap(const SyncSearch& S, int most) {
-    const uint64_t want = S.local || S.nnz <= 16384 ? 1 : (S.nnz + 4095) / 4096;
+    const uint64_t size = std::max<uint64_t>(S.nnz, S.n);
+    const uint64_t want = S.local || size <= 16384 ? 1 : (size + 4095) / 4096;
     return (int)std::min<uint64_t>((uint64_t)most, std::max<uint64_t>(want, 1));
 }
 
@@ -1286,7 +1297,12 @@ int batch_create(const abfs_graph_t* g, const uint32_t* sources, uint32_t count,
     }
     const uint32_t ninst = (uint32_t)inst.size();
     b->ninst = ninst;
-    const int most = sync_applies(g[0]->n, g[0]->nnz, p) ? sync_max_ctas(g[0]->device, g[0]->sms) : 0;
+    uint64_t all_n = 0, all_nnz = 0;
+    for (const Search& m : inst) {
+        all_n += g[m.gi]->n;
+        all_nnz += g[m.gi]->nnz;
+    }
+    const int most = sync_applies(all_n, all_nnz, p) ? sync_max_ctas(g[0]->device, g[0]->sms) : 0;
     const bool sync = most > 0;
     std::vector<Layout> L(ninst);
     std::vector<size_t> base(ninst);

@@ -388,9 +388,9 @@ int check_params(const abfs_params& p);
 EngineParams engine_params(const abfs_params& p);
 Layout layout_for(uint32_t n, uint64_t nnz, const abfs_params& p, uint32_t ms = 0,
                   bool relabel = false, bool sync = false);
-// Whether a search of this size with these parameters runs on the
-// level-synchronous engine.
-bool sync_applies(uint32_t n, uint64_t nnz, const abfs_params& p);
+// Whether searches of n vertices and nnz entries in all with these parameters
+// run on the level-synchronous engine.
+bool sync_applies(uint64_t n, uint64_t nnz, const abfs_params& p);
 Inst make_inst_raw(const uint32_t* colptr, const uint32_t* rowidx, uint32_t n, char* base,
                    const Layout& L, uint32_t src, int32_t* level, int32_t* parent);
 int grid_for(int sms, const abfs_params& p);
