@@ -45,7 +45,7 @@ enum SyncAct : uint32_t {
     kActThin = 0,    // the next level is thin, the lists stay where they are
     kActEven = 1,    // thin, after the lists were evened out through the global list
     kActWide = 2,    // the next level is wide
-    kActSlice = 3,   // thin, from the global list a wide level left
+    kActSlice = 3,   // thin, from the global list that a wide level left
     kActBottomUp = 4,
     kActDone = 5,
     kActFailed = 6,  // the bounded wait ran out, or an append failed
@@ -61,6 +61,7 @@ struct SyncSmem {
     uint32_t verts, ent;              // wide levels: vertices this CTA reached, their entries
     uint32_t tick;                    // wide levels: runs this CTA's warps have taken
     uint32_t base;
+    uint32_t at, left;                // what is left of this CTA's share of the global list
     uint32_t wsum[kSyncWarps], wpre[kSyncWarps];
     uint32_t act;                     // SyncAct after the last barrier
     uint32_t passed;                  // whether the last team_sync was passed (written there only)
@@ -283,20 +284,34 @@ __device__ __noinline__ void list_dump(SyncSmem& sm, const SyncSearch& S, uint32
         list_put(S, p, (unsigned long long)sm.base + i, sm.ij[q][i], sm.ib[q][i], sm.il[q][i]);
 }
 
-// Takes this CTA's even share of the global list of parity p (`items` items,
-// at most kThinCap per CTA) into its list `q`.  Whole CTA.
-__device__ __noinline__ void list_slice(SyncSmem& sm, const SyncSearch& S, const Team& T, uint32_t q,
-                                        uint32_t p, unsigned long long items) {
-    const uint32_t n = (uint32_t)items, lo = n * T.rank / T.size, hi = n * (T.rank + 1) / T.size;
-    const uint32_t c = hi - lo;
-    for (uint32_t i = threadIdx.x; i < c && lo + i < S.icap; i += kSyncThreads) {
-        sm.ij[q][i] = ld_l2(S.lj[p] + lo + i);
-        sm.ib[q][i] = ld_l2(S.lb[p] + lo + i);
-        sm.il[q][i] = ld_l2(S.ll[p] + lo + i);
+// The next items of this CTA's share of the global list of parity p (the share:
+// sm.left items from sm.at on) in its list `q`, as many as that holds.  Whole CTA.
+__device__ __noinline__ void list_round(SyncSmem& sm, const SyncSearch& S, uint32_t q, uint32_t p) {
+    const uint32_t at = sm.at, left = sm.left;
+    const uint32_t c = min(left, kThinCap);
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < c && at + i < S.icap; i += kSyncThreads) {
+        sm.ij[q][i] = ld_l2(S.lj[p] + at + i);
+        sm.ib[q][i] = ld_l2(S.lb[p] + at + i);
+        sm.il[q][i] = ld_l2(S.ll[p] + at + i);
     }
     if (threadIdx.x == 0) {
+        sync_beat(S, 0, 1);
+        sm.at = at + c;
+        sm.left = left - c;
         sm.app[q][0] = c;
         sm.app[q][1] = ~0u;  // entries: not known
+    }
+    __syncthreads();
+}
+
+// Gives this CTA its even share of the global list of parity p (`items` items),
+// the first round of it in its list `q`.  Whole CTA.
+__device__ __noinline__ void list_slice(SyncSmem& sm, const SyncSearch& S, const Team& T, uint32_t q,
+                                        uint32_t p, unsigned long long items) {
+    if (threadIdx.x == 0) {
+        sm.at = (uint32_t)(items * T.rank / T.size);
+        sm.left = (uint32_t)(items * (T.rank + 1) / T.size) - sm.at;
         // Every reservation in this list was made before the last barrier.  The
         // next barrier may be a thin level's, which orders no stores: the reset
         // is an atomic whose returned value this thread has stored before the
@@ -304,6 +319,7 @@ __device__ __noinline__ void list_slice(SyncSmem& sm, const SyncSearch& S, const
         if (T.rank == 0) sm.base = atomicExch(&S.bar->lcnt[p], 0u);
     }
     __syncthreads();
+    list_round(sm, S, q, p);
 }
 
 }  // namespace abfs

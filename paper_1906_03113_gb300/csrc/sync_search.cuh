@@ -126,6 +126,7 @@ __device__ __forceinline__ void sync_source(SyncSmem& sm, const SyncSearch& S, c
     }
     if (threadIdx.x == 0) {
         sm.step = sm.tick = 0;
+        sm.left = 0;
         sm.word[0] = sm.word[1] = sm.aux[0] = sm.aux[1] = 0;
         sm.app[0][0] = mine;
         sm.app[0][1] = ~0u;  // entries: not known
@@ -174,13 +175,26 @@ __device__ __forceinline__ uint32_t tot_ent(unsigned long long tot) {
 // entries, 150 us with its hub levels thin, 75 us wide.  Without hubs thin levels
 // stay ahead longer: ER of 150 000 vertices, degree 16, 82 us, 98 us with half
 // the line.
-constexpr uint32_t kWidePerCta = 10240, kHubPerCta = 1728;
+constexpr uint32_t kWidePerCta = 10240, kHubPerCta = 1728, kRoundsPart = 4;
 __device__ __forceinline__ uint32_t hub_line(const SyncSearch& S, const Team& T) {
     return kHubPerCta * T.size + S.n / 4;
 }
 __device__ __forceinline__ uint32_t wide_line(const SyncSearch& S, const Team& T, unsigned long long items,
                                               unsigned long long ent) {
     return ent >= S.hub_avg * items ? hub_line(S, T) : kWidePerCta * T.size + S.n;
+}
+
+// The line for a frontier whose items are counted exactly.  One that the lists do
+// not hold takes rounds, each with its own chain, and pays for the spilled items:
+// it stays thin only while its entries are few beside the vertices that a wide
+// level passes over.  (The levels of meshes stay under n / 9.  A batch of 128 ER
+// and R-MAT graphs on teams of a few CTAs, whose levels jump past the lists by a
+// factor of the degree: 688 us with wide_line alone, 583 with n / 4, 593 with
+// n / 8.)
+__device__ __forceinline__ uint32_t list_line(const SyncSearch& S, const Team& T, unsigned long long items,
+                                              unsigned long long ent) {
+    const uint32_t line = wide_line(S, T, items, ent);
+    return items > (unsigned long long)T.size * kThinCap ? min(line, S.n / kRoundsPart) : line;
 }
 
 // Thread 0 after the barrier that ended a thin level (tot: the barrier's
@@ -203,7 +217,7 @@ __device__ __forceinline__ uint32_t thin_next(SyncSmem& sm, const SyncSearch& S,
             if (sm.bu) return kActBottomUp;
         }
     }
-    if (ent >= wide_line(S, T, items, ent) || items > T.size * kThinCap) return kActWide;
+    if (ent >= wide_line(S, T, items, ent)) return kActWide;
     // a list is full, or a few CTAs hold much more than the others
     const uint32_t heavy = flags & 0xFFu;
     if ((flags >> 8) || (heavy && 2 * heavy <= T.size)) {
@@ -216,6 +230,14 @@ __device__ __forceinline__ uint32_t thin_next(SyncSmem& sm, const SyncSearch& S,
 // Runs thin levels from level k on until another kind of level follows
 // (sm.act); returns that level's number.  A function of its own, so that the
 // loop that long searches spend their time in has its own registers.
+//
+// The first level may take several rounds, where the lists do not hold it
+// (list_slice).  As a wide level it would cost, besides its entries, something
+// for every unvisited vertex, which a mesh of 10^8 vertices pays hundreds of
+// times and a small team on a small mesh all the same; in rounds the cost follows
+// the frontier (464^3: 98 -> 30 ms, on the unit scheduler 42; 152 searches of
+// 64^3 in a batch 13.9 -> 5.8 ms).  The test costs a thin level 2 %; rounds in a
+// function of their own cost the others their registers (R-MAT-20 182 -> 190 us).
 // Whole CTA.
 template <bool SIG>
 __device__ __noinline__ uint32_t thin_run(SyncSmem& sm, const SyncSearch& S, const Team& team, uint32_t k) {
@@ -226,14 +248,20 @@ __device__ __noinline__ uint32_t thin_run(SyncSmem& sm, const SyncSearch& S, con
     const bool want_aux = S.bu_alpha != 0 || S.trace != nullptr;
     SyncTally t;
     ThinStage st;
-    uint32_t act;
+    uint32_t act = kActThin;
     bool staged = false;
     __syncthreads();
     do {
         if (!staged) thin_stage(sm, S, k & 1, st);
         if (S.trace) sync_trace(S, T, kPhLevel, k, 4u, (uint32_t)sm.items, (uint32_t)sm.nf, (uint32_t)sm.entries);
         thin_claims<SIG>(sm, S, k, st, t);
+        const bool more = sm.left != 0;
         __syncthreads();
+        if (more) {
+            list_round(sm, S, k & 1, k & 1);
+            staged = false;
+            continue;
+        }
         const uint32_t cur = k & 1;
         unsigned long long add = 0, aux = 0;
         if (lead) {
@@ -286,9 +314,7 @@ __device__ __forceinline__ uint32_t wide_next(SyncSmem& sm, const SyncSearch& S,
         sm.bu = sm.bu ? sm.nf * S.bu_beta >= S.n : sm.entries * S.bu_alpha > mu;
         if (sm.bu) return kActBottomUp;
     }
-    if (bottom_up || tot > (unsigned long long)T.size * kThinCap ||
-        sm.entries >= wide_line(S, T, tot, sm.entries) / 2)
-        return kActWide;
+    if (bottom_up || sm.entries >= list_line(S, T, tot, sm.entries) / 2) return kActWide;
     heavy_limit(sm, T, (float)tot, (float)sm.entries);
     return kActSlice;
 }
@@ -313,9 +339,9 @@ __device__ __forceinline__ bool sync_leave(const SyncSearch& S, const Team& T) {
 // Runs one search on this team.  The outputs and the control block are written
 // when it returns (to be read after the kernel).
 //
-// Thin levels hold while the frontier fits the CTAs' lists and its entries
-// stay below wide_line; wide levels until it fits again with less than half
-// of that (each thin -> wide switch rebuilds the bitmap, 8 bytes per vertex).
+// Thin levels hold while the frontier's entries stay below wide_line; wide levels
+// until they are fewer than half of that (each thin -> wide switch rebuilds the
+// bitmap, 8 bytes per vertex).
 // After a barrier thread 0 alone decides what follows: the same decision made
 // by every thread took 1.3 us a level on 32 warps.
 // Returns, in thread 0, whether this CTA was the last to leave.
@@ -353,7 +379,7 @@ __device__ __forceinline__ bool sync_search(SyncSmem& sm, const SyncSearch& S, c
                 } else if (act == kActEven) {
                     // exact totals now: the thin level's were clamped per CTA
                     const unsigned long long all = sm.items, entries = sm.entries;
-                    if (all <= (unsigned long long)T.size * kThinCap && entries < wide_line(S, T, all, entries)) {
+                    if (entries < list_line(S, T, all, entries)) {
                         list_slice(sm, S, T, p, p, all);
                         // a failed append leaves the list incomplete
                         if (lead) sm.act = ld_relaxed(&S.bar->err) ? kActFailed : kActThin;
