@@ -78,10 +78,16 @@ typedef enum {
  * of the scheduling knobs (tile, unit_entries, narrow_*, ctas_per_sm,
  * claim_scan, cluster_*), submatrix searches without a physical shrink --
  * single ones, batches, and serving of graphs of up to 2^20 vertices and 2^25
- * entries -- run on the level-synchronous engine, where a team of CTAs runs one search at a time and none of those knobs
- * means anything.  A search that sets any of them, the comparator, shrinks and
- * abfs_run_static run on the unit scheduler, whose knobs they
- * are. */
+ * entries -- run on the level-synchronous engine, where a team of CTAs runs one
+ * search at a time and none of those knobs means anything.  A search that sets
+ * any of them, the comparator, shrinks and abfs_run_static run on the unit
+ * scheduler, whose knobs they are.  So do searches on graphs of over 2^25
+ * vertices and fewer than n / 128 entries, and single searches and batches while
+ * teams cannot run: where the device does not take a launch of CTAs that start
+ * together, and beside a server with ctas_per_sm 1, which leaves every SM half
+ * free.  A team's CTAs take whole SMs: beside a kernel of the caller's own that
+ * holds a part of the GPU for long, a search that is not to wait for its end
+ * sets a knob (ctas_per_sm = 1, for instance). */
 typedef struct {
     uint32_t mode;            /* ABFS_MODE_SUBMATRIX or ABFS_MODE_PLAIN */
     uint32_t tile;            /* frontier vertices staged per step, 32..1024, multiple of 32 */
@@ -502,6 +508,13 @@ int abfs_test_hold_first_phase(uint32_t extra_units);
  * nothing.  abfs_test_hold_first_phase(x) is abfs_test_hold_barrier(x, 0).
  */
 int abfs_test_hold_barrier(uint32_t extra_arrivals, uint32_t barriers);
+
+/*
+ * Test control: while `on` is non-zero, launches of teams (single searches and
+ * batches) fail on the host as if the device could not hold their CTAs at once,
+ * and the searches run on the unit scheduler.  Process-wide; needs no device.
+ */
+int abfs_test_refuse_teams(int on);
 
 /* On-chip ceilings of the expand step, measured on the current device. */
 typedef struct {

@@ -224,6 +224,24 @@ bool sync_applies(uint64_t n, uint64_t nnz, const abfs_params& p) {
            p.cluster_max == d.cluster_max && p.cluster_edges == d.cluster_edges;
 }
 
+namespace {
+constexpr int kMaxDevices = 64;
+std::atomic<int> g_room_servers[kMaxDevices];
+}  // namespace
+
+int room_servers(int device) {
+    return device >= 0 && device < kMaxDevices ? g_room_servers[device].load(std::memory_order_relaxed) : 0;
+}
+void room_servers_add(int device, int change) {
+    if (device >= 0 && device < kMaxDevices) g_room_servers[device].fetch_add(change, std::memory_order_relaxed);
+}
+
+bool teams_refused(cudaError_t e) {
+    if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorLaunchOutOfResources) return false;
+    cudaGetLastError();
+    return true;
+}
+
 // Whether one CTA can hold a search whole (sync_local.cuh): its keys in shared
 // memory, its graph in the L1.
 bool sync_local(uint32_t n, uint64_t nnz) { return n <= kLocalN && nnz <= kLocalNnz; }
@@ -614,14 +632,15 @@ int enqueue_single(abfs_graph_s* g, uint32_t source, int32_t* level, int32_t* pa
     // those that may take bottom-up levels: their scans need each column in
     // ascending input-label order, which only the input numbering has
     const bool bu_wanted = p.bottom_up_alpha && !g->directed && g->sorted;
-    const int most = sync_applies(g->n, g->nnz, p) ? sync_max_ctas(g->device, g->sms) : 0;
-    // (a graph that fits one CTA gains nothing from its relabelled copy)
-    const bool rel = w.relabel && p.mode == ABFS_MODE_SUBMATRIX && !sigma && !bu_wanted &&
-                     !(most > 0 && sync_local(g->n, g->nnz));
+    const int most =
+        sync_applies(g->n, g->nnz, p) && !room_servers(g->device) ? sync_max_ctas(g->device, g->sms) : 0;
+    const bool rel = w.relabel && p.mode == ABFS_MODE_SUBMATRIX && !sigma && !bu_wanted;
     const uint32_t bu_ok = (!rel && !g->directed && g->sorted && !sigma) ? 1u : 0u;
     if (most > 0) {
         SyncBar* bar = reinterpret_cast<SyncBar*>(reinterpret_cast<char*>(w.d_done) + kBarAt);
-        SyncSearch S = make_sync(g, w.base, w.L, bar, source, rel, p);
+        // (a graph that fits one CTA gains nothing from its relabelled copy)
+        const bool fits = sync_local(g->n, g->nnz), copy = rel && !fits;
+        SyncSearch S = make_sync(g, w.base, w.L, bar, source, copy, p);
         S.sigma = reinterpret_cast<unsigned long long*>(sigma);
         S.level = level;
         S.parent = reinterpret_cast<uint32_t*>(parent);
@@ -629,11 +648,14 @@ int enqueue_single(abfs_graph_s* g, uint32_t source, int32_t* level, int32_t* pa
         S.trace_cap = trace_cap;
         S.bu_alpha = bu_ok ? p.bottom_up_alpha : 0u;
         S.bu_beta = p.bottom_up_beta;
-        S.local = !rel && !sigma && !trace && !S.bu_alpha && sync_local(g->n, g->nnz);
-        CK(launch_sync(S, sync_team_cap(S, most), s));
-        CK(cudaEventRecord(g->last_use, s));
-        g->used = true;
-        return ABFS_OK;
+        S.local = fits && !sigma && !trace && !S.bu_alpha;
+        const cudaError_t e = launch_sync(S, sync_team_cap(S, most), s);
+        if (!teams_refused(e)) {
+            CK(e);
+            CK(cudaEventRecord(g->last_use, s));
+            g->used = true;
+            return ABFS_OK;
+        }
     }
     EngineArgs a;
     a.insts = rel ? w.d_inst_r : w.d_inst;
@@ -1153,6 +1175,11 @@ struct abfs_batch_s {
     uint32_t ninst = 0;          // search instances (a multi-source search answers several queries)
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
+    // the same searches on the unit scheduler, launched in place of the graph where
+    // teams cannot run
+    bool teams = false;          // what the graph holds
+    EngineArgs unit;
+    uint32_t max_n = 0;
     InstCtl* h_ctl = nullptr;    // pinned, ninst entries
 };
 
@@ -1233,6 +1260,12 @@ TeamPlan plan_teams(const std::vector<double>& work, const std::vector<uint32_t>
         best = std::move(t);
     }
     return best;
+}
+
+cudaError_t launch_unit_batch(const abfs_batch_s* b, cudaStream_t s) {
+    const cudaError_t e1 = launch_init(b->unit, b->max_n, s);
+    const cudaError_t e2 = launch_engine(b->unit, grid_size(b->graphs[0], b->p, 0), s);
+    return e1 != cudaSuccess ? e1 : e2;
 }
 
 // Shared by abfs_batch_create and abfs_batch_create_counts (sigma == NULL: no counts).
@@ -1451,14 +1484,7 @@ int batch_create(const abfs_graph_t* g, const uint32_t* sources, uint32_t count,
         sb.hold_units = test_hold_units();
         sb.next = reinterpret_cast<uint32_t*>(b->d_sync + at_next);
     }
-    // capture initialisation + the persistent launch in a CUDA graph
-    cudaStream_t cap;
-    e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
-    if (e != cudaSuccess) {
-        abfs_batch_destroy(b);
-        return cuda_fail(e);
-    }
-    EngineArgs a;
+    EngineArgs& a = b->unit;
     a.insts = b->d_insts;
     a.ninst = ninst;
     a.done_count = b->d_done;
@@ -1470,19 +1496,30 @@ int batch_create(const abfs_graph_t* g, const uint32_t* sources, uint32_t count,
     a.idle_exit_ns = 0;
     a.p = engine_params(p);
     a.hold_units = test_hold_units();
-    e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
-    if (e == cudaSuccess) {
-        cudaError_t e1 = cudaSuccess, e2;
-        if (sync) {
-            e2 = launch_sync_batch(sb, sigma != nullptr, sync_grid, cap);
-        } else {
-            e1 = launch_init(a, max_n, cap);
-            e2 = launch_engine(a, grid_size(g[0], p, 0), cap);
-        }
-        e = cudaStreamEndCapture(cap, &b->graph);
-        if (e == cudaSuccess) e = (e1 != cudaSuccess) ? e1 : e2;
+    b->max_n = max_n;
+    // capture the launch -- of teams, or initialisation and the scheduler's
+    // persistent launch -- in a CUDA graph
+    cudaStream_t cap;
+    e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
+    if (e != cudaSuccess) {
+        abfs_batch_destroy(b);
+        return cuda_fail(e);
     }
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec, b->graph, 0);
+    b->teams = sync;
+    for (;;) {
+        e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
+        if (e == cudaSuccess) {
+            const cudaError_t e1 = b->teams ? launch_sync_batch(sb, sigma != nullptr, sync_grid, cap)
+                                            : launch_unit_batch(b, cap);
+            e = cudaStreamEndCapture(cap, &b->graph);
+            if (e1 != cudaSuccess) e = e1;
+        }
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec, b->graph, 0);
+        if (!b->teams || !teams_refused(e)) break;
+        if (b->graph) cudaGraphDestroy(b->graph);
+        b->graph = nullptr;
+        b->teams = false;
+    }
     cudaStreamDestroy(cap);
     if (e != cudaSuccess) {
         abfs_batch_destroy(b);
@@ -1513,8 +1550,12 @@ extern "C" int abfs_batch_create_counts(const abfs_graph_t* g, const uint32_t* s
 
 extern "C" int abfs_batch_launch(abfs_batch_t b, abfs_stream_t stream) {
     if (!b) return ABFS_ERR_INVALID_ARG;
-    CK(cudaGraphLaunch(b->exec, (cudaStream_t)stream));
-    return ABFS_OK;
+    cudaStream_t s = (cudaStream_t)stream;
+    if (!b->teams || !room_servers(b->graphs[0]->device)) {
+        const cudaError_t e = cudaGraphLaunch(b->exec, s);
+        if (!b->teams || !teams_refused(e)) return cuda_fail(e);
+    }
+    return cuda_fail(launch_unit_batch(b, s));
 }
 
 extern "C" int abfs_batch_status(abfs_batch_t b, abfs_stream_t stream, int32_t* status) {
@@ -1764,7 +1805,8 @@ extern "C" int abfs_set_allocator(void* (*alloc)(size_t, void*), void (*free_fn)
 extern "C" const char* abfs_last_cuda_error(void) { return g_last_cuda_error.c_str(); }
 
 // ---------------------------------------------------------------------------
-// test controls: a first phase, or a barrier, that never completes
+// test controls: a first phase, or a barrier, that never completes; teams that
+// the device does not take
 // ---------------------------------------------------------------------------
 
 namespace {
@@ -1778,6 +1820,19 @@ uint32_t test_hold_from() { return g_hold_from.load(std::memory_order_relaxed); 
 
 extern "C" int abfs_test_hold_first_phase(uint32_t extra_units) {
     return abfs_test_hold_barrier(extra_units, 0);
+}
+
+namespace {
+std::atomic<bool> g_refuse_teams{false};
+}  // namespace
+
+namespace abfs {
+bool test_refuse_teams() { return g_refuse_teams.load(std::memory_order_relaxed); }
+}  // namespace abfs
+
+extern "C" int abfs_test_refuse_teams(int on) {
+    g_refuse_teams.store(on != 0, std::memory_order_relaxed);
+    return ABFS_OK;
 }
 
 extern "C" int abfs_test_hold_barrier(uint32_t extra_arrivals, uint32_t barriers) {

@@ -391,6 +391,15 @@ Layout layout_for(uint32_t n, uint64_t nnz, const abfs_params& p, uint32_t ms = 
 // Whether searches of n vertices and nnz entries in all with these parameters
 // run on the level-synchronous engine.
 bool sync_applies(uint64_t n, uint64_t nnz, const abfs_params& p);
+// Servers running on the unit scheduler whose CTAs leave room on every SM beside
+// them.  A search on the scheduler runs in that room; a team, whose CTAs take
+// whole SMs and start together, would wait until the server idles out.
+int room_servers(int device);
+void room_servers_add(int device, int change);
+// Whether a launch of teams failed because its CTAs cannot all be resident (fewer
+// SMs usable than the device reports, as under an MPS share): the scheduler runs
+// with any number of CTAs.  Clears the error.
+bool teams_refused(cudaError_t e);
 Inst make_inst_raw(const uint32_t* colptr, const uint32_t* rowidx, uint32_t n, char* base,
                    const Layout& L, uint32_t src, int32_t* level, int32_t* parent);
 int grid_for(int sms, const abfs_params& p);
@@ -409,6 +418,8 @@ uint32_t test_hold_units();
 // Barriers a held search of the level-synchronous engine passes first
 // (abfs_test_hold_barrier).
 uint32_t test_hold_from();
+// Test control set by abfs_test_refuse_teams.
+bool test_refuse_teams();
 
 // Launch helpers implemented in engine.cu.
 cudaError_t launch_put_inst(const Inst& inst, Inst* dst, cudaStream_t s);

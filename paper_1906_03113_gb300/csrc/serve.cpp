@@ -99,6 +99,7 @@ struct abfs_server_s {
     // queries on the level-synchronous engine (cfg.params permitting): their
     // slots, barriers (kBarStride bytes each) and teams being formed
     int ctas = 0;                 // CTAs of its launch, 0: the unit scheduler serves
+    bool leaves_room = false;     // ... with fewer CTAs per SM than fit (room_servers)
     SyncSlot* d_sync = nullptr;
     char* d_bars = nullptr;
     unsigned long long* d_join = nullptr;
@@ -150,6 +151,7 @@ void release_server(abfs_server_s* S) {
     if (S->h_notify) cudaFreeHost(S->h_notify);
     if (S->h_stage) cudaFreeHost(S->h_stage);
     if (S->h_words) cudaFreeHost(S->h_words);
+    if (S->leaves_room) room_servers_add(S->device, -1);
     delete S;
 }
 
@@ -414,6 +416,11 @@ extern "C" int abfs_serve_start(const abfs_graph_t* g, uint32_t ngraphs, const a
         cudaGetLastError();
         release_server(S);
         return e == cudaErrorMemoryAllocation ? ABFS_ERR_OOM : ABFS_ERR_CUDA;
+    }
+    int per_sm = 0;
+    if (!S->ctas && engine_occupancy(c.params.mode, &per_sm) == cudaSuccess && (int)c.params.ctas_per_sm < per_sm) {
+        S->leaves_room = true;
+        room_servers_add(S->device, 1);
     }
     S->slots.resize(ns);
     S->arena.init(c.memory_budget);

@@ -326,6 +326,7 @@ static cudaLaunchConfig_t sync_config(int ctas, cudaStream_t s, cudaLaunchAttrib
 }
 
 cudaError_t launch_sync(const SyncSearch& S, int ctas, cudaStream_t s) {
+    if (test_refuse_teams()) return cudaErrorCooperativeLaunchTooLarge;
     cudaLaunchAttribute at[1];
     const cudaLaunchConfig_t cfg = sync_config(ctas, s, at);
     cudaError_t e = S.sigma ? cudaLaunchKernelEx(&cfg, sync_kernel<true>, S)
@@ -339,6 +340,7 @@ cudaError_t launch_sync_serve(const SyncServe& A, int ctas, cudaStream_t s) {
 }
 
 cudaError_t launch_sync_batch(const SyncBatch& B, bool sigma, int ctas, cudaStream_t s) {
+    if (test_refuse_teams()) return cudaErrorCooperativeLaunchTooLarge;
     cudaLaunchAttribute at[1];
     const cudaLaunchConfig_t cfg = sync_config(ctas, s, at);
     cudaError_t e = sigma ? cudaLaunchKernelEx(&cfg, sync_batch_kernel<true>, B)
