@@ -517,6 +517,15 @@ int ensure_workspace(abfs_graph_s* g, const abfs_params& p) {
     }
     Layout L = layout_for(g->n, g->nnz, p, 0, g->relabeled, sync_layout(p));
     int rc = dev_alloc((void**)&w.base, L.total);
+    if (rc == ABFS_ERR_OOM && L.icap) {
+        // on graphs of hundreds of entries per vertex the teams' lists take more
+        // than the scheduler's arrays they are laid over
+        const Layout unit = layout_for(g->n, g->nnz, p, 0, g->relabeled, false);
+        if (unit.total < L.total) {
+            L = unit;
+            rc = dev_alloc((void**)&w.base, L.total);
+        }
+    }
     if (rc) return rc;
     rc = dev_alloc((void**)&w.d_done, kBarAt + sizeof(SyncBar));
     if (!rc) rc = dev_alloc((void**)&w.d_beat, 64);
@@ -632,8 +641,9 @@ int enqueue_single(abfs_graph_s* g, uint32_t source, int32_t* level, int32_t* pa
     // those that may take bottom-up levels: their scans need each column in
     // ascending input-label order, which only the input numbering has
     const bool bu_wanted = p.bottom_up_alpha && !g->directed && g->sorted;
-    const int most =
-        sync_applies(g->n, g->nnz, p) && !room_servers(g->device) ? sync_max_ctas(g->device, g->sms) : 0;
+    const int most = w.L.icap && sync_applies(g->n, g->nnz, p) && !room_servers(g->device)
+                         ? sync_max_ctas(g->device, g->sms)
+                         : 0;
     const bool rel = w.relabel && p.mode == ABFS_MODE_SUBMATRIX && !sigma && !bu_wanted;
     const uint32_t bu_ok = (!rel && !g->directed && g->sorted && !sigma) ? 1u : 0u;
     if (most > 0) {
@@ -1336,20 +1346,30 @@ int batch_create(const abfs_graph_t* g, const uint32_t* sources, uint32_t count,
         all_nnz += g[m.gi]->nnz;
     }
     const int most = sync_applies(all_n, all_nnz, p) ? sync_max_ctas(g[0]->device, g[0]->sms) : 0;
-    const bool sync = most > 0;
+    bool sync = most > 0;
     std::vector<Layout> L(ninst);
     std::vector<size_t> base(ninst);
-    size_t total = 0;
     uint32_t max_n = 0;
-    for (uint32_t t = 0; t < ninst; ++t) {
-        const abfs_graph_s* gt = g[inst[t].gi];
-        const uint32_t ms = inst[t].q.size() > 1 ? (uint32_t)inst[t].q.size() : 0u;
-        L[t] = layout_for(gt->n, gt->nnz, p, ms, false, sync);
-        base[t] = total;
-        total = align_up(total + L[t].total, 256);
-        max_n = std::max(max_n, gt->n);
-    }
+    auto lay_out = [&](bool teams) {
+        size_t total = 0;
+        for (uint32_t t = 0; t < ninst; ++t) {
+            const abfs_graph_s* gt = g[inst[t].gi];
+            const uint32_t ms = inst[t].q.size() > 1 ? (uint32_t)inst[t].q.size() : 0u;
+            L[t] = layout_for(gt->n, gt->nnz, p, ms, false, teams);
+            base[t] = total;
+            total = align_up(total + L[t].total, 256);
+            max_n = std::max(max_n, gt->n);
+        }
+        return total;
+    };
+    const size_t total = lay_out(sync);
     rc = dev_alloc((void**)&b->ws, total);
+    if (rc == ABFS_ERR_OOM && sync) {
+        // (as in ensure_workspace)
+        const size_t unit = lay_out(false);
+        if (unit < total) rc = dev_alloc((void**)&b->ws, unit);
+        sync = false;
+    }
     if (!rc) rc = dev_alloc((void**)&b->d_insts, sizeof(Inst) * ninst);
     if (!rc) rc = dev_alloc((void**)&b->d_done, 64);
     if (!rc) rc = dev_alloc((void**)&b->d_beat, 64);

@@ -339,7 +339,7 @@ extern "C" int abfs_serve_start(const abfs_graph_t* g, uint32_t ngraphs, const a
     if (!S) return ABFS_ERR_OOM;
     S->cfg = c;
     S->graphs.assign(g, g + ngraphs);
-    size_t largest = 0;
+    size_t largest;
     for (uint32_t i = 0; i < ngraphs; ++i) {
         const uint32_t* cp;
         const uint32_t* ri;
@@ -360,16 +360,24 @@ extern "C" int abfs_serve_start(const abfs_graph_t* g, uint32_t ngraphs, const a
         if (i == 0 && sync_applies(n, nnz, c.params)) S->ctas = sync_max_ctas(dev, sms);
         if (n > kTeamServeN || nnz > kTeamServeNnz) S->ctas = 0;
     }
-    for (uint32_t i = 0; i < ngraphs; ++i) {
-        const uint32_t* cp;
-        const uint32_t* ri;
-        uint32_t n;
-        uint64_t nnz;
-        int dev, sms;
-        graph_arrays(g[i], &cp, &ri, &n, &nnz, &dev, &sms);
-        S->layouts.push_back(layout_for(n, nnz, c.params, 0, false, S->ctas > 0));
-        S->work.push_back((uint32_t)std::min(8.0 * sync_work_us(n, nnz, 0) + 1.0, 16777215.0));
-        largest = std::max(largest, S->layouts.back().total);
+    for (;;) {
+        largest = 0;
+        S->layouts.clear();
+        S->work.clear();
+        for (uint32_t i = 0; i < ngraphs; ++i) {
+            const uint32_t* cp;
+            const uint32_t* ri;
+            uint32_t n;
+            uint64_t nnz;
+            int dev, sms;
+            graph_arrays(g[i], &cp, &ri, &n, &nnz, &dev, &sms);
+            S->layouts.push_back(layout_for(n, nnz, c.params, 0, false, S->ctas > 0));
+            S->work.push_back((uint32_t)std::min(8.0 * sync_work_us(n, nnz, 0) + 1.0, 16777215.0));
+            largest = std::max(largest, S->layouts.back().total);
+        }
+        // (teams' lists may take more than the scheduler's arrays)
+        if (largest + 256 <= c.memory_budget || !S->ctas) break;
+        S->ctas = 0;
     }
     if (largest + 256 > c.memory_budget) {
         delete S;

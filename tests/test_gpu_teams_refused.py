@@ -102,3 +102,66 @@ def test_searches_beside_a_server_that_leaves_room(lib):
     assert _same(abfs.run(G, srcs[2]), want[2])
     before.destroy()
     G.destroy()
+
+
+class _Limit:
+    """An allocator hook over torch that refuses blocks of more than `low` and at
+    most `high` bytes."""
+
+    def __init__(self, low, high):
+        import ctypes
+        self.live, self.refused = {}, 0
+
+        def alloc(nbytes, ctx):
+            if low < nbytes <= high:
+                self.refused += 1
+                return None
+            t = torch.empty(int(nbytes), dtype=torch.uint8, device="cuda")
+            self.live[t.data_ptr()] = t
+            return t.data_ptr()
+
+        self.a = ctypes.CFUNCTYPE(ctypes.c_void_p, ctypes.c_size_t, ctypes.c_void_p)(alloc)
+        self.f = ctypes.CFUNCTYPE(None, ctypes.c_void_p, ctypes.c_void_p)(lambda p, ctx: self.live.__delitem__(p))
+        self.ptr = [ctypes.cast(x, ctypes.c_void_p) for x in (self.a, self.f)]
+
+
+@pytest.mark.gpu
+def test_memory_that_holds_a_search_of_the_scheduler_only(lib):
+    """On a dense graph a team's lists take more than the scheduler's arrays.
+    Servers, searches and batches that fit with the scheduler's run there."""
+    n = 1200
+    a, b = np.nonzero(np.random.default_rng(4).random((n, n)) < 0.4)
+    g = synth.from_arcs(n, a.tolist(), b.tolist(), directed=False)
+    G = abfs.graph_create(g.colptr, g.rowidx, directed=False)
+    need = G.footprint()
+    # (smaller granules: a little more than the scheduler's own layout)
+    unit = G.footprint(abfs.default_params(unit_entries=512))
+    assert unit + 256 < need
+    want = [oracle.bfs(g, s) for s in range(3)]
+    srv = abfs.Server([G], abfs.serve_default_cfg(max_slots=4, memory_budget=unit + 256, idle_exit_ms=1))
+    outs = [[torch.empty(n, dtype=torch.int32, device="cuda") for _ in range(2)] for _ in want]
+    torch.cuda.synchronize()
+    tickets = [srv.submit(0, s, *outs[s]) for s in range(3)]
+    assert [srv.wait(t) for t in tickets] == [0] * 3
+    assert srv.stop()["failed"] == 0
+    assert all(_same(outs[s], want[s]) for s in range(3))
+    with pytest.raises(abfs.AbfsError) as ei:
+        abfs.Server([G], abfs.serve_default_cfg(memory_budget=unit // 2))
+    assert ei.value.status == abfs.binding.ERR_OOM
+    G.destroy()
+    hook = _Limit(unit, need + 256)
+    assert lib.abfs_set_allocator(*hook.ptr, None) == 0
+    try:
+        G = abfs.graph_create(g.colptr, g.rowidx, directed=False)
+        assert hook.refused == 0
+        assert _same(abfs.run(G, 0), want[0]) and hook.refused == 1
+        assert _same(abfs.run(G, 1), want[1]) and hook.refused == 1
+        plan = abfs.BatchPlan([G], [2])
+        plan.launch()
+        assert plan.status() == [0] and _same((plan.levels[0], plan.parents[0]), want[2])
+        assert hook.refused == 2
+        plan.destroy()
+        G.destroy()
+    finally:
+        assert lib.abfs_set_allocator(None, None, None) == 0
+    assert not hook.live
