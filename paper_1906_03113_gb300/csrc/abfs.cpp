@@ -1632,9 +1632,14 @@ std::string gpu_name(int dev) {
     return s;
 }
 
+// Number of the engines that a tuning cache's line was measured with.  Submatrix
+// lines without it are from before the level-synchronous engine: their choice is
+// among the scheduler's parameters only, so they are measured again.
+constexpr int kTuneEngines = 2;
+
 std::string params_json(const abfs_params& p) {
     std::ostringstream o;
-    o << "\"mode\":" << p.mode << ",\"tile\":" << p.tile << ",\"unit_entries\":" << p.unit_entries
+    o << "\"engines\":" << kTuneEngines << ",\"mode\":" << p.mode << ",\"tile\":" << p.tile << ",\"unit_entries\":" << p.unit_entries
       << ",\"narrow_max\":" << p.narrow_max
       << ",\"narrow_edges\":" << p.narrow_edges
       << ",\"ctas_per_sm\":" << p.ctas_per_sm << ",\"shrink_theta\":" << p.shrink_theta
@@ -1649,6 +1654,11 @@ bool json_num(const std::string& line, const std::string& key, double* v) {
     if (at == std::string::npos) return false;
     *v = std::strtod(line.c_str() + at + k.size(), nullptr);
     return true;
+}
+
+bool tuned_with_these(const std::string& line, uint32_t mode) {
+    double v = 1;
+    return mode != ABFS_MODE_SUBMATRIX || (json_num(line, "engines", &v) && (int)v == kTuneEngines);
 }
 
 bool json_str(const std::string& line, const std::string& key, std::string* v) {
@@ -1672,7 +1682,7 @@ extern "C" int abfs_tune(abfs_graph_t g, const uint32_t* sources, uint32_t count
     cudaStream_t s = (cudaStream_t)stream;
     const std::string key_gpu = gpu_name(g->device);
     const std::string key_cls = size_class(g);
-    // cache lookup: JSON lines {"gpu":..,"sms":..,"mode":..,"class":..,<params>,"ms":..}
+    // cache lookup: JSON lines {"gpu":..,"sms":..,"class":..,"engines":..,"mode":..,<params>,"ms":..}
     if (cache_path) {
         std::ifstream in(cache_path);
         std::string line, found;
@@ -1681,7 +1691,7 @@ extern "C" int abfs_tune(abfs_graph_t g, const uint32_t* sources, uint32_t count
             double sms = 0, md = -1;
             if (json_str(line, "gpu", &gpu) && json_str(line, "class", &cls) &&
                 json_num(line, "sms", &sms) && json_num(line, "mode", &md) && gpu == key_gpu &&
-                cls == key_cls && (int)sms == g->sms && (uint32_t)md == mode)
+                cls == key_cls && (int)sms == g->sms && (uint32_t)md == mode && tuned_with_these(line, mode))
                 found = line;
         }
         if (!found.empty()) {
@@ -1898,7 +1908,8 @@ extern "C" int abfs_batch_tune(const abfs_graph_t* g, const uint32_t* sources, u
             double sms = 0, md = -1;
             if (json_str(line, "gpu", &gpu) && json_str(line, "class", &cls) &&
                 json_num(line, "sms", &sms) && json_num(line, "mode", &md) && gpu == key_gpu &&
-                cls == key_cls && (int)sms == g[0]->sms && (uint32_t)md == mode)
+                cls == key_cls && (int)sms == g[0]->sms && (uint32_t)md == mode &&
+                tuned_with_these(line, mode))
                 found = line;
         }
         if (!found.empty()) {
