@@ -300,13 +300,15 @@ int abfs_run_host_many(abfs_graph_t g, const uint32_t* sources, uint32_t count,
  *   7 frontier bitmap of a bottom-up level, 8 bottom-up level,
  *   0xFE start, 0xFF end), [3] 0 if the phase was published to the whole
  *   grid, 1 if it ran on one CTA (or started a cluster run), 2 if it is a
- *   further level of a resident narrow run, 4 if it is a thin level of the
- *   level-synchronous engine ([5] then counts list items), 3 if it is a further
- *   level of a cluster run ([4] then holds the run's CTAs), [4] units or touched rows of
- *   the phase, [5] frontier
- *   vertices, [6] entry slots of that frontier (column entries plus up to 6
- *   per vertex, low 32 bits), [7] 0.  For a level, [4] is its number of work
- *   units (comparator mask: touched rows).
+ *   further level of a resident narrow run, 3 if it is a further level of a
+ *   cluster run ([4] then holds the run's CTAs), 4 if it is a thin level of the
+ *   level-synchronous engine ([5] then counts list items), [4] units or touched
+ *   rows of the phase, [5] frontier vertices, [6] entry slots of that frontier
+ *   (column entries plus up to 6 per vertex, low 32 bits), [7] 0.  For a level,
+ *   [4] is its number of work units (comparator mask: touched rows).
+ * A search on the unit scheduler is followed by six entries with the cycles its
+ * CTAs spent by activity: [2] of the first is 0xFD << 24, and from its [4] on they
+ * hold 19 64-bit totals (low word first).
  * *count receives the number written.  Synchronises `stream`.
  */
 int abfs_run_trace(abfs_graph_t g, uint32_t source, int32_t* level, int32_t* parent,

@@ -343,7 +343,9 @@ TRACE_KINDS = {0: "level", 1: "plain_mult", 2: "plain_mask", 3: "shrink", 4: "in
 
 
 def run_trace(g: Graph, source: int, params: Params | None = None, cap: int = 4096, stream=None):
-    """abfs_run_trace: (level, parent, list of per-phase dicts with t_us from start)."""
+    """abfs_run_trace: (level, parent, list of per-phase dicts with t_us from start,
+    after a search on the unit scheduler also one of kind "profile" with its CTAs'
+    cycles by activity)."""
     import torch
     level, parent = _outputs(g.n, None, None, torch.device("cuda", torch.cuda.current_device()))
     buf = np.zeros(cap * 8, dtype=np.uint32)

@@ -628,11 +628,13 @@ SyncSearch make_sync(const abfs_graph_s* g, char* base, const Layout& L, SyncBar
     return S;
 }
 
-// Enqueues one search into g's workspace; caller holds g->mu.
+// Enqueues one search into g's workspace; caller holds g->mu.  *teams tells
+// whether it runs on the level-synchronous engine, which fills no `prof`.
 int enqueue_single(abfs_graph_s* g, uint32_t source, int32_t* level, int32_t* parent,
                    cudaStream_t s, const abfs_params& p, uint4* trace = nullptr,
                    uint32_t trace_cap = 0, unsigned long long* prof = nullptr,
-                   uint64_t* sigma = nullptr) {
+                   uint64_t* sigma = nullptr, bool* teams = nullptr) {
+    if (teams) *teams = false;
     int rc = ensure_workspace(g, p);
     if (rc) return rc;
     Workspace& w = g->ws;
@@ -662,6 +664,7 @@ int enqueue_single(abfs_graph_s* g, uint32_t source, int32_t* level, int32_t* pa
         const cudaError_t e = launch_sync(S, sync_team_cap(S, most), s);
         if (!teams_refused(e)) {
             CK(e);
+            if (teams) *teams = true;
             CK(cudaEventRecord(g->last_use, s));
             g->used = true;
             return ABFS_OK;
@@ -1130,11 +1133,12 @@ extern "C" int abfs_run_trace(abfs_graph_t g, uint32_t source, int32_t* level, i
         dev_free(d_trace);
         return ABFS_ERR_CUDA;
     }
-    // the last kProfEntries entries carry the CTA cycle accounting (kind 0xFD):
-    // a header of 4 words, then kProfSlots 64-bit totals
+    // the last kProfEntries entries carry the scheduler's CTA cycle accounting
+    // (kind 0xFD): a header of 4 words, then kProfSlots 64-bit totals
     constexpr uint32_t kProfEntries = (4 + 2 * kProfSlots + 7) / 8;
     const uint32_t tcap = cap > kProfEntries ? cap - kProfEntries : 0;
-    rc = enqueue_single(g, source, level, parent, s, p, d_trace, tcap, d_prof);
+    bool teams = false;
+    rc = enqueue_single(g, source, level, parent, s, p, d_trace, tcap, d_prof, nullptr, &teams);
     if (!rc) {
         abfs_stats st;
         rc = finish_stats(g, s, &st);
@@ -1146,8 +1150,8 @@ extern "C" int abfs_run_trace(abfs_graph_t g, uint32_t source, int32_t* level, i
         if (cudaMemcpy(prof, d_prof, sizeof(prof), cudaMemcpyDeviceToHost) != cudaSuccess)
             rc = ABFS_ERR_CUDA;
         uint32_t* out = trace_host + (size_t)n * 8;
-        if (cap <= kProfEntries) out = nullptr;
-        if (out) {
+        const bool totals = cap > kProfEntries && !teams;
+        if (totals) {
         out[0] = 0;
         out[1] = 0;
         out[2] = 0xFDu << 24;
@@ -1158,7 +1162,7 @@ extern "C" int abfs_run_trace(abfs_graph_t g, uint32_t source, int32_t* level, i
         }
         for (uint32_t q = 4 + 2 * kProfSlots; q < 8 * kProfEntries; ++q) out[q] = 0;
         }
-        *count = (cap > kProfEntries) ? n + kProfEntries : n;
+        *count = totals ? n + kProfEntries : n;
         // the workspace descriptor keeps no pointer to the freed trace buffer
         launch_set_query(g->ws.d_inst, 0, nullptr, nullptr, nullptr, 0u, nullptr, 0, s);
         cudaStreamSynchronize(s);
