@@ -27,18 +27,22 @@ ABFS_TEAM_FN unsigned long long join_opened(unsigned long long before, uint32_t 
 
 // One thread of a CTA that has opened or joined a team: waits until the team is
 // closed and returns its size, the same in every CTA of the team.  The leader
-// closes it when it is full or after wait_ns.  A member whose own, much longer
+// closes it when it is full or after wait_ns, but while fewer than half of the
+// wanted CTAs have joined not before few_ns divided by their number.  A member whose own, much longer
 // wait runs out (the leader was not running meanwhile) closes it itself: the
 // size is the count in the word at the moment it was closed, whoever did that,
 // since nobody joins a closed team.  The word is not reused before this CTA
 // has left the search.
 template <class Io>
-ABFS_TEAM_FN uint32_t team_form(Io& io, bool leader, unsigned long long wait_ns) {
+ABFS_TEAM_FN uint32_t team_form(Io& io, bool leader, unsigned long long wait_ns, unsigned long long few_ns = 0) {
     const unsigned long long t0 = io.now();
     for (;;) {
         const unsigned long long w = io.load();
         if (!(w & kJoinOpen)) return join_count(w);
-        if ((leader && !join_room(w)) || io.now() - t0 > wait_ns) return join_count(io.close());
+        unsigned long long limit = wait_ns;
+        if (leader && 2 * join_count(w) < join_wanted(w) && few_ns / join_count(w) > limit)
+            limit = few_ns / join_count(w);
+        if ((leader && !join_room(w)) || io.now() - t0 > limit) return join_count(io.close());
     }
 }
 

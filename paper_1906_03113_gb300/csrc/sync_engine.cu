@@ -83,14 +83,18 @@ __global__ void __launch_bounds__(kSyncThreads, 1) sync_batch_kernel(const __gri
 // its part of the work at hand (all of them when it is alone): the claiming CTA
 // opens a team of that size, waits for others to come free, a quarter of the
 // time the query then takes and at most kJoinWaitNs, closes the team and runs
-// the query with whoever came.  Only CTAs that have joined are waited for
+// the query with whoever came.  While fewer than half have come it waits on, up
+// to half of what the query would take those few: the last CTA to come free, too
+// late for the other teams, took a query alone while they were about to finish
+// (16 queries on a 64^3 mesh 4.7 -> 1.1 ms, on 100^3 16.8 -> 3.9; the unit
+// scheduler 2.1 and 10.8).  Only CTAs that have joined are waited for
 // afterwards, so the launch needs no co-residency of all its CTAs, and a CTA
 // that idles out is never missed.  Claims are made one at a time, so that CTAs
 // that come free together do not each open a team that nobody is left to join.
 // (Counting on free CTAs alone left large queries on one CTA whenever the
 // launch was busy: 256 queries on 16 graphs 3.6 -> 6.7 ms.)
 constexpr unsigned long long kJoinWaitNs = 150000, kJoinWaitMinNs = 5000;
-constexpr unsigned long long kMemberWaitNs = 1000000000ull;
+constexpr unsigned long long kFewWaitNs = 100000000ull, kMemberWaitNs = 1000000000ull;
 
 struct ServeCmd {
     uint32_t what;  // 0: nothing to do, 1: run slot q, 2: leave
@@ -163,7 +167,7 @@ __device__ __forceinline__ ServeCmd serve_poll(const SyncServe& A, uint32_t curs
         if (atomicCAS(A.claim, 0u, 1u) == 0u) {
             const uint32_t st = ld_relaxed(A.state + q);
             const uint32_t run = (st & ~0xFFu) | kSlotRunning;
-            unsigned long long w = 0, wait = 0;
+            unsigned long long w = 0, wait = 0, few = 0;
             // (a launch that has been closed claims nothing more)
             if ((st & 0xFFu) == kSlotSubmitted && ld_relaxed(A.closed) != A.launch &&
                 atomicCAS(A.state + q, st, run) == st) {
@@ -174,6 +178,7 @@ __device__ __forceinline__ ServeCmd serve_poll(const SyncServe& A, uint32_t curs
                 if (size > 1) {
                     // (work is in eighths of a microsecond)
                     wait = min(kJoinWaitNs, max(kJoinWaitMinNs, 125ull * mine / (4 * size)));
+                    few = min(kFewWaitNs, 125ull * mine / 2);
                     w = join_opened(ld_relaxed64(A.join + q), size);
                     __threadfence();
                     st_relaxed64(A.join + q, w);
@@ -184,7 +189,7 @@ __device__ __forceinline__ ServeCmd serve_poll(const SyncServe& A, uint32_t curs
             st_relaxed(A.claim, 0u);
             if (w) {
                 JoinIo io{A.join + q};
-                size = team_form(io, true, wait);
+                size = team_form(io, true, wait, few);
             }
         }
     }

@@ -108,3 +108,41 @@ def test_servers_on_either_side_of_the_team_limit(n):
     assert srv.stop()["failed"] == 0
     for G in dev:
         G.destroy()
+
+
+def _burst_ms(dev, params, outs, src, reps=11):
+    """The median time of a burst of one query per output pair."""
+    cfg = abfs.serve_default_cfg(max_slots=32, memory_budget=1 << 30, idle_exit_ms=50)
+    cfg.params = params
+    srv = abfs.Server([dev], cfg)
+    times = []
+    for _ in range(reps):
+        t0 = time.perf_counter()
+        tickets = [srv.submit(0, src + q, *out) for q, out in enumerate(outs)]
+        assert [srv.wait(t) for t in tickets] == [0] * len(outs)
+        times.append((time.perf_counter() - t0) * 1e3)
+    assert srv.stop()["failed"] == 0
+    return sorted(times)[reps // 2]
+
+
+def test_no_query_of_a_burst_is_left_to_one_cta():
+    """Sixteen deep queries, more than the CTAs that come free at a time make up
+    teams for: the burst takes no longer than on the unit scheduler (it took
+    twice as long while a late CTA took the last query alone)."""
+    m = 64
+    v = np.arange(m ** 3)
+    x, y, z = v % m, (v // m) % m, v // (m * m)
+    a = np.concatenate([v[x < m - 1], v[y < m - 1], v[z < m - 1]])
+    b = np.concatenate([v[x < m - 1] + 1, v[y < m - 1] + m, v[z < m - 1] + m * m])
+    g = synth.from_arcs(m ** 3, a.tolist(), b.tolist(), directed=False)
+    G = abfs.graph_create(g.colptr, g.rowidx, directed=False)
+    src = int(g.n // 2 + m // 2)
+    outs = [_outputs(g.n) for _ in range(16)]
+    torch.cuda.synchronize()
+    scheduler = abfs.default_params(cluster_edges=abfs.default_params().cluster_edges - 1)
+    slow = _burst_ms(G, scheduler, outs, src)
+    fast = _burst_ms(G, abfs.default_params(), outs, src)
+    for q in (0, 15):
+        assert _exact(*outs[q], oracle.bfs(g, src + q))
+    assert fast < 1.3 * slow, (fast, slow)
+    G.destroy()

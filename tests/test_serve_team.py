@@ -52,7 +52,7 @@ int main() {
             if (round % 2) std::this_thread::sleep_for(std::chrono::microseconds(600));
             Io io{&word};
             rank[0] = 0;
-            size[0] = team_form(io, true, 100000);
+            size[0] = team_form(io, true, 100000, round % 3 ? 0 : 400000);
         });
         for (uint32_t c = 1; c <= ctas; ++c)
             th.emplace_back([&, c] {
