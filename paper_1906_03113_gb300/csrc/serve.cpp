@@ -170,11 +170,16 @@ EngineArgs serve_args(abfs_server_s* S) {
     return a;
 }
 
-// Servers with a graph above either size run on the unit scheduler: a team holds
-// its CTAs for a whole search, so a few large or long searches keep the others
-// waiting, where the scheduler's CTAs move from search to search (32 graphs of up
-// to 128 M entries: 394 queries/s on teams, 3264 on the scheduler; 256 queries on 16
-// graphs of up to 2^19 vertices: 4.8 ms on teams, 14.1).
+// Servers with a graph above either size run on the unit scheduler: a team's CTAs
+// wait for one another at the barriers of its wide levels, where the scheduler's
+// move on to another search, and large levels leave little to gain elsewhere.
+// 32 queries on one graph, teams and scheduler (ms): R-MAT of 31 M entries 6.5 and
+// 7.4, of 64 M 14.8 and 14.2, of 128 M 42 and 29, of 259 M 88 and 62; ER of degree
+// 16 and 2^20 vertices 5.0 and 7.4, 2^21 11.7 and 12.8, 2^22 26.8 and 24.7.  A line
+// drawn by sizes does not see depth (16 queries on a 2000^2 grid 13 and 28, on a
+// 200^3 mesh 33 and 90) nor how often the large graphs are asked for (32 graphs of
+// 2^16..2^22 vertices, one of 128 M entries among them: 6160 queries/s on teams,
+// 3250 on the scheduler).
 constexpr uint32_t kTeamServeN = 1u << 20;
 constexpr uint64_t kTeamServeNnz = 1ull << 25;
 

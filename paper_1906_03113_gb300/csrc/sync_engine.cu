@@ -1,12 +1,12 @@
 // Level-synchronous BFS engine for sm_103a: one search on a team of CTAs that
 // are resident together.
 //
-// The unit scheduler (engine.cu) lets any CTA take work of any search, which
-// batches and serving need, and pays for it with a hand-off of 10-20 us
-// between levels (publish, poll, take, block lists, unit starts, flush,
-// count down).  A single search needs none of that: its levels are separated
-// by one barrier whose word also carries the next level's size, so a level
-// costs its dependent chain -- row index, claim, barrier -- and nothing else.
+// The unit scheduler (engine.cu) lets any CTA take work of any search and pays
+// for it with a hand-off of 10-20 us between levels (publish, poll, take, block
+// lists, unit starts, flush, count down).  A search on a team of its own needs
+// none of that: its levels are separated by one barrier whose word also carries
+// the next level's size, so a level costs its dependent chain -- row index,
+// claim, barrier -- and nothing else.
 //
 // Three kinds of level, chosen from the totals the barrier delivers (see
 // sync_levels.cuh): thin (claims on the key words, private lists in shared
