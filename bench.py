@@ -49,22 +49,37 @@ def _peaks():
         return FALLBACK_HBM_GBS, "fallback"
 
 
-def _engine_sha256() -> str:
+# a search that sets one of these runs on the unit scheduler (abfs.h)
+SCHEDULER_KNOBS = ("tile", "unit_entries", "narrow_max", "narrow_edges", "ctas_per_sm", "narrow_resident",
+                   "claim_scan", "cluster_ctas", "cluster_min", "cluster_max", "cluster_edges")
+
+
+def on_teams(abfs, params) -> bool:
+    """Whether searches with these parameters run on the level-synchronous engine."""
+    d = abfs.default_params()
+    shrinks = 0.0 < params.shrink_theta < 1.0 and params.shrink_max > 0
+    return (params.mode == abfs.MODE_SUBMATRIX and not shrinks
+            and all(getattr(params, k) == getattr(d, k) for k in SCHEDULER_KNOBS))
+
+
+def _engine_sha256(prefix: str = "engine") -> str:
     import hashlib
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_1906_03113_gb300", "csrc")
-    names = sorted(f for f in os.listdir(csrc) if f.startswith("engine") and f.endswith((".cu", ".cuh")))
+    names = sorted(f for f in os.listdir(csrc) if f.startswith(prefix) and f.endswith((".cu", ".cuh")))
+    if prefix == "sync":
+        names.append("engine_common.cuh")
     for f in names + ["internal.h"]:
         with open(os.path.join(csrc, f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()
 
 
-def _profiled_traffic(workload: str):
+def _profiled_traffic(workload: str, prefix: str):
     """(DRAM bytes per engine launch, ncu duration of that launch in us) from
     the committed ncu summary of this workload, or (None, None) when the
     engine source changed since the capture."""
-    path = os.path.join(ROOT, "profiles", f"engine_kernel_{workload}.md")
+    path = os.path.join(ROOT, "profiles", f"{prefix}_kernel_{workload}.md")
     if not os.path.exists(path):
         return None, None
     fields = {}
@@ -74,7 +89,7 @@ def _profiled_traffic(workload: str):
             if len(m) == 2 and m[0] in ("traffic_bytes_per_launch", "engine_source_sha256",
                                         "ncu_duration_us"):
                 fields[m[0]] = m[1].strip()
-    if fields.get("engine_source_sha256") != _engine_sha256():
+    if fields.get("engine_source_sha256") != _engine_sha256(prefix):
         return None, None
     try:
         return int(fields["traffic_bytes_per_launch"]), float(fields.get("ncu_duration_us", "nan"))
@@ -346,7 +361,7 @@ def measure_batch(args, local, torch, abfs, big=None, G22=None, clocks=True):
             "single_query_ms": single_ms,
             "single_query_gteps": total_edges / (single_ms * 1e-3) / 1e9,
             "speedup_vs_single": single_ms / batch_ms, "parts": parts,
-            "tuned_params": tuned.as_dict(), "tuner_ms": tuned_ms,
+            "tuned_params": tuned.as_dict(), "tuner_ms": tuned_ms, "teams": on_teams(abfs, tuned),
             "launch": "one persistent launch (CUDA graph replay) of all 576 queries, parameters "
                       "from the batch autotuner",
             "graph": "512 ER/R-MAT graphs, n log-uniform in [2^10, 2^18], avg degree U[4,32] "
@@ -368,7 +383,7 @@ def bench_batch(args, ws, rank, local, torch, abfs, dist):
                                       "single_query_gteps", "speedup_vs_single", "parts",
                                       "tuned_params", "tuner_ms")},
         "hybrid": r["hybrid"],
-        "gpu_launches": 3 * r["steps"], "clocks": r["clocks"],
+        "gpu_launches": (1 if r["teams"] else 3) * r["steps"], "clocks": r["clocks"],
     }
     if rank == 0:
         print(json.dumps(line), flush=True)
@@ -684,7 +699,8 @@ def main():
     cal = abfs.calibrate(22)
     l2_bound_s = float(nnz_c.mean()) / (cal["load_gops"] * 1e9) + float(e_adj.mean()) / (
         cal["red_gops"] * 1e9)
-    traffic, ncu_us = _profiled_traffic(wname)
+    teams = on_teams(abfs, params)
+    traffic, ncu_us = _profiled_traffic(wname, "sync" if teams else "engine")
     dram_gbs = traffic / (ncu_us * 1e-6) / 1e9 if traffic and ncu_us and ncu_us == ncu_us else None
     line = {
         "metric": "GTEPS", "value": value, "unit": "GTEPS", "n_gpus": ws, "steps": args.steps,
@@ -709,7 +725,8 @@ def main():
                      "dram_frac": None if dram_gbs is None else dram_gbs / hbm,
                      "dram_from": "ncu dram__bytes of one engine launch / its ncu duration "
                                   "(profiles/), null if the engine changed since",
-                     "kernel": "engine_kernel<0> (one launch per BFS, after one initialisation "
+                     "kernel": "sync_kernel<0> (one launch per BFS)" if teams else
+                               "engine_kernel<0> (one launch per BFS, after one initialisation "
                                "kernel" + (", before one relabel_out_kernel)" if relabel else ")"),
                      "bytes_per_bfs": float(b_alg.mean()),
                      "bytes_formula": "4*E_adj + 24*n_c",
@@ -718,7 +735,7 @@ def main():
                             "formula": "nnz_c / load rate + E_adj / red rate",
                             "bound_ms_per_bfs": l2_bound_s * 1e3,
                             "frac": l2_bound_s / mean_t}},
-        "gpu_launches": (3 if relabel else 2) * nsrc * args.steps,
+        "gpu_launches": (1 if teams else 3 if relabel else 2) * nsrc * args.steps,
         "clocks": clk,
         "per_bfs_ms": float(per_bfs_ms.mean()),
         "reached_mean": float(n_c.mean()), "nnz_c_mean": float(nnz_c.mean()),
