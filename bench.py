@@ -693,9 +693,10 @@ def main():
     hbm, peak_kind = _peaks()
     mean_t = float(per_bfs_ms.mean()) * 1e-3
     achieved = float(b_alg.mean()) / mean_t / 1e9
-    # the on-chip ceiling: every stored entry of a reached column costs one
+    # the on-chip estimate: every stored entry of a reached column costs one
     # random visited-bitmap load, every entry that passes the mask one random
-    # reduction, both served by L2 (rates measured on this GPU, now)
+    # reduction, at the rates of the L2 (measured on this GPU, now); tests that
+    # hit the L1 can go below it
     cal = abfs.calibrate(22)
     l2_bound_s = float(nnz_c.mean()) / (cal["load_gops"] * 1e9) + float(e_adj.mean()) / (
         cal["red_gops"] * 1e9)
