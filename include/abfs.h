@@ -362,7 +362,8 @@ int abfs_batch_destroy(abfs_batch_t b);
  * submatrix method).  *best (may be NULL) receives the
  * choice and *best_ms its mean device time per search.  With `cache_path`
  * non-NULL the result is read from / appended to that JSON-lines file, keyed
- * by GPU name, SM count, mode and the graph's size class.  Synchronises.
+ * by GPU name, SM count, mode and the graph's size class; submatrix lines from
+ * before there were two engines do not count.  Synchronises.
  */
 int abfs_tune(abfs_graph_t g, const uint32_t* sources, uint32_t count, uint32_t mode,
               const char* cache_path, abfs_stream_t stream, abfs_params* best, float* best_ms);

@@ -76,8 +76,13 @@ def test_searches_beside_a_server_that_leaves_room(lib):
     # (kernels are loaded at their first use, which waits for the device)
     for t in before.levels + before.parents:
         t.fill_(9)
+    unit = abfs.default_params(ctas_per_sm=1)
     abfs.run(G, srcs[0])
-    abfs.run(G, srcs[0], params=abfs.default_params(ctas_per_sm=1))
+    abfs.run(G, srcs[0], params=unit)
+    plan = abfs.BatchPlan([G] * 3, srcs, params=unit)
+    plan.launch()
+    assert plan.status() == [0] * 3
+    plan.destroy()
     cfg = abfs.serve_default_cfg(max_slots=4, memory_budget=1 << 28, idle_exit_ms=3000)
     cfg.params = abfs.default_params(ctas_per_sm=1)
     srv = abfs.Server([G], cfg)
